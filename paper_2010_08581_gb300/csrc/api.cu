@@ -1632,11 +1632,18 @@ tr_status tr_rel_error(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, cons
   DeviceGuard g(ctx->device);
   int blocks;
   const bool xf64 = X_dtype == TR_F64;
-  const size_t bytes = fit_workspace(fa, xf64, &blocks);
-  TR_TRY(ensure_ws(ctx, bytes));
+  size_t tables;
+  const size_t bytes = fit_workspace(fa, xf64, &blocks, &tables);
+  // the slice tables only where the budget leaves room for them
+  if (ctx->budget && bytes + tables > ctx->arena_bytes &&
+      bytes + tables + ctx->host_stage_bytes > ctx->budget)
+    tables = 0;
+  TR_TRY(ensure_ws(ctx, bytes + tables));
   double* partial = reinterpret_cast<double*>(ctx->arena);
   cudaStream_t st = S(stream);
-  TR_LAUNCH("fit", launch_fit(fa, X, xf64, ctx->arena, blocks, ctx->d_err, st));
+  TR_LAUNCH("fit", launch_fit(fa, X, xf64, ctx->arena, blocks,
+                              tables ? reinterpret_cast<float*>(ctx->arena + bytes) : nullptr,
+                              ctx->d_err, st));
   std::vector<double> h(2 * static_cast<size_t>(blocks));
   TR_CUDA(cudaMemcpyAsync(h.data(), partial, h.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   TR_TRY(read_device_error(ctx, st));

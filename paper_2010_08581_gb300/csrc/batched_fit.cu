@@ -20,9 +20,9 @@ __device__ __forceinline__ bool fit_due(const BInst& d) {
 }
 
 // Partial sums of one slot's fit: one per CTA, at most kFitParts.
-__device__ __forceinline__ int fit_parts(const FitSplit& f, bool xf64) {
-  const int64_t nblk = fit_row_blocks(f, xf64);
-  return nblk < kFitParts ? static_cast<int>(nblk) : kFitParts;
+__device__ __forceinline__ int fit_parts(const FitArgs& fa, const FitSplit& f, bool xf64) {
+  const int64_t n = xf64 ? (fit_units(f) + 7) / 8 : fit_tc_parts(fit_tc_plan(fa, f));
+  return n < kFitParts ? static_cast<int>(n) : kFitParts;
 }
 
 __device__ __forceinline__ void fit_args(const BInst& d, FitArgs& fa) {
@@ -34,14 +34,35 @@ __device__ __forceinline__ void fit_args(const BInst& d, FitArgs& fa) {
   }
 }
 
-constexpr int kFitRightCtas = 64;   // CTAs per slot forming the right factors
+// The FP32 slice tables of the left and right groups (fit_tc.cuh) live in the slot's fibre
+// buffer, which no stage reads between the LS step and the next draws; they are skipped (null)
+// where they would not fit (J smaller than about twice the largest L).
+__device__ __forceinline__ float* fit_tables(const BInst& d, const FitArgs& fa, const FitSplit& f) {
+  int64_t Imax = 0;
+  for (int m = 0; m < fa.N; ++m) Imax = fa.dims[m] > Imax ? fa.dims[m] : Imax;
+  return fit_tc_tables_fit(fa, f) && fit_tc_tables_floats(fa, f) <= d.J * Imax
+             ? static_cast<float*>(d.Y) : nullptr;
+}
 
-// Right factors of the fit: e-major W^T for the SIMT contraction, or the swizzled hi/lo
-// tiles of the tensor-core contraction.
-template <typename T>
+constexpr int kFitRightCtas = 128;  // CTAs per slot forming the right factors
+
+__global__ void __launch_bounds__(256) kb_fit_tables(const BInst* __restrict__ tab) {
+  __shared__ FitArgs fa;
+  const BInst& d = tab[blockIdx.x];
+  if (!fit_due(d)) return;
+  if (threadIdx.x == 0) fit_args(d, fa);
+  __syncthreads();
+  const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
+  float* out = fit_tables(d, fa, f);
+  if (!out) return;
+  fit_tables_warps(fa, f, out, (static_cast<int64_t>(blockIdx.y) * blockDim.x + threadIdx.x) >> 5,
+                   static_cast<int64_t>(gridDim.y) * (blockDim.x >> 5));
+}
+
+// Right factors of the fit: e-major W^T for FP64 X ...
 __global__ void __launch_bounds__(FNT) kb_fit_right(const BInst* __restrict__ tab) {
-  __shared__ T chain[8][kMaxL];
-  __shared__ T slice[8][kMaxL];
+  __shared__ double chain[8][kMaxL];
+  __shared__ double slice[8][kMaxL];
   __shared__ FitArgs fa;
   const BInst& d = tab[blockIdx.x];
   if (!fit_due(d)) return;
@@ -50,28 +71,36 @@ __global__ void __launch_bounds__(FNT) kb_fit_right(const BInst* __restrict__ ta
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t step = static_cast<int64_t>(gridDim.y) * (FNT / 32);
-  const int64_t q0 = static_cast<int64_t>(blockIdx.y) * (FNT / 32) + warp;
-  if constexpr (sizeof(T) == 4) {
-    if (fit_use_tc(f, false)) {
-      unsigned char* WS = static_cast<unsigned char*>(d.fitw);
-      const int64_t ncol = (f.cols + FTN - 1) / FTN * FTN;
-      for (int64_t q = q0; q < ncol; q += step)
-        fit_right_tc_warp(fa, f, q, WS, chain[warp], slice[warp], lane);
-      return;
-    }
-  }
-  T* WT = static_cast<T*>(d.fitw);
-  for (int64_t q = q0; q < f.cols; q += step)
-    fit_right_warp<T>(fa, f, q, WT, chain[warp], slice[warp], lane);
+  double* WT = static_cast<double*>(d.fitw);
+  for (int64_t q = static_cast<int64_t>(blockIdx.y) * (FNT / 32) + warp; q < f.cols; q += step)
+    fit_right_warp(fa, f, q, WT, chain[warp], slice[warp], lane);
 }
 
-// Slots whose contraction length K lies in (k_lo, k_hi] (two launches with different
-// shared-memory sizes keep the common small-K case at several CTAs per SM).
-template <typename T>
-__global__ void __launch_bounds__(FNT) kb_fit(const BInst* __restrict__ tab, int k_lo, int k_hi) {
+// ... or the split operand tiles of the tensor-core contraction.
+__global__ void __launch_bounds__(FT_Q) kb_fit_right_tc(const BInst* __restrict__ tab) {
+  __shared__ __align__(16) float P[32 * 256];
+  __shared__ float G[4 * kMaxL];
+  __shared__ FitArgs fa;
+  const BInst& d = tab[blockIdx.x];
+  if (!fit_due(d)) return;
+  if (threadIdx.x == 0) fit_args(d, fa);
+  __syncthreads();
+  const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
+  const float* tables = fit_tables(d, fa, f);
+  if (tables) tables += fit_tc_table_floats(fa, f.s - 1);
+  const int nj = (f.K + 2 * FT_KS - 1) / (2 * FT_KS);      // jobs of two k-steps
+  const int64_t jobs = (f.cols + FT_Q - 1) / FT_Q * nj;
+  for (int64_t j = blockIdx.y; j < jobs; j += gridDim.y) {
+    const int ks = 2 * static_cast<int>(j % nj);
+    fit_right_tc_tile(fa, f, j / nj, ks, ks + 2, tables, static_cast<unsigned char*>(d.fitw), P, G);
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(FNT) kb_fit(const BInst* __restrict__ tab) {
   extern __shared__ __align__(16) unsigned char fit_dyn[];
-  __shared__ T chain[8][kMaxL];
-  __shared__ T slice[8][kMaxL];
+  __shared__ double chain[8][kMaxL];
+  __shared__ double slice[8][kMaxL];
   __shared__ double red[2 * (FNT / 32)];
   __shared__ FitArgs fa;
   const BInst& d = tab[blockIdx.x];
@@ -79,12 +108,13 @@ __global__ void __launch_bounds__(FNT) kb_fit(const BInst* __restrict__ tab, int
   if (threadIdx.x == 0) fit_args(d, fa);
   __syncthreads();
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
-  if (fit_use_tc(f, sizeof(T) == 8) || f.K <= k_lo || f.K > k_hi) return;
-  const int parts = fit_parts(f, sizeof(T) == 8);
+  const int parts = fit_parts(fa, f, true);
   if (static_cast<int>(blockIdx.y) >= parts) return;
+  const int64_t units = fit_units(f);
   double se = 0.0, sx = 0.0;
-  fit_blocks<T>(fa, f, static_cast<const T*>(d.X), static_cast<const T*>(d.fitw), blockIdx.y,
-                parts, fit_dyn, chain, slice, se, sx);
+  fit_units_f64(fa, f, static_cast<const double*>(d.X), static_cast<const double*>(d.fitw),
+                units * blockIdx.y / parts, units * (blockIdx.y + 1) / parts, fit_dyn, chain, slice,
+                se, sx);
   fit_block_reduce(se, sx, red);
   if (threadIdx.x == 0) {
     d.fitp[blockIdx.y] = se;
@@ -92,28 +122,27 @@ __global__ void __launch_bounds__(FNT) kb_fit(const BInst* __restrict__ tab, int
   }
 }
 
-// Slots with FP32 X and K <= 128: the contraction on the tensor cores (fit_tc.cuh).
-__global__ void __launch_bounds__(FNT, 1) kb_fit_tc(const BInst* __restrict__ tab,
-                                                    unsigned* err) {
-  extern __shared__ __align__(1024) unsigned char fit_tc_dyn[];
-  __shared__ float chain[8][kMaxL];
-  __shared__ float slice[8][kMaxL];
-  __shared__ double red[2 * (FNT / 32)];
+// Slots with FP32 X: the contraction on the tensor cores (fit_tc.cuh).
+__global__ void __launch_bounds__(FT_NT, 1) kb_fit_tc(const BInst* __restrict__ tab,
+                                                      unsigned* err) {
+  extern __shared__ __align__(128) unsigned char fit_tc_dyn[];
+  __shared__ double red[2 * FT_EW];
   __shared__ FitArgs fa;
   __shared__ FitTcShared sh;
   const BInst& d = tab[blockIdx.x];
-  if (!fit_due(d) || d.xf64) return;
+  if (!fit_due(d)) return;
   if (threadIdx.x == 0) fit_args(d, fa);
   __syncthreads();
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
-  if (!fit_use_tc(f, false)) return;
-  const int parts = fit_parts(f, false);
+  const FitTcPlan pl = fit_tc_plan(fa, f);
+  const int parts = fit_parts(fa, f, false);
   if (static_cast<int>(blockIdx.y) >= parts) return;
   double se = 0.0, sx = 0.0;
-  fit_tc_blocks(fa, f, static_cast<const float*>(d.X),
-                static_cast<const unsigned char*>(d.fitw),
-                blockIdx.y, parts, fit_tc_dyn, chain, slice, sh, err, se, sx);
-  fit_block_reduce(se, sx, red);
+  fit_tc_units(fa, f, pl, static_cast<const float*>(d.X),
+               static_cast<const unsigned char*>(d.fitw), fit_tables(d, fa, f),
+               pl.units * blockIdx.y / parts, pl.units * (blockIdx.y + 1) / parts, fit_tc_dyn, sh,
+               err, se, sx);
+  fit_tc_reduce(se, sx, red);
   if (threadIdx.x == 0) {
     d.fitp[blockIdx.y] = se;
     d.fitp[kFitParts + blockIdx.y] = sx;
@@ -131,8 +160,9 @@ __global__ void __launch_bounds__(128) kb_advance(const BInst* __restrict__ tab,
   const int t = s.step;
   if (t >= 0 && *d.info != 0) s.singular += 1;
   if (fit_due(d)) {
-    const FitSplit f = fit_split(d.N, d.dims, d.ranks);
-    const int parts = fit_parts(f, xf64 != 0);
+    FitArgs fa;
+    fit_args(d, fa);
+    const int parts = fit_parts(fa, fit_split(d.N, d.dims, d.ranks), xf64 != 0);
     double se = 0.0, sx = 0.0;
     for (int q = 0; q < parts; ++q) {
       se += d.fitp[q];
@@ -157,18 +187,13 @@ __global__ void __launch_bounds__(128) kb_advance(const BInst* __restrict__ tab,
 cudaError_t bl_fit(const BLaunch& b, unsigned* err, cudaStream_t st) {
   dim3 rgrid(b.count, kFitRightCtas);
   dim3 grid(b.count, kFitParts);
-  constexpr int kSplitK = 128;
-  const int k_small = b.Lmax < kSplitK ? b.Lmax : kSplitK;
   if (b.xf64) {
-    kb_fit_right<double><<<rgrid, FNT, 0, st>>>(b.tab);
-    kb_fit<double><<<grid, FNT, fit_smem_bytes<double>(k_small), st>>>(b.tab, 0, kSplitK);
-    if (b.Lmax > kSplitK)
-      kb_fit<double><<<grid, FNT, fit_smem_bytes<double>(b.Lmax), st>>>(b.tab, kSplitK, kMaxL);
+    kb_fit_right<<<rgrid, FNT, 0, st>>>(b.tab);
+    kb_fit<<<grid, FNT, fit_smem_bytes(b.Lmax), st>>>(b.tab);
   } else {
-    kb_fit_right<float><<<rgrid, FNT, 0, st>>>(b.tab);
-    kb_fit_tc<<<grid, FNT, kFitTcSmem, st>>>(b.tab, err);
-    if (b.Lmax > kFitTcMaxK)
-      kb_fit<float><<<grid, FNT, fit_smem_bytes<float>(b.Lmax), st>>>(b.tab, kFitTcMaxK, kMaxL);
+    kb_fit_tables<<<dim3(b.count, 16), 256, 0, st>>>(b.tab);
+    kb_fit_right_tc<<<rgrid, FT_Q, 0, st>>>(b.tab);
+    kb_fit_tc<<<grid, FT_NT, kFitTcSmem, st>>>(b.tab, err);
   }
   return cudaGetLastError();
 }
@@ -179,14 +204,11 @@ cudaError_t bl_advance(const BLaunch& b, cudaStream_t st) {
 }
 
 cudaError_t batched_fit_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(kb_fit<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(fit_smem_bytes<float>(kMaxL)));
+  cudaError_t e = cudaFuncSetAttribute(kb_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(fit_smem_bytes(kMaxL)));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(kb_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kFitTcSmem));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kb_fit<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(fit_smem_bytes<double>(kMaxL)));
+  return cudaFuncSetAttribute(kb_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kFitTcSmem));
 }
 
 }  // namespace trk

@@ -6,26 +6,27 @@
 namespace trk {
 namespace {
 
-template <typename T>
-__global__ void __launch_bounds__(FNT) k_fit_right(FitArgs a, FitSplit f, T* __restrict__ WT) {
-  __shared__ T chain[8][kMaxL];
-  __shared__ T slice[8][kMaxL];
+__global__ void __launch_bounds__(FNT) k_fit_right(FitArgs a, FitSplit f,
+                                                   double* __restrict__ WT) {
+  __shared__ double chain[8][kMaxL];
+  __shared__ double slice[8][kMaxL];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t q = static_cast<int64_t>(blockIdx.x) * (FNT / 32) + warp;
   if (q >= f.cols) return;
-  fit_right_warp<T>(a, f, q, WT, chain[warp], slice[warp], lane);
+  fit_right_warp(a, f, q, WT, chain[warp], slice[warp], lane);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const T* __restrict__ X,
-                                             const T* __restrict__ WT,
+__global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const double* __restrict__ X,
+                                             const double* __restrict__ WT,
                                              double* __restrict__ partial, int blocks) {
   extern __shared__ __align__(16) unsigned char fit_smem_raw[];
-  __shared__ T chain[8][kMaxL];
-  __shared__ T slice[8][kMaxL];
+  __shared__ double chain[8][kMaxL];
+  __shared__ double slice[8][kMaxL];
   __shared__ double red[2 * (FNT / 32)];
+  const int64_t units = fit_units(f);
   double se = 0.0, sx = 0.0;
-  fit_blocks<T>(a, f, X, WT, blockIdx.x, gridDim.x, fit_smem_raw, chain, slice, se, sx);
+  fit_units_f64(a, f, X, WT, units * blockIdx.x / gridDim.x, units * (blockIdx.x + 1) / gridDim.x,
+                fit_smem_raw, chain, slice, se, sx);
   fit_block_reduce(se, sx, red);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = se;
@@ -33,30 +34,34 @@ __global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const T* __r
   }
 }
 
-__global__ void __launch_bounds__(FNT) k_fit_right_tc(FitArgs a, FitSplit f,
-                                                     unsigned char* __restrict__ WS) {
-  __shared__ float chain[8][kMaxL];
-  __shared__ float slice[8][kMaxL];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t ncol = (f.cols + FTN - 1) / FTN * FTN;
-  const int64_t q = static_cast<int64_t>(blockIdx.x) * (FNT / 32) + warp;
-  if (q >= ncol) return;
-  fit_right_tc_warp(a, f, q, WS, chain[warp], slice[warp], lane);
+// FP32 slice tables of the modes s - 1 and N - 1 (fit_tc.cuh), one warp per slice.
+__global__ void __launch_bounds__(256) k_fit_tables(FitArgs a, FitSplit f,
+                                                    float* __restrict__ out) {
+  fit_tables_warps(a, f, out, (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5,
+                   static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5));
 }
 
-__global__ void __launch_bounds__(FNT, 1) k_fit_tc(FitArgs a, FitSplit f,
-                                                   const float* __restrict__ X,
-                                                   const unsigned char* __restrict__ WS,
-                                                   double* __restrict__ partial, int blocks,
-                                                   unsigned* err) {
-  extern __shared__ __align__(1024) unsigned char fit_tc_raw[];
-  __shared__ float chain[8][kMaxL];
-  __shared__ float slice[8][kMaxL];
-  __shared__ double red[2 * (FNT / 32)];
+__global__ void __launch_bounds__(FT_Q) k_fit_right_tc(FitArgs a, FitSplit f, const float* tables,
+                                                       unsigned char* __restrict__ WS) {
+  __shared__ __align__(16) float P[32 * 256];
+  __shared__ float G[4 * kMaxL];
+  fit_right_tc_tile(a, f, blockIdx.x, 2 * blockIdx.y, 2 * blockIdx.y + 2,
+                    tables ? tables + fit_tc_table_floats(a, f.s - 1) : nullptr, WS, P, G);
+}
+
+__global__ void __launch_bounds__(FT_NT, 1) k_fit_tc(FitArgs a, FitSplit f, FitTcPlan pl,
+                                                     const float* __restrict__ X,
+                                                     const unsigned char* __restrict__ WS,
+                                                     const float* tables,
+                                                     double* __restrict__ partial, int blocks,
+                                                     unsigned* err) {
+  extern __shared__ __align__(128) unsigned char fit_tc_raw[];
+  __shared__ double red[2 * FT_EW];
   __shared__ FitTcShared sh;
   double se = 0.0, sx = 0.0;
-  fit_tc_blocks(a, f, X, WS, blockIdx.x, gridDim.x, fit_tc_raw, chain, slice, sh, err, se, sx);
-  fit_block_reduce(se, sx, red);
+  fit_tc_units(a, f, pl, X, WS, tables, pl.units * blockIdx.x / gridDim.x,
+               pl.units * (blockIdx.x + 1) / gridDim.x, fit_tc_raw, sh, err, se, sx);
+  fit_tc_reduce(se, sx, red);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = se;
     partial[blocks + blockIdx.x] = sx;
@@ -69,57 +74,59 @@ size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
 }  // namespace
 
-size_t fit_workspace(const FitArgs& a, bool x_f64, int* blocks) {
+size_t fit_workspace(const FitArgs& a, bool x_f64, int* blocks, size_t* table_bytes) {
   const FitSplit f = split_of(a);
-  int64_t b = fit_row_blocks(f, x_f64);
-  const int64_t cap = fit_use_tc(f, x_f64) ? sm_count() : sm_count() * 4;   // the tensor-core form: 1 CTA/SM
+  int64_t b = x_f64 ? fit_units(f) : fit_tc_plan(a, f).units;
+  // the tensor-core form: one CTA per SM. FP64: four per SM, but with a chain of three or more
+  // modes a CTA's own V costs more than a tile of products, so the CTAs are then whole row
+  // blocks, or equal parts of them while SMs are left over (4^10, rank 10: 279 us with 128 row
+  // blocks on as many CTAs, 352 us with 304 CTAs that form V twice each)
+  int64_t cap = x_f64 ? 4 * sm_count() : sm_count();
+  if (x_f64 && f.s > 2) {
+    const int64_t rb = (f.rows + FL - 1) / FL;
+    const int64_t whole = rb * (sm_count() / rb > 1 ? sm_count() / rb : 1);
+    cap = whole < cap ? whole : cap;
+  }
   if (b > cap) b = cap;
-  if (b < 1) b = 1;
   *blocks = static_cast<int>(b);
-  const size_t es = x_f64 ? 8 : 4;
-  const size_t right = fit_use_tc(f, x_f64) ? fit_tc_right_bytes(f)
-                                            : static_cast<size_t>(f.cols) * f.K * es;
-  return round256(static_cast<size_t>(2 * b) * sizeof(double)) + right;
+  const size_t right = x_f64 ? static_cast<size_t>(f.cols) * f.K * 8 : fit_tc_right_bytes(f);
+  *table_bytes = x_f64 || !fit_tc_tables_fit(a, f)
+                     ? 0 : static_cast<size_t>(fit_tc_tables_floats(a, f)) * sizeof(float);
+  return round256(round256(static_cast<size_t>(2 * b) * sizeof(double)) + right);
 }
 
 cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, void* ws, int blocks,
-                       unsigned* err, cudaStream_t st) {
+                       float* tables, unsigned* err, cudaStream_t st) {
   const FitSplit f = split_of(a);
   double* partial = static_cast<double*>(ws);
   char* wt = static_cast<char*>(ws) + round256(static_cast<size_t>(2 * blocks) * sizeof(double));
-  const unsigned rb = static_cast<unsigned>((f.cols + FNT / 32 - 1) / (FNT / 32));
   if (x_f64) {
+    const unsigned rb = static_cast<unsigned>((f.cols + FNT / 32 - 1) / (FNT / 32));
     double* WT = reinterpret_cast<double*>(wt);
-    k_fit_right<double><<<rb, FNT, 0, st>>>(a, f, WT);
-    k_fit<double><<<blocks, FNT, fit_smem_bytes<double>(f.K), st>>>(
-        a, f, static_cast<const double*>(X), WT, partial, blocks);
+    k_fit_right<<<rb, FNT, 0, st>>>(a, f, WT);
+    k_fit<<<blocks, FNT, fit_smem_bytes(f.K), st>>>(a, f, static_cast<const double*>(X), WT,
+                                                    partial, blocks);
   } else {
-    if (fit_use_tc(f, false)) {
-      unsigned char* WS = reinterpret_cast<unsigned char*>(wt);
-      const int64_t ncol = (f.cols + FTN - 1) / FTN * FTN;
-      k_fit_right_tc<<<static_cast<unsigned>((ncol + FNT / 32 - 1) / (FNT / 32)), FNT, 0, st>>>(
-          a, f, WS);
-      k_fit_tc<<<blocks, FNT, kFitTcSmem, st>>>(a, f, static_cast<const float*>(X), WS, partial,
-                                                 blocks, err);
-    } else {
-      float* WT = reinterpret_cast<float*>(wt);
-      k_fit_right<float><<<rb, FNT, 0, st>>>(a, f, WT);
-      k_fit<float><<<blocks, FNT, fit_smem_bytes<float>(f.K), st>>>(
-          a, f, static_cast<const float*>(X), WT, partial, blocks);
+    const FitTcPlan pl = fit_tc_plan(a, f);
+    unsigned char* WS = reinterpret_cast<unsigned char*>(wt);
+    if (tables) {
+      const int64_t n = (a.dims[f.s - 1] + a.dims[a.N - 1] + 7) / 8;
+      const int64_t tb = n < 8 * sm_count() ? n : 8 * sm_count();
+      k_fit_tables<<<static_cast<unsigned>(tb), 256, 0, st>>>(a, f, tables);
     }
+    k_fit_right_tc<<<dim3(static_cast<unsigned>(pl.tiles), (pl.ks + 1) / 2), FT_Q, 0, st>>>(a, f, tables, WS);
+    k_fit_tc<<<blocks, FT_NT, kFitTcSmem, st>>>(a, f, pl, static_cast<const float*>(X), WS, tables,
+                                                partial, blocks, err);
   }
   return cudaGetLastError();
 }
 
 cudaError_t fit_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_fit<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(fit_smem_bytes<double>(kMaxL)));
+  cudaError_t e = cudaFuncSetAttribute(k_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(fit_smem_bytes(kMaxL)));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kFitTcSmem));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_fit<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(fit_smem_bytes<float>(kMaxL)));
+  return cudaFuncSetAttribute(k_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kFitTcSmem));
 }
 
 cudaError_t cholesky_attributes();

@@ -181,9 +181,7 @@ void free_all(tr_server* s) {
 void carve_request(Carver& c, const tr_request& r, bool f64, bool xf64, BInst& d) {
   carve_instance(c, r.N, r.dims, r.ranks, r.J, f64, d);
   const FitSplit f = fit_split(r.N, r.dims, r.ranks);
-  const size_t simt = static_cast<size_t>(f.cols) * f.K * (xf64 ? 8 : 4);
-  const size_t tcb = fit_use_tc(f, xf64) ? fit_tc_right_bytes(f) : 0;
-  d.fitw = c.take<char>(simt > tcb ? simt : tcb);
+  d.fitw = c.take<char>(xf64 ? static_cast<size_t>(f.cols) * f.K * 8 : fit_tc_right_bytes(f));
 }
 
 size_t request_ws(const tr_request& r, bool f64, bool xf64) {

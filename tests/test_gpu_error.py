@@ -1,0 +1,85 @@
+"""tr_rel_error over the forms its kernels take (Sec. 5.1): row blocks of 64, 128 and 256, one
+column tile and many, ragged rows and columns, left groups of one and of many modes (short last
+modes included), contraction lengths up to 256, misaligned X, and a context whose budget leaves
+no room for the FP32 slice tables.
+
+FP32 X: the products are TF32 pairs with FP32 accumulation, so TR carries at most 3 K / 8 + 2
+truncations of 2^-23 (K <= 256 terms) and the FP32 slice products a few more: 1.2e-5 of ||TR||.
+FP64 X: sums of FP64 products, 1e-12."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from paper_2010_08581_gb300 import inputs
+from paper_2010_08581_gb300 import trals as T
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def _case(dims, ranks, dtype):
+    X, cores = inputs.tr_plus_noise(dims, ranks, seed=5, rel_noise=1e-2, dtype=dtype)
+    off = inputs.random_cores(dims, ranks, 6)
+    return X, [c + 0.02 * e for c, e in zip(cores, off)]
+
+
+def _error(ctx, X, ranks, cores):
+    return T.tr_rel_error(ctx, X, ranks, [inputs.slice_major(c).to(DEV) for c in cores])
+
+
+SHAPES = [((2, 2), (1, 1)), ((1, 1, 500), (2, 3, 4)), ((500, 1, 1), (2, 3, 4)),
+          ((40, 30, 20), (3, 4, 2)), ((65, 3, 257), (7, 9, 11)), ((3, 200, 2, 129), (16, 15, 16, 16)),
+          ((70, 60, 50), (16, 12, 14)), ((9, 8, 7, 6, 5, 4, 3, 2), (3, 4, 5, 6, 7, 8, 9, 10)),
+          ((2,) * 16, (3,) * 16), ((300, 300), (16, 16)), ((100, 3, 90, 31), (5, 10, 10, 8)),
+          ((60, 50, 1031), (10, 10, 10))]
+
+
+@pytest.mark.parametrize("dims,ranks", SHAPES)
+@pytest.mark.parametrize("dtype,tol", [(torch.float32, 1.2e-5), (torch.float64, 1e-12)])
+def test_error_matches_oracle(dims, ranks, dtype, tol):
+    X, cores = _case(dims, ranks, dtype)
+    ctx = T.Context(0)
+    try:
+        got = _error(ctx, X.to(DEV), ranks, cores)
+    finally:
+        ctx.close()
+    ref = orc.rel_error([c.numpy() for c in cores], X.double().numpy())
+    assert abs(got - ref) <= tol
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_error_of_a_misaligned_tensor(shift):
+    dims, ranks = (33, 21, 47), (5, 6, 7)
+    X, cores = _case(dims, ranks, torch.float32)
+    buf = torch.zeros(X.numel() + 8, dtype=torch.float32, device=DEV)
+    view = buf[shift:shift + X.numel()].view(dims)
+    view.copy_(X)
+    ctx = T.Context(0)
+    try:
+        got = _error(ctx, view, ranks, cores)
+    finally:
+        ctx.close()
+    assert abs(got - orc.rel_error([c.numpy() for c in cores], X.double().numpy())) <= 1.2e-5
+
+
+def test_error_without_room_for_the_slice_tables():
+    dims, ranks = (900, 40, 130), (12, 10, 14)
+    X, cores = _case(dims, ranks, torch.float32)
+    Xd = X.to(DEV)
+    ref = orc.rel_error([c.numpy() for c in cores], X.double().numpy())
+    done = 0
+    for kb in range(64, 2048, 64):      # the smallest budgets that the call accepts
+        ctx = T.Context(0, kb << 10)
+        try:
+            assert abs(_error(ctx, Xd, ranks, cores) - ref) <= 1.2e-5
+            done += 1
+        except T.TrError as e:
+            assert e.status == T.TR_ERR_BUDGET
+        finally:
+            ctx.close()
+        if done == 2:
+            break
+    assert done == 2

@@ -410,13 +410,14 @@ size_t solve_bytes(int64_t J, int L, int64_t I, bool f64) {
 
 tr_status solve_contract(tr_ctx* ctx, const SolvePlan& s, const void* A, const void* Y,
                          bool f64, int64_t J, int L, int64_t I, cudaStream_t st,
-                         const int64_t* jdev = nullptr, bool bt_planes = false) {
+                         const int64_t* jdev = nullptr, bool bt_planes = false,
+                         int64_t post = 1) {
   const int64_t ld = L + I;
   if (use_tensor_cores(f64)) {
     TR_LAUNCH("normal_eq_tc", launch_normal_eq_tc(static_cast<const float*>(A),
                                                   static_cast<const float*>(Y), J, L, I,
                                                   static_cast<float*>(s.partial), s.splits,
-                                                  ctx->d_err, st, ctx->wait_limit, jdev));
+                                                  ctx->d_err, st, ctx->wait_limit, jdev, post));
   } else {
     TR_LAUNCH("normal_eq", launch_normal_eq(A, Y, f64, J, L, I, s.partial, s.splits, st, jdev));
   }
@@ -513,7 +514,7 @@ tr_status solve_run(tr_ctx* ctx, char* ws, const void* A, const void* Y, bool f6
 tr_status update_run(tr_ctx* ctx, char* ws, size_t solve_ws, const void* A, const void* Y,
                      bool f64, int64_t J, int Rl, int Rr, int64_t I, double* core_out, double* p,
                      double* cdf, cudaStream_t st, cudaStream_t side,
-                     const int64_t* jdev = nullptr) {
+                     const int64_t* jdev = nullptr, int64_t post = 1) {
   const int L = Rl * Rr;
   Carver c(ws);
   SolvePlan s;
@@ -521,7 +522,7 @@ tr_status update_run(tr_ctx* ctx, char* ws, size_t solve_ws, const void* A, cons
   const bool mixed_lev = !f64 && ctx->factorization != TR_FACTOR_FP64;
   // the distribution branch's tall Gram of B^T runs in double-float from B^T's planes
   const bool bt_planes = p && mixed_lev && ctx->ls_rank != TR_LS_RANK_DROP && I >= L;
-  TR_TRY(solve_contract(ctx, s, A, Y, f64, J, L, I, st, jdev, bt_planes));
+  TR_TRY(solve_contract(ctx, s, A, Y, f64, J, L, I, st, jdev, bt_planes, post));
   if (!p) {   // uniform sampling: the new core needs no distribution
     TR_TRY(solve_cholesky(ctx, s, f64, L, st));
     return solve_rhs(ctx, s, Rl, Rr, I, !f64, core_out, st);
@@ -1362,8 +1363,12 @@ tr_status tr_als(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, const int6
       return fail(ctx, TR_ERR_INVALID_ARG, "dims[%d]=%lld exceeds 2097120 (dense unfolding)", n,
                   static_cast<long long>(dims[n]));
   }
+  size_t core_floats = 0;
+  for (int k = 0; k < N; ++k)
+    core_floats += static_cast<size_t>(dims[k]) * rl_of(ranks, N, k) * ranks[k];
+  const size_t head = static_cast<size_t>(Pmax) * (N - 1);
   Carver dry(nullptr);
-  dry.take<int32_t>(static_cast<size_t>(Pmax) * (N - 1));
+  dry.take<int32_t>(head);
   dry.take<char>(static_cast<size_t>(Pmax) * Lmax * es);
   dry.take<char>(static_cast<size_t>(numel) * es);
   const size_t persist = (dry.off + 255) & ~size_t(255);
@@ -1375,7 +1380,7 @@ tr_status tr_als(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, const int6
   DeviceGuard g(ctx->device);
   TR_TRY(ensure_ws(ctx, persist + solve_max + 256));
   Carver c(ctx->arena);
-  int32_t* idx = c.take<int32_t>(static_cast<size_t>(Pmax) * (N - 1));
+  int32_t* idx = c.take<int32_t>(head);   // or FP32 copies of the cores
   void* A = c.take<char>(static_cast<size_t>(Pmax) * Lmax * es);
   void* Y = c.take<char>(static_cast<size_t>(numel) * es);
   char* ws = ctx->arena + persist;
@@ -1403,13 +1408,30 @@ tr_status tr_als(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, const int6
         ca.rl[m] = rl_of(ranks, N, mode);
         ca.rr[m] = ranks[mode];
       }
-      TR_LAUNCH("enumerate", launch_enumerate(N, n, dd, idx, st));
-      TR_LAUNCH("subchain", launch_subchain(ca, idx, nullptr, P[n], A, f64, ctx->d_err, st));
-      // the last mode's rows are X itself when X already has the LS step's type
-      const void* Yn = (n == N - 1 && x64 == f64) ? X : Y;
-      if (Yn == Y) TR_LAUNCH("unfold", launch_unfold(X, x64, N, n, dd, Y, f64, st));
+      // FP32 rows by runs of the fastest mode where the index buffer has room for FP32 cores
+      // (sums over a sweep: 64 x 8192 x 2, rank 8: 315 -> 144 us; 64 x 256 x 64: 56 -> 43).
+      // FP64 rows are bound by the FP64 pipe and were slower by runs (40 x 30 x 20 x 12: 27 us a
+      // mode row by row, 47 by runs).
+      if (!f64 && core_floats <= head) {
+        TR_LAUNCH("dense_rows", launch_dense_rows(N, n, ca, reinterpret_cast<float*>(idx),
+                                                  static_cast<float*>(A), st));
+      } else {
+        TR_LAUNCH("enumerate", launch_enumerate(N, n, dd, idx, st));
+        TR_LAUNCH("subchain", launch_subchain(ca, idx, nullptr, P[n], A, f64, ctx->d_err, st));
+      }
+      // X_[n]^T is X itself where X already has the LS step's type: in place for the last mode,
+      // and through its strides in the tensor-core contraction, where rows that follow one
+      // another in X fill whole 32-byte sectors (8 of them; fewer are transposed first)
+      int64_t post = 1;
+      for (int k = n + 1; k < N; ++k) post *= dims[k];
+      const bool in_place = x64 == f64 && (post == 1 || (post >= 8 && use_tensor_cores(f64)));
+      const void* Yn = in_place ? X : Y;
+      if (!in_place) {
+        TR_LAUNCH("unfold", launch_unfold(X, x64, N, n, dd, Y, f64, st));
+        post = 1;
+      }
       TR_TRY(update_run(ctx, ws, solve_max, A, Yn, f64, P[n], rl_of(ranks, N, n), ranks[n],
-                        dims[n], cores[n], nullptr, nullptr, st, ctx->side));
+                        dims[n], cores[n], nullptr, nullptr, st, ctx->side, nullptr, post));
     }
   }
   return read_device_error(ctx, st);

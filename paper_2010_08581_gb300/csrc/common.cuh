@@ -99,12 +99,16 @@ cudaError_t launch_gather(const GatherArgs& a, const void* X, bool x_f64, const 
                           cudaStream_t st);
 
 // Dense TR-ALS (Alg. 1) rows: every multi-index of the modes other than n in row-major order
-// (the last mode fastest), written in ring order as idx[P][N-1]; and Y = X_[n]^T with rows
-// in that order (Y[r][i], r = pre * P_post + post for X viewed as [P_pre][I_n][P_post]).
+// (the last mode fastest), written in ring order as idx[P][N-1] (launch_enumerate) or straight
+// as the FP32 rows of G_[2]^{!=n}, A [P][L] (launch_dense_rows; f32_cores: room for FP32 copies
+// of the other cores, sum I_k L_k floats); and Y = X_[n]^T with rows in that order (Y[r][i],
+// r = pre * P_post + post for X viewed as [P_pre][I_n][P_post]).
 struct DenseDims {
   int64_t I[kMaxModes];
 };
 cudaError_t launch_enumerate(int N, int n, const DenseDims& d, int32_t* idx, cudaStream_t st);
+cudaError_t launch_dense_rows(int N, int n, const ChainArgs& ca, float* f32_cores, float* A,
+                              cudaStream_t st);
 cudaError_t launch_unfold(const void* X, bool x_f64, int N, int n, const DenseDims& d, void* Y,
                           bool y_f64, cudaStream_t st);
 
@@ -119,9 +123,12 @@ size_t normal_eq_tc_workspace(int64_t J, int L, int64_t I, int* splits);
 // wait expires the kernel records kErrTimeout in *err and writes no partials.
 // jdev (optional, device): the number of rows actually present (<= J); rows beyond it are
 // not read and the partials of chunks beyond it are zero.
+// post > 1: Y is the tensor X viewed as [J / post][I][post], and the fibre matrix is read from
+// it in place (row r, column i: X[r / post][i][r % post]).
 cudaError_t launch_normal_eq_tc(const float* A, const float* Y, int64_t J, int L, int64_t I,
                                 float* partial, int splits, unsigned* err, cudaStream_t st,
-                                long long wait_limit = -1, const int64_t* jdev = nullptr);
+                                long long wait_limit = -1, const int64_t* jdev = nullptr,
+                                int64_t post = 1);
 cudaError_t launch_normal_eq(const void* A, const void* Y, bool f64, int64_t J, int L,
                              int64_t I, void* partial, int splits, cudaStream_t st,
                              const int64_t* jdev = nullptr);

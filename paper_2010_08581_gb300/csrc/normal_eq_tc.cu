@@ -7,11 +7,20 @@
 // close to FP32 accuracy (Markidis et al., "NVIDIA Tensor Core Programmability,
 // Performance & Precision", 2018; Ootomo & Yokota, 2022).
 //
-// One CTA = one 128 x BN output tile over one chunk of the J samples (split-K, partials
+// One CTA = one 128 x TN output tile over one chunk of the J samples (split-K, partials
 // reduced downstream in a fixed order). All 256 threads load the chunk from global memory
-// (16-byte vectors along the feature / fibre index), split it and store it into K-major,
-// 128-byte-swizzled shared-memory tiles; one elected thread issues the MMAs and commits
-// them to an mbarrier per pipeline stage; TMEM is read back with tcgen05.ld. Every
+// (16-byte vectors along the feature / fibre index), two 32-sample stages ahead in registers,
+// split it and store it into K-major, 128-byte-swizzled shared-memory tiles; one elected thread
+// issues the MMAs and commits them to an mbarrier per pipeline stage; TMEM is read back with
+// tcgen05.ld. The dense method's right-hand sides (X_[n]^T of a strided mode) are read from X
+// where it lies: there 32 consecutive samples of one column are consecutive words of X.
+//
+// A stage is latency: loads, conversion, two barriers and twelve MMAs follow one another. With
+// 128 columns per CTA (129 KB of shared memory) one CTA ran per SM: 2.2 us a stage, and 155
+// CTAs on 152 SMs took two rounds at J = 250,000 (1134 us). With 64 or 80 columns two CTAs
+// share an SM and one's loads and conversions cover the other's MMAs (788 us).
+// The column tile does not change a result: an entry is the same sequence of FP32
+// accumulations over the same chunk of samples whatever the tile. Every
 // mbarrier wait is bounded: a wait of the main loop polls at most `wait_limit` times; on
 // expiry the CTA records an error, stops issuing, waits (bounded by the default limit) for
 // the MMAs it has committed, frees its TMEM and returns without writing its partials.
@@ -22,27 +31,35 @@ namespace trk {
 namespace {
 
 constexpr int TM = 128;          // UMMA M
-constexpr int TN = 128;          // UMMA N (output columns per CTA)
 constexpr int TK = 32;           // samples per pipeline stage (one 128-byte swizzle row)
 constexpr int NT = 256;
 static_assert(TK == 32 && TM == 4 * (NT / 32) * 4,
               "operand loader: one sample per lane, 4 groups of 4 rows per warp");
 constexpr int STAGES = 2;
 constexpr int A_BYTES = TM * TK * 4;   // 16 KB
-constexpr int B_BYTES = TN * TK * 4;   // 16 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // hi and lo of both operands
-constexpr uint32_t TMEM_COLS = TN;     // FP32 accumulator: 128 lanes x TN columns
+constexpr uint32_t TMEM_COLS = 128;    // FP32 accumulator: 128 lanes x TN <= 128 columns
+
+template <int TN>
+constexpr int stage_bytes() { return 2 * A_BYTES + 2 * TN * TK * 4; }   // hi and lo of both
 
 using namespace tc;
 
-constexpr uint32_t kIdesc = idesc_tf32(TM, TN);
-
-__global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict__ A,
+// TN output columns per CTA (MMA N). kDense: the columns from L on are X viewed as
+// [J / post][I][post] (Y points to X, post > 1): Y[r][i] = X[r / post][i][r % post].
+template <int TN, bool kDense>
+__global__ void __launch_bounds__(NT, 2) k_normal_eq_tc(const float* __restrict__ A,
                                                         const float* __restrict__ Y, int64_t J,
-                                                        int L, int64_t I, int64_t chunk,
+                                                        int L, int64_t I, int64_t post,
+                                                        int64_t chunk,
                                                         float* __restrict__ partial,
                                                         unsigned* err, long long wait_limit,
                                                         const int64_t* __restrict__ jdev) {
+  constexpr uint32_t kIdesc = idesc_tf32(TM, TN);
+  constexpr int B_BYTES = TN * TK * 4;
+  constexpr int STAGE_BYTES = stage_bytes<TN>();
+  constexpr int NG = TN / 4;                        // column groups of 4
+  constexpr int NQ = (NG + NT / 32 - 1) / (NT / 32);   // groups per warp, rounded up
+  static_assert(TN % 16 == 0 && TN <= static_cast<int>(TMEM_COLS), "MMA N");
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   // 1024-byte alignment of the tiles (required by the 128-byte swizzle atoms)
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -75,73 +92,103 @@ __global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict_
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_d = tmem_slot;
 
-  // Loaders. Each thread holds TK/2 values of each operand per chunk: 4-wide groups g = u / 4
-  // (u < TK/2) of 4 consecutive tile rows (features for A, output columns for B) at one
-  // sample. With rows of A and Y that are multiples of 16 bytes long (and 16-byte aligned
-  // bases) a group is one 16-byte load; otherwise four scalar loads with bounds.
-  const bool vec = (L % 4) == 0 && (I % 4) == 0 &&
-                   (reinterpret_cast<uintptr_t>(A) % 16) == 0 &&
-                   (reinterpret_cast<uintptr_t>(Y) % 16) == 0;
-  // group q (0..3) of thread t: sample k = lane, tile rows 4 g .. 4 g + 3 with
-  // g = warp + 8 q. Lanes cover consecutive samples, so the stores into the K-major swizzled
-  // tile below hit 32 different banks (consecutive k of one row span the whole 128-byte line).
-  auto load_chunk = [&](int c, float (&ra)[TK / 2], float (&rb)[TK / 2]) {
-    const int64_t jb = j0 + static_cast<int64_t>(c) * TK;
+  // Loaders. Groups of 4 consecutive tile rows (features for A, output columns for B) at one
+  // sample: with rows of A and Y that are multiples of 16 bytes long (and 16-byte aligned
+  // bases) a group is one 16-byte load, otherwise four scalar loads with bounds. Group q of
+  // thread t: sample k = lane, tile rows 4 g .. 4 g + 3 with g = warp + 8 q. Lanes cover
+  // consecutive samples, so the stores into the K-major swizzled tile below hit 32 different
+  // banks (consecutive k of one row span the whole 128-byte line).
+  const bool vec_a = (L % 4) == 0 && (reinterpret_cast<uintptr_t>(A) % 16) == 0;
+  const bool vec_y = !kDense && vec_a && (I % 4) == 0 && (reinterpret_cast<uintptr_t>(Y) % 16) == 0;
+  auto load_chunk = [&](int c, float (&ra)[TK / 2], float (&rb)[4 * NQ]) {
+    if (c >= nchunks) return;
+    const int64_t j = j0 + static_cast<int64_t>(c) * TK + lane;
+    const bool in = j < j1;
+    const float* arow = A + j * L;
+    const float* yrow = Y + (kDense ? 0 : j * I);
+    if constexpr (kDense) {
+      int64_t pre, at;
+      if (J <= INT32_MAX) {
+        const uint32_t p = static_cast<uint32_t>(j) / static_cast<uint32_t>(post);
+        pre = p;
+        at = static_cast<uint32_t>(j) - p * static_cast<uint32_t>(post);
+      } else {
+        pre = j / post;
+        at = j - pre * post;
+      }
+      yrow = Y + pre * I * post + at;
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int64_t j = jb + lane;
-      const int r4 = 4 * (warp + (NT / 32) * q);
-      const int am = m0 + r4;
-      const int64_t bn = n0 + r4;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-      if (j < j1) {
-        if (vec) {
-          if (am < L) a = __ldg(reinterpret_cast<const float4*>(A + j * L + am));
-          if (bn < L) b = __ldg(reinterpret_cast<const float4*>(A + j * L + bn));
-          else if (bn < ldc) b = __ldg(reinterpret_cast<const float4*>(Y + j * I + (bn - L)));
+      const int am = m0 + 4 * (warp + (NT / 32) * q);
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in) {
+        if (vec_a) {
+          if (am < L) a = __ldg(reinterpret_cast<const float4*>(arow + am));
         } else {
-          float av[4], bv[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            av[i] = (am + i < L) ? __ldg(A + j * L + am + i) : 0.f;
-            const int64_t c2 = bn + i;
-            bv[i] = c2 < L ? __ldg(A + j * L + c2)
-                           : (c2 < ldc ? __ldg(Y + j * I + (c2 - L)) : 0.f);
-          }
-          a = make_float4(av[0], av[1], av[2], av[3]);
-          b = make_float4(bv[0], bv[1], bv[2], bv[3]);
+          if (am < L) a.x = __ldg(arow + am);
+          if (am + 1 < L) a.y = __ldg(arow + am + 1);
+          if (am + 2 < L) a.z = __ldg(arow + am + 2);
+          if (am + 3 < L) a.w = __ldg(arow + am + 3);
         }
       }
       ra[4 * q] = a.x; ra[4 * q + 1] = a.y; ra[4 * q + 2] = a.z; ra[4 * q + 3] = a.w;
-      rb[4 * q] = b.x; rb[4 * q + 1] = b.y; rb[4 * q + 2] = b.z; rb[4 * q + 3] = b.w;
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int g = warp + (NT / 32) * q;
+      const int64_t bn = n0 + 4 * g;
+      float b[4] = {0.f, 0.f, 0.f, 0.f};
+      if (in && g < NG && bn < ldc) {
+        if (vec_a && bn < L) {             // L % 4 == 0: the whole group is in A
+          const float4 v = __ldg(reinterpret_cast<const float4*>(arow + bn));
+          b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+        } else if (vec_y) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(yrow + (bn - L)));
+          b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int64_t c2 = bn + i;
+            if (c2 < L) b[i] = __ldg(arow + c2);
+            else if (c2 < ldc) b[i] = __ldg(yrow + (c2 - L) * (kDense ? post : 1));
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rb[4 * q + i] = b[i];
     }
   };
-  float ca[TK / 2], cb[TK / 2], na[TK / 2], nb[TK / 2];
-  if (nchunks > 0) load_chunk(0, ca, cb);
   int issued = 0;
-
-  for (int c = 0; c < nchunks; ++c) {
+  // Splits chunk c's values, stores them into its stage and issues its MMAs; false when a
+  // bounded wait expired.
+  auto run_chunk = [&](int c, const float (&ra)[TK / 2], const float (&rb)[4 * NQ]) -> bool {
+    if (c >= nchunks) return false;
     const int s = c % STAGES;
     unsigned char* st = base + s * STAGE_BYTES;
-    if (c + 1 < nchunks) load_chunk(c + 1, na, nb);   // in flight while this chunk is stored
     if (c >= STAGES) {   // wait until the MMAs that read this stage have finished
       const bool ok = mbar_wait(smem_u32(&mbar[s]), ((c / STAGES) - 1) & 1, wait_limit);
       if (!ok) atomicExch(&s_abort, 1);
     }
     __syncthreads();
-    if (s_abort) break;
+    if (s_abort) return false;
 #pragma unroll
     for (int u = 0; u < TK / 2; ++u) {
-      const int k = lane;
       const int row = 4 * (warp + (NT / 32) * (u / 4)) + (u % 4);
-      const float a = ca[u], b = cb[u];
-      const float ah = tf32_rna(a), bh = tf32_rna(b);
-      const float al = tf32_rna(a - ah), bl = tf32_rna(b - bh);
-      const uint32_t oa = sw128_offset(row, k);
-      *reinterpret_cast<float*>(st + oa) = ah;
-      *reinterpret_cast<float*>(st + A_BYTES + oa) = al;
-      *reinterpret_cast<float*>(st + 2 * A_BYTES + oa) = bh;
-      *reinterpret_cast<float*>(st + 2 * A_BYTES + B_BYTES + oa) = bl;
+      const float ah = tf32_rna(ra[u]);
+      const uint32_t o = sw128_offset(row, lane);
+      *reinterpret_cast<float*>(st + o) = ah;
+      *reinterpret_cast<float*>(st + A_BYTES + o) = tf32_rna(ra[u] - ah);
+    }
+#pragma unroll
+    for (int u = 0; u < 4 * NQ; ++u) {
+      const int g = warp + (NT / 32) * (u / 4);
+      if (g < NG) {
+        const float bh = tf32_rna(rb[u]);
+        const uint32_t o = sw128_offset(4 * g + (u % 4), lane);
+        *reinterpret_cast<float*>(st + 2 * A_BYTES + o) = bh;
+        *reinterpret_cast<float*>(st + 2 * A_BYTES + B_BYTES + o) = tf32_rna(rb[u] - bh);
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -160,8 +207,20 @@ __global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict_
       mma_commit(smem_u32(&mbar[s]));
     }
     issued = c + 1;
-#pragma unroll
-    for (int r = 0; r < TK / 2; ++r) { ca[r] = na[r]; cb[r] = nb[r]; }
+    return true;
+  };
+  {
+    float a0[TK / 2], b0[4 * NQ], a1[TK / 2], b1[4 * NQ], a2[TK / 2], b2[4 * NQ];
+    load_chunk(0, a0, b0);
+    load_chunk(1, a1, b1);
+    for (int c = 0; c < nchunks; c += 3) {   // two chunks in flight while one is stored
+      load_chunk(c + 2, a2, b2);
+      if (!run_chunk(c, a0, b0)) break;
+      load_chunk(c + 3, a0, b0);
+      if (!run_chunk(c + 1, a1, b1)) break;
+      load_chunk(c + 4, a1, b1);
+      if (!run_chunk(c + 2, a2, b2)) break;
+    }
   }
   __syncthreads();
   const int aborted = s_abort;
@@ -194,19 +253,17 @@ __global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict_
     }
   } else {
     // Epilogue through shared memory (every MMA has completed, so the stage buffers are
-    // free): warp w moves TMEM lanes 32*(w%4).. (tile rows) of column half w/4 into a
-    // [TM][TN + 1] tile (odd stride: no bank conflicts), then the warps write whole rows,
-    // 32 consecutive columns per store instruction.
+    // free): warp w moves TMEM lanes 32*(w%4).. (tile rows) of every other 16-column piece
+    // into a [TM][TN + 1] tile (odd stride: no bank conflicts), then the warps write whole
+    // rows, 32 consecutive columns per store instruction.
     float* tile = reinterpret_cast<float*>(base);
     const int quad = warp & 3, half = warp >> 2;
     const int rl = quad * 32 + lane;
+    for (int col = half * 16; col < TN; col += 32) {
+      float v[16];
+      tmem_load16(tmem_d + (static_cast<uint32_t>(quad * 32) << 16) + col, v);
 #pragma unroll
-    for (int cc = 0; cc < TN / 64; ++cc) {
-      const int col = half * (TN / 2) + cc * 32;
-      float v[32];
-      tmem_load32(tmem_d + (static_cast<uint32_t>(quad * 32) << 16) + col, v);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) tile[rl * (TN + 1) + col + i] = v[i];
+      for (int i = 0; i < 16; ++i) tile[rl * (TN + 1) + col + i] = v[i];
     }
     __syncthreads();
     for (int r = warp; r < TM; r += NT / 32) {
@@ -214,9 +271,9 @@ __global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict_
       if (m >= L) break;
       float* out = partial + (static_cast<int64_t>(blockIdx.z) * L + m) * ldc + n0;
 #pragma unroll
-      for (int q = 0; q < TN / 32; ++q) {
+      for (int q = 0; q < (TN + 31) / 32; ++q) {
         const int c = lane + 32 * q;
-        if (n0 + c < ldc) out[c] = tile[r * (TN + 1) + c];
+        if (c < TN && n0 + c < ldc) out[c] = tile[r * (TN + 1) + c];
       }
     }
   }
@@ -227,8 +284,11 @@ __global__ void __launch_bounds__(NT, 1) k_normal_eq_tc(const float* __restrict_
                  :: "r"(tmem_d), "r"(TMEM_COLS) : "memory");
 }
 
+// The split of the samples: every entry of the result is summed within these chunks, in
+// order. It was laid down for 128-column tiles, one CTA per SM, and is kept because it fixes
+// the result's rounding; the launch below chooses the column tile.
 void plan_tc(int64_t J, int L, int64_t I, int* splits, int64_t* chunk) {
-  const int64_t tiles = ((L + TM - 1) / TM) * ((L + I + TN - 1) / TN);
+  const int64_t tiles = ((L + TM - 1) / TM) * ((L + I + 127) / 128);
   int64_t s = (sm_count() + tiles - 1) / tiles;
   const int64_t maxs = (J + 4 * TK - 1) / (4 * TK);   // at least 4 stages per CTA
   if (s > maxs) s = maxs;
@@ -238,6 +298,16 @@ void plan_tc(int64_t J, int L, int64_t I, int* splits, int64_t* chunk) {
   s = (J + c - 1) / c;
   *splits = static_cast<int>(s);
   *chunk = c;
+}
+
+template <int TN, bool kDense>
+cudaError_t launch_tn(const float* A, const float* Y, int64_t J, int L, int64_t I, int64_t post,
+                      int64_t chunk, int splits, float* partial, unsigned* err, cudaStream_t st,
+                      long long wait_limit, const int64_t* jdev) {
+  dim3 grid(static_cast<unsigned>((L + I + TN - 1) / TN), (L + TM - 1) / TM, splits);
+  k_normal_eq_tc<TN, kDense><<<grid, NT, STAGES * stage_bytes<TN>() + 1024, st>>>(
+      A, Y, J, L, I, post, chunk, partial, err, wait_limit < 0 ? kTcSpinLimit : wait_limit, jdev);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -250,21 +320,41 @@ size_t normal_eq_tc_workspace(int64_t J, int L, int64_t I, int* splits) {
 
 cudaError_t launch_normal_eq_tc(const float* A, const float* Y, int64_t J, int L, int64_t I,
                                 float* partial, int splits, unsigned* err, cudaStream_t st,
-                                long long wait_limit, const int64_t* jdev) {
+                                long long wait_limit, const int64_t* jdev, int64_t post) {
   int s;
   int64_t chunk;
   plan_tc(J, L, I, &s, &chunk);
   if (s != splits) return cudaErrorInvalidValue;
-  dim3 grid(static_cast<unsigned>((L + I + TN - 1) / TN), (L + TM - 1) / TM, s);
-  const size_t dyn = STAGES * STAGE_BYTES + 1024;
-  k_normal_eq_tc<<<grid, NT, dyn, st>>>(A, Y, J, L, I, chunk, partial, err,
-                                        wait_limit < 0 ? kTcSpinLimit : wait_limit, jdev);
-  return cudaGetLastError();
+  // The busiest SM's share: CTAs per SM times the work of a stage (the tile's columns plus A's
+  // 128 rows, which every column tile converts again). 64 columns unless 80 save a round of
+  // CTAs: J = 250,000, L = 100, I = 500 gives 310 CTAs or 248, three or two on an SM.
+  const int64_t mt = (L + TM - 1) / TM, sms = sm_count();
+  auto share = [&](int tn) {
+    const int64_t ctas = mt * ((L + I + tn - 1) / tn) * splits;
+    return ((ctas + sms - 1) / sms) * (tn + TM);
+  };
+  const bool wide = share(80) < share(64);
+  if (post > 1)
+    return wide ? launch_tn<80, true>(A, Y, J, L, I, post, chunk, splits, partial, err, st,
+                                      wait_limit, jdev)
+                : launch_tn<64, true>(A, Y, J, L, I, post, chunk, splits, partial, err, st,
+                                      wait_limit, jdev);
+  return wide ? launch_tn<80, false>(A, Y, J, L, I, 1, chunk, splits, partial, err, st, wait_limit,
+                                     jdev)
+              : launch_tn<64, false>(A, Y, J, L, I, 1, chunk, splits, partial, err, st, wait_limit,
+                                     jdev);
 }
 
 cudaError_t normal_eq_tc_attributes() {
-  return cudaFuncSetAttribute(k_normal_eq_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              STAGES * STAGE_BYTES + 1024);
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_normal_eq_tc<64, false>, attr, STAGES * stage_bytes<64>() + 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_normal_eq_tc<80, false>, attr, STAGES * stage_bytes<80>() + 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_normal_eq_tc<64, true>, attr, STAGES * stage_bytes<64>() + 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_normal_eq_tc<80, true>, attr, STAGES * stage_bytes<80>() + 1024);
+  return e;
 }
 
 }  // namespace trk

@@ -20,8 +20,8 @@ __device__ __forceinline__ bool fit_due(const BInst& d) {
 }
 
 // Partial sums of one slot's fit: one per CTA, at most kFitParts.
-__device__ __forceinline__ int fit_parts(const FitArgs& fa, const FitSplit& f, bool xf64) {
-  const int64_t n = xf64 ? (fit_units(f) + 7) / 8 : fit_tc_parts(fit_tc_plan(fa, f));
+__device__ __forceinline__ int fit_parts(const FitArgs& fa, const FitSplit& f, bool f64_form) {
+  const int64_t n = f64_form ? (fit_units(f) + 7) / 8 : fit_tc_parts(fit_tc_plan(fa, f));
   return n < kFitParts ? static_cast<int>(n) : kFitParts;
 }
 
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(FNT) kb_fit_right(const BInst* __restrict__ ta
 
 // ... or the split operand tiles of the tensor-core contraction.
 __global__ void __launch_bounds__(FT_Q) kb_fit_right_tc(const BInst* __restrict__ tab) {
-  __shared__ __align__(16) float P[32 * 256];
+  __shared__ __align__(16) float P[32 * 256];   // 8 chains of kMaxL doubles in the FP64 form
   __shared__ float G[4 * kMaxL];
   __shared__ FitArgs fa;
   const BInst& d = tab[blockIdx.x];
@@ -88,6 +88,14 @@ __global__ void __launch_bounds__(FT_Q) kb_fit_right_tc(const BInst* __restrict_
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
   const float* tables = fit_tables(d, fa, f);
   if (tables) tables += fit_tc_table_floats(fa, f.s - 1);
+  if (d.fit_plain) {        // FP32 W^T for the FP64 form
+    double (*chain)[kMaxL] = reinterpret_cast<double (*)[kMaxL]>(P);
+    const int warp = threadIdx.x >> 5;
+    for (int64_t q = static_cast<int64_t>(blockIdx.y) * 4 + warp; q < f.cols; q += 4 * gridDim.y)
+      fit_right_warp(fa, f, q, static_cast<float*>(d.fitw), chain[warp], chain[4 + warp],
+                     static_cast<int>(threadIdx.x & 31));
+    return;
+  }
   const int nj = (f.K + 2 * FT_KS - 1) / (2 * FT_KS);      // jobs of two k-steps
   const int64_t jobs = (f.cols + FT_Q - 1) / FT_Q * nj;
   for (int64_t j = blockIdx.y; j < jobs; j += gridDim.y) {
@@ -135,9 +143,23 @@ __global__ void __launch_bounds__(FT_NT, 1) kb_fit_tc(const BInst* __restrict__ 
   __syncthreads();
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
   const FitTcPlan pl = fit_tc_plan(fa, f);
-  const int parts = fit_parts(fa, f, false);
+  const int parts = fit_parts(fa, f, d.fit_plain);
   if (static_cast<int>(blockIdx.y) >= parts) return;
   double se = 0.0, sx = 0.0;
+  if (d.fit_plain) {        // admitted without room for the operand of W
+    if (threadIdx.x >= FNT) return;
+    double (*chain)[kMaxL] = reinterpret_cast<double (*)[kMaxL]>(fit_tc_dyn + fit_smem_bytes(f.K));
+    const int64_t units = fit_units(f);
+    fit_units_f64(fa, f, static_cast<const float*>(d.X), static_cast<const float*>(d.fitw),
+                  units * blockIdx.y / parts, units * (blockIdx.y + 1) / parts, fit_tc_dyn, chain,
+                  chain + FNT / 32, se, sx);
+    fit_block_reduce(se, sx, red);
+    if (threadIdx.x == 0) {
+      d.fitp[blockIdx.y] = se;
+      d.fitp[kFitParts + blockIdx.y] = sx;
+    }
+    return;
+  }
   fit_tc_units(fa, f, pl, static_cast<const float*>(d.X),
                static_cast<const unsigned char*>(d.fitw), fit_tables(d, fa, f),
                pl.units * blockIdx.y / parts, pl.units * (blockIdx.y + 1) / parts, fit_tc_dyn, sh,
@@ -162,7 +184,7 @@ __global__ void __launch_bounds__(128) kb_advance(const BInst* __restrict__ tab,
   if (fit_due(d)) {
     FitArgs fa;
     fit_args(d, fa);
-    const int parts = fit_parts(fa, fit_split(d.N, d.dims, d.ranks), xf64 != 0);
+    const int parts = fit_parts(fa, fit_split(d.N, d.dims, d.ranks), xf64 != 0 || d.fit_plain);
     double se = 0.0, sx = 0.0;
     for (int q = 0; q < parts; ++q) {
       se += d.fitp[q];

@@ -6,8 +6,8 @@
 namespace trk {
 namespace {
 
-__global__ void __launch_bounds__(FNT) k_fit_right(FitArgs a, FitSplit f,
-                                                   double* __restrict__ WT) {
+template <typename T>
+__global__ void __launch_bounds__(FNT) k_fit_right(FitArgs a, FitSplit f, T* __restrict__ WT) {
   __shared__ double chain[8][kMaxL];
   __shared__ double slice[8][kMaxL];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -16,8 +16,9 @@ __global__ void __launch_bounds__(FNT) k_fit_right(FitArgs a, FitSplit f,
   fit_right_warp(a, f, q, WT, chain[warp], slice[warp], lane);
 }
 
-__global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const double* __restrict__ X,
-                                             const double* __restrict__ WT,
+template <typename T>
+__global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const T* __restrict__ X,
+                                             const T* __restrict__ WT,
                                              double* __restrict__ partial, int blocks) {
   extern __shared__ __align__(16) unsigned char fit_smem_raw[];
   __shared__ double chain[8][kMaxL];
@@ -72,10 +73,34 @@ FitSplit split_of(const FitArgs& a) { return fit_split(a.N, a.dims, a.ranks); }
 
 size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
+template <typename T>
+void fit_f64(const FitArgs& a, const FitSplit& f, const void* X, char* wt, double* partial,
+             int blocks, cudaStream_t st) {
+  const unsigned rb = static_cast<unsigned>((f.cols + FNT / 32 - 1) / (FNT / 32));
+  T* WT = reinterpret_cast<T*>(wt);
+  k_fit_right<T><<<rb, FNT, 0, st>>>(a, f, WT);
+  k_fit<T><<<blocks, FNT, fit_smem_bytes(f.K), st>>>(a, f, static_cast<const T*>(X), WT, partial,
+                                                     blocks);
+}
+
+// FP32 X on the FP64 form (fit_body.cuh).
+bool fit_plain(const FitSplit& f, bool x_f64, bool tight) { return tight && !x_f64 && f.K > FKPlain; }
+
 }  // namespace
 
-size_t fit_workspace(const FitArgs& a, bool x_f64, int* blocks, size_t* table_bytes) {
+size_t fit_workspace(const FitArgs& a, bool x_f64, bool tight, int* blocks, size_t* table_bytes) {
   const FitSplit f = split_of(a);
+  if (tight) {   // as little room as one CTA per row block takes
+    const bool plain = fit_plain(f, x_f64, true);
+    const int64_t edge = x_f64 ? FL : (plain ? 2 * FL : FT_Q);
+    const int64_t most = x_f64 || plain ? 4 * sm_count() : sm_count();
+    const int64_t rb = (f.rows + edge - 1) / edge;
+    *blocks = static_cast<int>(rb < most ? rb : most);
+    *table_bytes = 0;
+    return round256(static_cast<size_t>(2 * *blocks) * sizeof(double)) +
+           (x_f64 || plain ? static_cast<size_t>(f.cols) * f.K * (x_f64 ? 8 : 4)
+                           : fit_tc_right_bytes(f));
+  }
   int64_t b = x_f64 ? fit_units(f) : fit_tc_plan(a, f).units;
   // the tensor-core form: one CTA per SM. FP64: four per SM, but with a chain of three or more
   // modes a CTA's own V costs more than a tile of products, so the CTAs are then whole row
@@ -95,17 +120,15 @@ size_t fit_workspace(const FitArgs& a, bool x_f64, int* blocks, size_t* table_by
   return round256(round256(static_cast<size_t>(2 * b) * sizeof(double)) + right);
 }
 
-cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, void* ws, int blocks,
-                       float* tables, unsigned* err, cudaStream_t st) {
+cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, bool tight, void* ws,
+                       int blocks, float* tables, unsigned* err, cudaStream_t st) {
   const FitSplit f = split_of(a);
   double* partial = static_cast<double*>(ws);
   char* wt = static_cast<char*>(ws) + round256(static_cast<size_t>(2 * blocks) * sizeof(double));
   if (x_f64) {
-    const unsigned rb = static_cast<unsigned>((f.cols + FNT / 32 - 1) / (FNT / 32));
-    double* WT = reinterpret_cast<double*>(wt);
-    k_fit_right<<<rb, FNT, 0, st>>>(a, f, WT);
-    k_fit<<<blocks, FNT, fit_smem_bytes(f.K), st>>>(a, f, static_cast<const double*>(X), WT,
-                                                    partial, blocks);
+    fit_f64<double>(a, f, X, wt, partial, blocks, st);
+  } else if (fit_plain(f, x_f64, tight)) {
+    fit_f64<float>(a, f, X, wt, partial, blocks, st);
   } else {
     const FitTcPlan pl = fit_tc_plan(a, f);
     unsigned char* WS = reinterpret_cast<unsigned char*>(wt);
@@ -122,8 +145,11 @@ cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, void* ws, in
 }
 
 cudaError_t fit_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_fit<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(fit_smem_bytes(kMaxL)));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_fit<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(fit_smem_bytes(kMaxL)));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kFitTcSmem));

@@ -11,7 +11,8 @@
 //
 // The split is chosen so that cols is large enough to amortise the row chains while the right
 // factors stay small (fit_split). FP32 X is evaluated on the tensor cores (fit_tc.cuh). This
-// file holds the split and the FP64 form: W is formed once per evaluation (fit_right_warp,
+// file holds the split and the FP64 form (also for FP32 X with K > 128 where the budget has no
+// room for the tensor cores' operand of W, twice the size of FP32 W^T): W is formed once per evaluation (fit_right_warp,
 // e-major: W^T[e][q]) and V per block of FL rows in shared memory; each thread computes a
 // 2 x 2 register tile of TR from two vector loads per e.
 //
@@ -30,6 +31,7 @@ constexpr int FNT = 256;                       // threads of a fit CTA
 constexpr int64_t kFitMinCols = 256;           // grow cols (move s left) up to this
 constexpr int64_t kFitMaxRight = 1ll << 22;    // max elements of W^T (cols * K)
 
+constexpr int FKPlain = 128;                   // FP32 X: W's operand is never larger than W^T up to here
 constexpr int FL = 32, FI = 32;                // rows and columns of an FP64 tile
 constexpr int FMI = 2, FMJ = 2;                // outputs per thread
 
@@ -107,22 +109,27 @@ __device__ __forceinline__ int warp_slice_product(const FitArgs& a, int m0, int 
 
 // W^T[e][q] = P_right(q)[b][a] (e = b * R_{N-1} + a: the row-major index of P_right) for
 // column q, one warp; S and G are per-warp scratch of kMaxL elements.
+template <typename T>
 __device__ __forceinline__ void fit_right_warp(const FitArgs& a, const FitSplit& f, int64_t q,
-                                               double* __restrict__ WT, double* S, double* G,
-                                               int lane) {
+                                               T* __restrict__ WT, double* S, double* G, int lane) {
   const int N = a.N;
   int64_t ii[kMaxModes];
   int64_t rem = q;
   for (int m = N - 1; m >= f.s; --m) { ii[m] = rem % a.dims[m]; rem /= a.dims[m]; }
   warp_slice_product(a, f.s, N, ii, S, G, lane);
   __syncwarp();
-  for (int e = lane; e < f.K; e += 32) WT[e * f.cols + q] = S[e];
+  for (int e = lane; e < f.K; e += 32) WT[e * f.cols + q] = static_cast<T>(S[e]);
   __syncwarp();
+}
+
+// Barrier of the first FNT threads of a CTA.
+__device__ __forceinline__ void fit_sync() {
+  asm volatile("bar.sync 2, %0;" :: "n"(FNT) : "memory");
 }
 
 // V_p[e] (e = b * R_{N-1} + a, V_p[e] = P_left(p)[a][b]) for the rows p0 .. p0 + nb - 1 of a
 // block and the entries e0 <= e < e1, handed to put(ll, e, value) (rows past the end give
-// zeros). All threads of the CTA call it; it ends with a CTA barrier.
+// zeros). The first FNT threads of the CTA call it; it ends with their barrier.
 //
 // Rows p = pre * J + last (J = I_{s-1}) share the prefix G^(0) .. G^(s-2) of their slice
 // chain, and consecutive rows mostly share it: each distinct prefix of the block is formed
@@ -147,7 +154,7 @@ __device__ void build_left(const FitArgs& a, const FitSplit& f, int64_t p0, int 
       const int b = e / Rlast, aa = e - b * Rlast;
       put(ll, e, p < rows ? a.core[0][(p * Rlast + aa) * Rs + b] : 0.0);
     }
-    __syncthreads();
+    fit_sync();
     return;
   }
   const int64_t J = a.dims[s - 1];
@@ -173,7 +180,7 @@ __device__ void build_left(const FitArgs& a, const FitSplit& f, int64_t p0, int 
       }
       __syncwarp();
     }
-    __syncthreads();
+    fit_sync();
     return;
   }
   const int Rm = a.ranks[s - 2];   // the rank between the prefix and G^(s-1)
@@ -183,7 +190,7 @@ __device__ void build_left(const FitArgs& a, const FitSplit& f, int64_t p0, int 
     for (int m = s - 2; m >= 0; --m) { ii[m] = rem % a.dims[m]; rem /= a.dims[m]; }
     warp_slice_product(a, 0, s - 1, ii, chain[warp], slice[warp], lane);   // Rlast x Rm
   }
-  __syncthreads();
+  fit_sync();
   const double* Gs = a.core[s - 1];
   // columns b whose entries b * Rlast .. b * Rlast + Rlast - 1 meet [e0, K)
   const int b0 = e0 / Rlast, b1 = (K + Rlast - 1) / Rlast;
@@ -212,15 +219,15 @@ __device__ void build_left(const FitArgs& a, const FitSplit& f, int64_t p0, int 
       put(ll, b * Rlast + aa, acc);
     }
   }
-  __syncthreads();
+  fit_sync();
 }
 
 // Accumulates the squared residual (se) and ||X||^2 (sx) over the units lo .. hi - 1 (unit =
-// row block * column tiles + tile). All threads of the CTA must call it. `chain` and `slice`
+// row block * column tiles + tile). The first FNT threads of the CTA call it. `chain` and `slice`
 // are per-warp scratch of kMaxL elements (8 warps); `dyn` holds fit_smem_bytes(f.K).
-__device__ inline void fit_units_f64(const FitArgs& a, const FitSplit& f,
-                                     const double* __restrict__ X,
-                                     const double* __restrict__ WT, int64_t lo, int64_t hi,
+template <typename T>
+__device__ inline void fit_units_f64(const FitArgs& a, const FitSplit& f, const T* __restrict__ X,
+                                     const T* __restrict__ WT, int64_t lo, int64_t hi,
                                      unsigned char* dyn, double (*chain)[kMaxL],
                                      double (*slice)[kMaxL], double& se, double& sx) {
   constexpr int TX = FI / FMJ;   // threads along the columns (16)
@@ -244,7 +251,7 @@ __device__ inline void fit_units_f64(const FitArgs& a, const FitSplit& f,
     const int nq = static_cast<int>((cols - q0 < FI) ? cols - q0 : FI);
     for (int o = threadIdx.x; o < K * FI; o += FNT) {
       const int e = o / FI, iq = o - e * FI;
-      Qt[o] = iq < nq ? WT[e * cols + q0 + iq] : 0.0;
+      Qt[o] = iq < nq ? static_cast<double>(WT[e * cols + q0 + iq]) : 0.0;
     }
     // X in flight while the tile of W lands
     double x[FMI][FMJ];
@@ -254,9 +261,9 @@ __device__ inline void fit_units_f64(const FitArgs& a, const FitSplit& f,
       for (int v = 0; v < FMJ; ++v) {
         const int64_t p = p0 + ty * FMI + i;
         const int iq = tx * FMJ + v;
-        x[i][v] = (p < rows && iq < nq) ? X[p * cols + q0 + iq] : 0.0;
+        x[i][v] = (p < rows && iq < nq) ? static_cast<double>(X[p * cols + q0 + iq]) : 0.0;
       }
-    __syncthreads();
+    fit_sync();
     double acc[FMI][FMJ] = {};
     const double* qp = Qt + tx * FMJ;
 #pragma unroll 4
@@ -279,11 +286,11 @@ __device__ inline void fit_units_f64(const FitArgs& a, const FitSplit& f,
         sx += x[i][v] * x[i][v];
       }
     }
-    __syncthreads();
+    fit_sync();
   }
 }
 
-// Block sum of (se, sx) to thread 0; `red` holds 2 * (FNT / 32) doubles.
+// Sum of (se, sx) over the first FNT threads to thread 0; `red` holds 2 * (FNT / 32) doubles.
 __device__ __forceinline__ void fit_block_reduce(double& se, double& sx, double* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
@@ -292,7 +299,7 @@ __device__ __forceinline__ void fit_block_reduce(double& se, double& sx, double*
     sx += __shfl_xor_sync(0xffffffffu, sx, o);
   }
   if (lane == 0) { red[warp] = se; red[FNT / 32 + warp] = sx; }
-  __syncthreads();
+  fit_sync();
   if (threadIdx.x == 0) {
     double a0 = 0.0, a1 = 0.0;
     for (int w = 0; w < FNT / 32; ++w) { a0 += red[w]; a1 += red[FNT / 32 + w]; }

@@ -91,6 +91,7 @@ struct Pending {
   int64_t ticket;
   tr_request req;
   size_t ws_bytes, charge;
+  bool plain;
 };
 
 std::string g_server_error;   // message of the last failed tr_server_create
@@ -177,17 +178,19 @@ void free_all(tr_server* s) {
 }
 
 // Workspace of one request: distributions, per-update scratch, and the right factors of
-// the fit's mode split (in X's precision).
-void carve_request(Carver& c, const tr_request& r, bool f64, bool xf64, BInst& d) {
+// the fit's mode split (in X's precision; plain: FP32 W^T instead of the larger operand tiles).
+void carve_request(Carver& c, const tr_request& r, bool f64, bool xf64, bool plain, BInst& d) {
   carve_instance(c, r.N, r.dims, r.ranks, r.J, f64, d);
   const FitSplit f = fit_split(r.N, r.dims, r.ranks);
-  d.fitw = c.take<char>(xf64 ? static_cast<size_t>(f.cols) * f.K * 8 : fit_tc_right_bytes(f));
+  d.fitw = c.take<char>(xf64 || plain ? static_cast<size_t>(f.cols) * f.K * (xf64 ? 8 : 4)
+                                      : fit_tc_right_bytes(f));
+  d.fit_plain = plain ? 1 : 0;
 }
 
-size_t request_ws(const tr_request& r, bool f64, bool xf64) {
+size_t request_ws(const tr_request& r, bool f64, bool xf64, bool plain) {
   Carver c(nullptr);
   BInst d{};
-  carve_request(c, r, f64, xf64, d);
+  carve_request(c, r, f64, xf64, plain, d);
   return round256(c.off);
 }
 
@@ -220,11 +223,11 @@ cudaError_t issue_tick(tr_server* s, int count, cudaStream_t st) {
 }
 
 // Fills the table entry and initial state of a newly admitted request.
-void setup_slot(tr_server* s, int id, const tr_request& r) {
+void setup_slot(tr_server* s, int id, const tr_request& r, bool plain) {
   BInst& d = s->htab[id];
   d = BInst{};
   Carver c(s->arena + s->slots[id].ws_off);
-  carve_request(c, r, s->f64, s->xf64, d);
+  carve_request(c, r, s->f64, s->xf64, plain, d);
   d.X = r.X;
   d.N = r.N;
   d.xf64 = s->xf64 ? 1 : 0;
@@ -314,7 +317,7 @@ tr_status run_tick(tr_server* s, int* active_out) {
       sl.charge = p.charge;
       s->charged += p.charge;
       s->stats.peak_charged_bytes = std::max(s->stats.peak_charged_bytes, s->charged);
-      setup_slot(s, id, p.req);
+      setup_slot(s, id, p.req, p.plain);
       s->results[p.ticket].t_admit_ns = now_ns();
       admitted.push_back(id);
       s->hi = std::max(s->hi, id + 1);
@@ -579,9 +582,16 @@ tr_status tr_server_submit(tr_server* s, const tr_request* req, int64_t* ticket)
     s->stats.rejected += 1;
     return chk;
   }
-  const size_t ws = request_ws(r, s->f64, s->xf64);
-  const size_t charge = request_charge(r, s->xf64, ws);
-  if (ws > s->cfg.arena_bytes || charge > s->cfg.hbm_budget_bytes) {
+  size_t ws = request_ws(r, s->f64, s->xf64, false);
+  size_t charge = request_charge(r, s->xf64, ws);
+  auto too_large = [&] { return ws > s->cfg.arena_bytes || charge > s->cfg.hbm_budget_bytes; };
+  // the fit's smaller, slower form rather than a refusal
+  const bool plain = too_large() && !s->xf64 && fit_split(r.N, r.dims, r.ranks).K > FKPlain;
+  if (plain) {
+    ws = request_ws(r, s->f64, s->xf64, true);
+    charge = request_charge(r, s->xf64, ws);
+  }
+  if (too_large()) {
     {
       std::lock_guard<std::mutex> lk(s->mu);
       s->stats.rejected += 1;
@@ -599,7 +609,7 @@ tr_status tr_server_submit(tr_server* s, const tr_request* req, int64_t* ticket)
     tr_result res{};
     res.t_submit_ns = now_ns();
     s->results[t] = res;
-    s->queue.push_back(Pending{t, r, ws, charge});
+    s->queue.push_back(Pending{t, r, ws, charge, plain});
     s->stats.submitted += 1;
     *ticket = t;
   }

@@ -83,3 +83,66 @@ def test_error_without_room_for_the_slice_tables():
         if done == 2:
             break
     assert done == 2
+
+
+def test_error_in_the_least_room():
+    """Ranks of 16 (K = 256) with a budget for FP32 right factors only: the FP64 form, W in FP32
+    (5e-7 of ||TR||); one byte less is refused. FP64 X with one partial sum per 32 rows."""
+    dims, ranks = (70, 13, 9, 50), (16, 16, 16, 16)
+    for dtype, es, edge in ((torch.float32, 4, 64), (torch.float64, 8, 32)):
+        X, cores = _case(dims, ranks, dtype)
+        ref = orc.rel_error([c.numpy() for c in cores], X.double().numpy())
+        cols, rows = 9 * 50, 70 * 13       # the split at 256 columns
+        blocks = min((rows + edge - 1) // edge, 4 * torch.cuda.get_device_properties(0).multi_processor_count)
+        need = (16 * blocks + 255) // 256 * 256 + cols * 256 * es
+        ctx = T.Context(0, need)
+        try:
+            assert abs(_error(ctx, X.to(DEV), ranks, cores) - ref) <= 1e-6
+        finally:
+            ctx.close()
+        ctx = T.Context(0, need - 1)
+        try:
+            with pytest.raises(T.TrError) as e:
+                _error(ctx, X.to(DEV), ranks, cores)
+            assert e.value.status == T.TR_ERR_BUDGET
+        finally:
+            ctx.close()
+
+
+def test_served_request_in_the_least_arena():
+    """A request with K = 256 in the smallest arena that admits it: the same cores as with room
+    to spare, and fits within the two forms' bounds of each other (1.2e-5 + 1e-6)."""
+    dims, ranks, J = (40, 30, 60), (16, 16, 16), 2560
+    X, _ = inputs.tr_plus_noise(dims, (4, 4, 4), seed=21, rel_noise=1e-2)
+    X = X.to(DEV)
+    init = inputs.random_cores(dims, ranks, 22)
+
+    def run(arena):
+        srv = T.Server(max_slots=1, max_modes=3, max_dim=60, max_rank=16, max_samples=J, max_sweeps=2,
+                       fit_tol=0.0, X_dtype=T.TR_F32, prec=T.TR_PREC_MIXED,
+                       hbm_budget_bytes=1 << 30, arena_bytes=arena)
+        try:
+            cores = [inputs.slice_major(c).to(DEV) for c in init]
+            t = srv.submit(X, ranks, J, 23, cores, init_given=True)
+            for _ in range(200):
+                if srv.poll(t)["done"]:
+                    break
+                srv.tick()
+            r = srv.poll(t)
+            assert r["done"]
+            return r["fit_history"][:r["sweeps"]], cores
+        finally:
+            srv.close()
+
+    with pytest.raises(T.TrError) as e:
+        run(1 << 20)
+    assert e.value.status == T.TR_ERR_BUDGET
+    need = int(str(e.value).split("workspace ")[1].split(")")[0])
+    with pytest.raises(T.TrError):
+        run(need - 256)
+    fits, cores = run(need)
+    big, ref = run(64 << 20)
+    assert len(fits) == len(big) == 2
+    assert np.abs(np.asarray(fits) - np.asarray(big)).max() <= 1.3e-5
+    for u, v in zip(cores, ref):
+        assert torch.equal(u, v)

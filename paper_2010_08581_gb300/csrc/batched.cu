@@ -116,19 +116,20 @@ __global__ void __launch_bounds__(SW * 32) kb_sample(const BInst* __restrict__ t
 // Normal equations C = A^T [A | Y] per instance, square output tiles over all samples
 // (no split: one fixed summation order per entry); M = C[:, :L], B^T = C[:, L:]^T in FP64.
 // ------------------------------------------------------------------------------------
-// TILE x TILE outputs per CTA, 4 x 4 per thread; every entry is summed over the samples in
-// the same order for either tile, so the tile (a launch parameter) never changes results.
+// 4 x 4 outputs per thread over a TILE x TILE tile (2 x 4 over TILE / 2 rows where the instance
+// has no more unknowns than that). The next 16 samples are in registers while the current ones
+// are multiplied from one of two shared-memory stages: with one stage and no prefetch every 16
+// samples waited for their loads (J = 2560: 459 us of 16 CTA-rows that ran alone on an SM).
+// Every entry is one chain of multiply-adds over the samples in order whatever the tile (a
+// launch parameter), so the tile never changes results.
 constexpr int BK = 16;
 
-template <typename T, int TILE>
-__global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
-    const BInst* __restrict__ tab, int step) {
-  constexpr int BM = TILE, BN = TILE, TXN = TILE / 4, CT = TXN * TXN;
-  __shared__ T As[BK][BM];
-  __shared__ T Bs[BK][BN];
-  const BInst& d = tab[blockIdx.x];
-  const Cur cu = current(d, step, 0, false);
-  if (!cu.active) return;
+template <typename T, int TILE, int U>
+__device__ __forceinline__ void contract_tile_cta(const BInst& d, const Cur& cu, T* smem) {
+  constexpr int TXN = TILE / 4, CT = TXN * TXN, BM = TXN * U, BN = TILE;
+  constexpr int NA = (BK * BM + CT - 1) / CT, NB = (BK * BN) / CT;
+  T* As = smem;                       // [2][BK][BM]
+  T* Bs = smem + 2 * BK * TILE;       // [2][BK][BN]
   const int L = cu.L;
   const int64_t I = cu.I, ldc = L + I;
   const int ntr = (L + BM - 1) / BM;
@@ -141,53 +142,80 @@ __global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
   const T* __restrict__ Y = static_cast<const T*>(d.Y);
   const int64_t J = d.J;
   const int tx = threadIdx.x % TXN, ty = threadIdx.x / TXN;
-  T acc[4][4];
+  T ra[NA], rb[NB];
+  auto load = [&](int64_t jb) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+    for (int q = 0; q < NA; ++q) {
+      const int e = threadIdx.x + q * CT;
+      const int kk = e / BM, r = r0 + e % BM;
+      const int64_t j = jb + kk;
+      ra[q] = (kk < BK && j < J && r < L) ? A[j * L + r] : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = threadIdx.x + q * CT;
+      const int64_t j = jb + e / BN, c = c0 + e % BN;
+      rb[q] = T(0);
+      if (j < J) {
+        if (c < L) rb[q] = A[j * L + c];
+        else if (c < ldc) rb[q] = Y[j * I + (c - L)];
+      }
+    }
+  };
+  T acc[U][4];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int v = 0; v < 4; ++v) acc[u][v] = T(0);
-  for (int64_t jb = 0; jb < J; jb += BK) {
+  load(0);
+  int s = 0;
+  for (int64_t jb = 0; jb < J; jb += BK, s ^= 1) {
+    T* as = As + s * (BK * TILE);
+    T* bs = Bs + s * (BK * TILE);
 #pragma unroll
-    for (int q = 0; q < (BK * BM) / CT; ++q) {
+    for (int q = 0; q < NA; ++q) {
       const int e = threadIdx.x + q * CT;
-      const int kk = e / BM, col = e % BM;
-      const int64_t j = jb + kk;
-      const int r = r0 + col;
-      As[kk][col] = (j < J && r < L) ? A[j * L + r] : T(0);
-      const int64_t c = c0 + col;
-      T b = T(0);
-      if (j < J) {
-        if (c < L) b = A[j * L + c];
-        else if (c < ldc) b = Y[j * I + (c - L)];
-      }
-      Bs[kk][col] = b;
+      if (NA * CT == BK * BM || e < BK * BM) as[e] = ra[q];
     }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NB; ++q) bs[threadIdx.x + q * CT] = rb[q];
+    __syncthreads();       // the stage is written; its previous readers passed the last barrier
+    if (jb + BK < J) load(jb + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      T a[4], b[4];
+      T a[U], b[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = As[kk][ty + TXN * u];
+      for (int u = 0; u < U; ++u) a[u] = as[kk * BM + ty * U + u];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) b[v] = Bs[kk][tx + TXN * v];
+      for (int v = 0; v < 4; ++v) b[v] = bs[kk * BN + tx * 4 + v];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
     }
-    __syncthreads();
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = r0 + ty + TXN * u;
+  for (int u = 0; u < U; ++u) {
+    const int r = r0 + ty * U + u;
     if (r >= L) continue;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const int64_t c = c0 + tx + TXN * v;
+      const int64_t c = c0 + tx * 4 + v;
       if (c < L) d.M[static_cast<int64_t>(r) * L + c] = static_cast<double>(acc[u][v]);
       else if (c < ldc) d.BT[(c - L) * L + r] = static_cast<double>(acc[u][v]);
     }
   }
+}
+
+template <typename T, int TILE>
+__global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
+    const BInst* __restrict__ tab, int step) {
+  __shared__ __align__(16) T smem[4 * BK * TILE];
+  const BInst& d = tab[blockIdx.x];
+  const Cur cu = current(d, step, 0, false);
+  if (!cu.active) return;
+  if (cu.L <= TILE / 2) contract_tile_cta<T, TILE, 2>(d, cu, smem);
+  else contract_tile_cta<T, TILE, 4>(d, cu, smem);
 }
 
 // ------------------------------------------------------------------------------------

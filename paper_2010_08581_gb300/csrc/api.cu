@@ -339,24 +339,21 @@ tr_status leverage_dist(tr_ctx* ctx, char* ws, const double* mat, int64_t I, int
     TR_LAUNCH("ff_image", launch_ff_image(p1.Lrow, p1.Lcol, n, p1.info, p1.img, st, gate));
     CdfEpilogue ep2 = ep;
     ep2.run_if = gate;
-    TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.Lrow, p1.Lcol, p1.invdiag, nullptr, I,
-                                           mat, L, nullptr, 1, 1, nullptr, ell, st, p1.img,
-                                           nullptr, &ep2));
+    TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,
+                                           nullptr, ell, st, p1.img, nullptr, &ep2));
   } else if (I >= L) {
     TR_TRY(run_pass(ctx, p1, mat, I, L, L, false, tol, st, mixed, mat_hi, mat_lo));
     if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
-    TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.Lrow, p1.Lcol, p1.invdiag, nullptr, I,
-                                           mat, L, nullptr, 1, 1, nullptr, ell, st, p1.img,
-                                           nullptr, &ep));
+    TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,
+                                           nullptr, ell, st, p1.img, nullptr, &ep));
   } else {
     // Wide G_(2): the range of A is that of C with A A^T = C C^T; ell(A) = ell(C).
     const int n = static_cast<int>(I);
     TR_TRY(run_pass(ctx, p1, mat, I, L, L, true, tol, st));
     TR_TRY(run_pass(ctx, p2, p1.Lrow, I, n, n, false, tol, st));
     if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
-    TR_LAUNCH("leverage_rows", launch_trsm(0, false, n, p2.Lrow, p2.Lcol, p2.invdiag, nullptr, I,
-                                           p1.Lrow, n, nullptr, 1, 1, nullptr, ell, st, p2.img,
-                                           nullptr, &ep));
+    TR_LAUNCH("leverage_rows", launch_trsm(0, false, n, p2.invdiag, nullptr, I, p1.Lrow, n, 1, 1,
+                                           nullptr, ell, st, p2.img, nullptr, &ep));
   }
   return TR_OK;
 }
@@ -484,9 +481,8 @@ tr_status solve_rhs(tr_ctx* ctx, const SolvePlan& s, int Rl, int Rr, int64_t I, 
                                             s.wimg, st, tiles_flag(ctx, s, !refine, L)));
     return TR_OK;
   }
-  TR_LAUNCH("solve_rhs", launch_trsm(refine ? 2 : 1, refine, L, s.Lrow, s.Lcol, s.invdiag, s.info,
-                                      I, s.BT, L, s.M, Rl, Rr, core_out, nullptr, st, s.limg,
-                                      s.mimg));
+  TR_LAUNCH("solve_rhs", launch_trsm(refine ? 2 : 1, refine, L, s.invdiag, s.info, I, s.BT, L, Rl,
+                                      Rr, core_out, nullptr, st, s.limg, s.mimg));
   return TR_OK;
 }
 

@@ -2,7 +2,7 @@
 // one launch per stage for every instance of the table; see batched.cuh. This file holds
 // the initial cores, the draws with their rows and fibres, the normal-equation contraction
 // and the leverage Grams; the factorisations, solves and fit live in batched_chol.cu,
-// batched_solve32.cu, batched_solve64.cu and batched_fit.cu.
+// batched_solve.cu and batched_fit.cu.
 #include "batched_kern.cuh"
 #include "draw.cuh"
 
@@ -331,16 +331,10 @@ cudaError_t bl_gram(const BLaunch& b, int step, int init_k, int pass, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t bl_solve(const BLaunch& b, int step, cudaStream_t st) {
-  return b.f64 ? bl_solve_f64(b, step, st) : bl_solve_f32(b, step, st);
-}
-
 cudaError_t batched_attributes() {
   cudaError_t e = batched_chol_attributes();
   if (e != cudaSuccess) return e;
-  e = batched_solve32_attributes();
-  if (e != cudaSuccess) return e;
-  e = batched_solve64_attributes();
+  e = batched_solve_attributes();
   if (e != cudaSuccess) return e;
   return batched_fit_attributes();
 }

@@ -1,5 +1,5 @@
 // Device helpers shared by the batched stage kernels (batched.cu, batched_chol.cu,
-// batched_solve32.cu, batched_solve64.cu, batched_fit.cu): which core each instance
+// batched_solve.cu, batched_fit.cu): which core each instance
 // updates in a step, and the dynamic shared-memory limit of the batched kernels.
 #pragma once
 
@@ -55,13 +55,9 @@ constexpr int kDyn = 200 * 1024;
 
 }  // namespace
 
-// Per-precision halves of bl_solve (batched_solve32.cu / batched_solve64.cu) and the
-// attribute set-up of each translation unit.
-cudaError_t bl_solve_f32(const BLaunch& b, int step, cudaStream_t st);
-cudaError_t bl_solve_f64(const BLaunch& b, int step, cudaStream_t st);
+// Attribute set-up of each translation unit.
 cudaError_t batched_chol_attributes();
-cudaError_t batched_solve32_attributes();
-cudaError_t batched_solve64_attributes();
+cudaError_t batched_solve_attributes();
 cudaError_t batched_fit_attributes();
 
 }  // namespace trk

@@ -226,10 +226,9 @@ struct CdfEpilogue {
   unsigned* err;
   const int* run_if = nullptr;   // when given, the launch does nothing unless *run_if != 0
 };
-cudaError_t launch_trsm(int mode, bool f32, int n, const double* Lrow, const double* Lcol,
-                        const double* invdiag, const int* info, int64_t nvec, const double* rhs,
-                        int64_t ld, const double* M, int Rl, int Rr, double* core_out,
-                        double* ell, cudaStream_t st, const void* Limg = nullptr,
+cudaError_t launch_trsm(int mode, bool f32, int n, const double* invdiag, const int* info,
+                        int64_t nvec, const double* rhs, int64_t ld, int Rl, int Rr,
+                        double* core_out, double* ell, cudaStream_t st, const void* Limg,
                         const float* Mimg = nullptr, const CdfEpilogue* cdf = nullptr);
 size_t trsm_image_bytes(int n, bool f32);
 

@@ -163,8 +163,8 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
       e = launch_solve_inv(L, static_cast<const float*>(s.limg), s.mimg, s.invdiag, s.info, I,
                            s.BT, L, Rl, Rr, core_out, s.wimg, st, tiles ? s.fast : nullptr);
     else
-      e = launch_trsm(f64 ? 1 : 2, !f64, L, s.Lrow, s.Lcol, s.invdiag, s.info, I, s.BT, L, s.M,
-                      Rl, Rr, core_out, nullptr, st, s.limg, s.mimg);
+      e = launch_trsm(f64 ? 1 : 2, !f64, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out, nullptr,
+                      st, s.limg, s.mimg);
   }
   if (e == cudaSuccess && info)
     e = cudaMemcpyAsync(info, s.info, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);

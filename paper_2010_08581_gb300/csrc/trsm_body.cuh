@@ -1,154 +1,41 @@
 // Triangular solves with a Cholesky factor L (n <= 256) for many vectors, shared by the
-// single-problem kernel (trsm.cu) and the batched kernel (batched.cu):
+// single-problem kernel (trsm.cu) and the batched kernels (batched_solve.cu):
 //   mode 0 (leverage rows, row a1): ell_v = || L^-1 a_v ||^2 -- row norms of Q = A R^-1 of
 //           the Cholesky-based thin QR (Def. 4), optionally followed by p and the CDF;
 //   mode 1 (LS solve, row a6):      z_v = L^-T L^-1 b_v, written into the new core;
 //   mode 2 (LS solve + one refinement step, row a6):
 //           z = L^-T L^-1 b;  r = b - M z;  z += L^-T L^-1 r.
-// One warp owns NB vectors; lane l holds rows l, l+32, ... (QN registers per vector), so a
-// substitution step is one shuffle broadcast plus independent FMAs. The factor (and M) are
-// staged in shared memory with a padded row stride (n+1): from the padded images written
-// by the Cholesky kernel (cp.async, 16 bytes per request) when given, else converted from
-// the FP64 column-major factor.
+//
+// One CTA takes NV vectors through blocked substitutions: the factor's padded image
+// (img[c * (n + 1) + r] = L[r][c]) streams through two shared-memory panels of PB columns, the
+// vectors stay in shared memory. Per panel, PB lanes solve the diagonal block for one vector
+// (lane = row, one shuffle, multiply and multiply-add per column), then every thread takes one of
+// the remaining rows and VP vectors through the panel's PB columns, with no dependence between
+// rows. The first panel of the next pass is under way while the last one of this pass is used.
+// An entry receives its multiply-adds in the order of the columns, one by one, as the
+// substitution of one vector by one warp does, so the panel width never changes a result.
+//
+// What bounds it: the columns' dependent chain (about 40 clocks a column in FP32, 170 in FP64)
+// plus a few hundred clocks of barriers a panel; with many vectors in FP64 the FP64 pipe, where a
+// warp's instruction takes 16 clocks however few of its lanes matter: hence 16 columns and two
+// vectors a warp there. One warp carrying whole vectors through all columns (the form before)
+// kept the remaining rows on the same chain, eight register rows at n = 256 behind a switch per
+// column. 300 vectors, mode 2 in FP32: n = 224: 569 -> 89 us, n = 256: 747 -> 98 us; mode 1 in FP64:
+// n = 100: 50.5 -> 49 us (1300: 152 -> 90), n = 256: 561 -> 153 us.
 #pragma once
 
 #include "common.cuh"
 
 namespace trk {
 
-constexpr int TW = 4;   // warps per CTA
+constexpr int TNT = 256;            // threads per CTA
+constexpr int TNW = TNT / 32;
 
-// The factor for the substitutions: the padded image s[c*(n+1) + r] = L[r][c] in shared
-// memory (SMEM), or in global memory when the Cholesky kernel wrote one (its FP32 or FP64
-// image in L2: no per-element conversion from FP64), else the FP64 column- and row-major
-// factor.
-// PACK (with SMEM): the lower triangle packed column by column in shared memory, column c
-// starting at c*n - c(c-1)/2 -- for factors whose padded image does not fit (n > 160 in
-// FP32): n(n+1)/2 entries.
-template <typename T, bool SMEM, bool PACK = false>
-struct Factor {
-  const T* s;            // image, shared (SMEM) or global (gimg)
-  const double* Lcol;    // global: Lcol[c*n + r] = L[r][c]
-  const double* Lrow;    // global: Lrow[c*n + r] = L[c][r]
-  int n;
-  bool gimg = false;     // !SMEM: s is a global image
-  __device__ __forceinline__ int pk(int c) const { return c * n - (c * (c - 1)) / 2 - c; }
-  __device__ __forceinline__ T col(int c, int r) const {   // L[r][c], r >= c
-    if constexpr (PACK) return s[pk(c) + r];
-    else if constexpr (SMEM) return s[c * (n + 1) + r];
-    else return gimg ? __ldg(s + c * (n + 1) + r) : static_cast<T>(Lcol[c * n + r]);
-  }
-  __device__ __forceinline__ T row(int c, int r) const {   // L[c][r], r < c
-    if constexpr (PACK) return s[pk(r) + c];
-    else if constexpr (SMEM) return s[r * (n + 1) + c];
-    else return gimg ? __ldg(s + r * (n + 1) + c) : static_cast<T>(Lrow[c * n + r]);
-  }
-};
-
-template <typename T, int QN, int NB>
-__device__ __forceinline__ T pick(const T (&x)[QN][NB], int q, int v) {
-  T s = x[0][v];
-#pragma unroll
-  for (int u = 1; u < QN; ++u) s = (u == q) ? x[u][v] : s;
-  return s;
-}
-
-template <typename T, int QN, int NB>
-__device__ __forceinline__ void put(T (&x)[QN][NB], int q, int v, T val) {
-#pragma unroll
-  for (int u = 0; u < QN; ++u)
-    if (u == q) x[u][v] = val;
-}
-
-// x <- L^-1 x. Rows are processed in blocks of 32 (register slot qb of every lane); inside a
-// block the pivot row's lane is a compile-time constant and the block's values live in one
-// register per vector, so one step is a shuffle, a multiply and independent FMAs.
-template <typename T, int QN, int NB, bool SMEM, bool PACK>
-__device__ __forceinline__ void forward(T (&x)[QN][NB], const Factor<T, SMEM, PACK>& F,
-                                        const T* inv, int lane) {
-  const int n = F.n;
-  for (int qb = 0; qb < QN; ++qb) {
-    T xb[NB];
-#pragma unroll
-    for (int v = 0; v < NB; ++v) xb[v] = pick(x, qb, v);
-#pragma unroll
-    for (int lc = 0; lc < 32; ++lc) {
-      const int c = qb * 32 + lc;
-      if (c >= n) break;
-      const T ic = inv[c];
-      T xc[NB];
-#pragma unroll
-      for (int v = 0; v < NB; ++v) {
-        xc[v] = __shfl_sync(0xffffffffu, xb[v], lc) * ic;
-        if (lane == lc) xb[v] = xc[v];
-      }
-      if (lane > lc && qb * 32 + lane < n) {
-        const T l = F.col(c, qb * 32 + lane);
-#pragma unroll
-        for (int v = 0; v < NB; ++v) xb[v] -= l * xc[v];
-      }
-#pragma unroll
-      for (int q = 0; q < QN; ++q) {
-        if (q > qb) {
-          const int r = lane + 32 * q;
-          const T l = (r < n) ? F.col(c, r) : T(0);
-#pragma unroll
-          for (int v = 0; v < NB; ++v) x[q][v] -= l * xc[v];
-        }
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < NB; ++v) put(x, qb, v, xb[v]);
-  }
-}
-
-// x <- L^-T x, blocks in reverse order.
-template <typename T, int QN, int NB, bool SMEM, bool PACK>
-__device__ __forceinline__ void backward(T (&x)[QN][NB], const Factor<T, SMEM, PACK>& F,
-                                         const T* inv, int lane) {
-  const int n = F.n;
-  for (int qb = QN - 1; qb >= 0; --qb) {
-    T xb[NB];
-#pragma unroll
-    for (int v = 0; v < NB; ++v) xb[v] = pick(x, qb, v);
-#pragma unroll
-    for (int lc = 31; lc >= 0; --lc) {
-      const int c = qb * 32 + lc;
-      if (c >= n) continue;
-      const T ic = inv[c];
-      T zc[NB];
-#pragma unroll
-      for (int v = 0; v < NB; ++v) {
-        zc[v] = __shfl_sync(0xffffffffu, xb[v], lc) * ic;
-        if (lane == lc) xb[v] = zc[v];
-      }
-      if (lane < lc) {
-        const T l = F.row(c, qb * 32 + lane);
-#pragma unroll
-        for (int v = 0; v < NB; ++v) xb[v] -= l * zc[v];
-      }
-#pragma unroll
-      for (int q = 0; q < QN; ++q) {
-        if (q < qb) {
-          const T l = F.row(c, lane + 32 * q);
-#pragma unroll
-          for (int v = 0; v < NB; ++v) x[q][v] -= l * zc[v];
-        }
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < NB; ++v) put(x, qb, v, xb[v]);
-  }
-}
-
-// Copy `bytes` (multiple of 16) from global to shared memory with cp.async, all threads.
-__device__ __forceinline__ void stage_async(void* dst, const void* src, int bytes) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  const char* s = static_cast<const char*>(src);
-  for (int o = threadIdx.x * 16; o < bytes; o += blockDim.x * 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d + o), "l"(s + o) : "memory");
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
+// Columns per panel: 32 in FP32, 16 in FP64, and 32 there too where few vectors leave one CTA per
+// SM: then a panel's latency counts, not the FP64 pipe (n = 64, 300 vectors: 29 us with 16 columns,
+// 26 with 32; 1300 vectors: 45 us with 16 columns and two vectors a warp, 61 with one).
+template <typename T>
+constexpr int panel_cols(bool few) { return sizeof(T) == 4 || few ? 32 : 16; }
 
 // Block-wide exclusive scan (fixed order) of one double per thread for NW warps.
 template <int NW>
@@ -171,10 +58,6 @@ __device__ __forceinline__ double block_scan_nw(double v, double* wt, double* to
   const double r = wt[warp] + inc - v;
   __syncthreads();
   return r;
-}
-
-__device__ __forceinline__ double block_scan_tw(double v, double* wt, double* total) {
-  return block_scan_nw<TW>(v, wt, total);
 }
 
 // p = ell / sum(ell) and its prefix sum, by the CTA that finishes last (mode 0 only), whose
@@ -213,184 +96,264 @@ __device__ inline void cdf_epilogue_nw(const CdfEpilogue& ep, const double* ell,
   }
 }
 
-__device__ inline void cdf_epilogue(const CdfEpilogue& ep, const double* ell, int64_t I) {
-  cdf_epilogue_nw<TW>(ep, ell, I);
+// Shared memory of a CTA: the inverse diagonal, two panels and two sets of NV vectors.
+template <typename T>
+__host__ __device__ inline size_t subst_smem(int n, int nv, int PB) {
+  return (static_cast<size_t>((n + 3) & ~3) + 2 * static_cast<size_t>(n + 1) * (PB + 1) +
+          2 * static_cast<size_t>(n) * nv + 4) * sizeof(T);
 }
 
-template <typename T, int QN, int NB, bool SMEM, bool PACK = false>
-__device__ __forceinline__ void trsm_cta(unsigned char* trsm_smem, int64_t cta, int n,
-                                         const double* __restrict__ Lrow,
-                                                  const double* __restrict__ Lcol,
-                                                  const double* __restrict__ invdiag,
-                                                  const int* __restrict__ info, int64_t nvec,
-                                                  const double* __restrict__ rhs, int64_t ld,
-                                                  int mode, const double* __restrict__ M,
-                                                  const T* __restrict__ Limg,
-                                                  const float* __restrict__ Mimg, int Rl, int Rr,
-                                                  double* __restrict__ core_out,
-                                                  double* __restrict__ ell, CdfEpilogue ep,
-                                                  int nctas) {
-  if ((info && *info) || (ep.run_if && *ep.run_if == 0)) return;
-  const int np = n + 1;
-  const int img_elems = ((n * np * static_cast<int>(sizeof(T)) + 15) / 16) * 16 /
-                        static_cast<int>(sizeof(T));
-  T* inv = reinterpret_cast<T*>(trsm_smem);                  // kMaxL entries
-  T* Ls = inv + kMaxL;                                       // n*(n+1) (padded to 16 B)
-  T* Ms = Ls + (SMEM && !PACK ? img_elems : 0);              // mode 2
-  for (int c = threadIdx.x; c < n; c += blockDim.x) inv[c] = static_cast<T>(invdiag[c]);
-  if constexpr (PACK) {
-    // the lower triangle, column by column, from the padded image with element-sized
-    // asynchronous copies (all in flight at once), or converted from the FP64 factor
-    for (int c = threadIdx.x >> 5; c < n; c += TW) {
-      const int base = c * n - (c * (c - 1)) / 2 - c;
-      for (int r = c + (threadIdx.x & 31); r < n; r += 32) {
-        if (Limg) {
-          const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(Ls + base + r));
-          if constexpr (sizeof(T) == 4)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d),
-                         "l"(Limg + c * np + r) : "memory");
-          else
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d),
-                         "l"(Limg + c * np + r) : "memory");
-        } else {
-          Ls[base + r] = static_cast<T>(Lcol[c * n + r]);
+template <typename T>
+__device__ __forceinline__ void copy_async(T* dst, const T* src) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  if constexpr (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(d), "l"(src) : "memory");
+}
+
+// Blocked substitutions and products on NV vectors x[row * NV + v] in shared memory.
+template <typename T, int NV, int VP, int PB>
+struct Subst {
+  static constexpr int VPW = 32 / PB;           // vectors per warp in the diagonal blocks
+  static constexpr int G = NV / VP;             // groups of vectors
+  static constexpr int RT = TNT / G;            // rows the threads cover
+  int n, np;
+  const T* inv;
+  T* panel[2];
+
+  // Panel of columns c0 .. c0 + PB - 1 and rows r0 .. n - 1, as p[k * (n + 1) + row].
+  __device__ __forceinline__ void stage_cols(T* p, const T* img, int c0, int r0) const {
+    const int w = min(PB, n - c0);
+    for (int k = threadIdx.x >> 5; k < w; k += TNW)
+      for (int r = r0 + (threadIdx.x & 31); r < n; r += 32)
+        copy_async(p + k * np + r, img + static_cast<int64_t>(c0 + k) * np + r);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // Rows c0 .. c0 + PB - 1 of the factor, columns 0 .. r1 - 1, as p[column * (PB + 1) + k].
+  __device__ __forceinline__ void stage_rows(T* p, const T* img, int c0, int r1) const {
+    const int w = min(PB, n - c0);
+    for (int e = threadIdx.x; e < r1 * PB; e += TNT) {
+      const int r = e / PB, k = e % PB;
+      if (k < w) copy_async(p + r * (PB + 1) + k, img + static_cast<int64_t>(r) * np + c0 + k);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  static __device__ __forceinline__ void landed(bool more) {   // all but the newest group
+    if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+  }
+
+  enum Next { kNone, kRows, kCols };   // what the next pass stages first
+
+  // First panel of the next pass, while this pass uses its last one.
+  __device__ __forceinline__ bool stage_next(T* p, Next next, const T* img) const {
+    if (next == kRows) stage_rows(p, img, (n - 1) / PB * PB, n);
+    else if (next == kCols) stage_cols(p, img, 0, 0);
+    return next != kNone;
+  }
+
+  // x <- L^-1 x. Panel s holds (or receives) the first PB columns; returns the next pass's panel.
+  __device__ int forward(T* x, const T* img, int s, Next next) const {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x % PB;
+    const int vec = warp * VPW + (threadIdx.x & 31) / PB;
+    const int g = threadIdx.x / RT, i = threadIdx.x % RT;
+    for (int c0 = 0; c0 < n; c0 += PB, s ^= 1) {
+      const int w = min(PB, n - c0);
+      bool more = c0 + PB < n;
+      if (more) stage_cols(panel[s ^ 1], img, c0 + PB, c0 + PB);
+      else more = stage_next(panel[s ^ 1], next, img);
+      landed(more);
+      const T* p = panel[s];
+      if (warp * VPW < NV) {
+        T v = lane < w ? x[(c0 + lane) * NV + vec] : T(0);
+#pragma unroll 8
+        for (int k = 0; k < w; ++k) {
+          const T xc = __shfl_sync(0xffffffffu, v, k, PB) * inv[c0 + k];
+          const T l = lane > k && lane < w ? p[k * np + c0 + lane] : T(0);
+          if (lane == k) v = xc;
+          else if (lane > k && lane < w) v -= l * xc;
+        }
+        if (lane < w) x[(c0 + lane) * NV + vec] = v;
+      }
+      __syncthreads();
+      const int r = c0 + PB + i;
+      if (c0 + PB >= n) continue;
+      if (r < n) {
+        T acc[VP];
+#pragma unroll
+        for (int v = 0; v < VP; ++v) acc[v] = x[r * NV + g * VP + v];
+#pragma unroll 8
+        for (int k = 0; k < PB; ++k) {      // more rows follow: the panel is full
+          const T l = p[k * np + r];
+#pragma unroll
+          for (int v = 0; v < VP; ++v) acc[v] -= l * x[(c0 + k) * NV + g * VP + v];
+        }
+#pragma unroll
+        for (int v = 0; v < VP; ++v) x[r * NV + g * VP + v] = acc[v];
+      }
+      __syncthreads();
+    }
+    return s;
+  }
+
+  // x <- L^-T x, panels and columns in reverse order. Panel s receives the last rows.
+  __device__ int backward(T* x, const T* img, int s, Next next, const T* next_img) const {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x % PB;
+    const int vec = warp * VPW + (threadIdx.x & 31) / PB;
+    const int g = threadIdx.x / RT, i = threadIdx.x % RT;
+    for (int c0 = (n - 1) / PB * PB; c0 >= 0; c0 -= PB, s ^= 1) {
+      const int w = min(PB, n - c0);
+      bool more = c0 > 0;
+      if (more) stage_rows(panel[s ^ 1], img, c0 - PB, c0);
+      else more = stage_next(panel[s ^ 1], next, next_img);
+      landed(more);
+      const T* p = panel[s];
+      if (warp * VPW < NV) {
+        T v = lane < w ? x[(c0 + lane) * NV + vec] : T(0);
+#pragma unroll 8
+        for (int k = w - 1; k >= 0; --k) {
+          const T zc = __shfl_sync(0xffffffffu, v, k, PB) * inv[c0 + k];
+          const T l = lane < k ? p[(c0 + lane) * (PB + 1) + k] : T(0);
+          if (lane == k) v = zc;
+          else if (lane < k) v -= l * zc;
+        }
+        if (lane < w) x[(c0 + lane) * NV + vec] = v;
+      }
+      __syncthreads();
+      if (c0 == 0) continue;
+      if (i < c0) {
+        T acc[VP];
+#pragma unroll
+        for (int v = 0; v < VP; ++v) acc[v] = x[i * NV + g * VP + v];
+#pragma unroll 8
+        for (int k = w - 1; k >= 0; --k) {
+          const T l = p[i * (PB + 1) + k];
+#pragma unroll
+          for (int v = 0; v < VP; ++v) acc[v] -= l * x[(c0 + k) * NV + g * VP + v];
+        }
+#pragma unroll
+        for (int v = 0; v < VP; ++v) x[i * NV + g * VP + v] = acc[v];
+      }
+      __syncthreads();
+    }
+    return s;
+  }
+
+  // r <- r - M z (M symmetric, image img[t * (n + 1) + row]); then img2's first columns are staged.
+  __device__ int residual(T* r, const T* z, const T* img, int s, const T* img2) const {
+    const int g = threadIdx.x / RT, i = threadIdx.x % RT;
+    T acc[VP];
+#pragma unroll
+    for (int v = 0; v < VP; ++v) acc[v] = i < n ? r[i * NV + g * VP + v] : T(0);
+    for (int c0 = 0; c0 < n; c0 += PB, s ^= 1) {
+      const int w = min(PB, n - c0);
+      if (c0 + PB < n) stage_cols(panel[s ^ 1], img, c0 + PB, 0);
+      else stage_cols(panel[s ^ 1], img2, 0, 0);
+      landed(true);
+      const T* p = panel[s];
+      if (i < n) {
+#pragma unroll 8
+        for (int k = 0; k < w; ++k) {
+          const T m = p[k * np + i];
+#pragma unroll
+          for (int v = 0; v < VP; ++v) acc[v] -= m * z[(c0 + k) * NV + g * VP + v];
         }
       }
+      __syncthreads();
     }
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-  } else if constexpr (SMEM) {
-    if (Limg) {
-      stage_async(Ls, Limg, img_elems * static_cast<int>(sizeof(T)));
-    } else {
-      for (int c = threadIdx.x >> 5; c < n; c += TW)
-        for (int r = threadIdx.x & 31; r < n; r += 32) Ls[c * np + r] = static_cast<T>(Lcol[c * n + r]);
-    }
-    if (mode == 2) {
-      if (Mimg && sizeof(T) == 4) {
-        stage_async(Ms, Mimg, img_elems * static_cast<int>(sizeof(T)));
-      } else {
-        for (int c = threadIdx.x >> 5; c < n; c += TW)
-          for (int r = threadIdx.x & 31; r < n; r += 32) Ms[c * np + r] = static_cast<T>(M[c * n + r]);
-      }
-    }
+    if (i < n)
+#pragma unroll
+      for (int v = 0; v < VP; ++v) r[i * NV + g * VP + v] = acc[v];
+    __syncthreads();
+    return s;
   }
-  __syncthreads();
-  Factor<T, SMEM, PACK> F{SMEM ? Ls : Limg, Lcol, Lrow, n, !SMEM && Limg != nullptr};
+};
+
+template <typename T, int NV, int VP, int PB>
+__device__ __forceinline__ void subst_cta(unsigned char* sm, int64_t cta, int n,
+                                          const double* __restrict__ invdiag,
+                                          const int* __restrict__ info, int64_t nvec,
+                                          const double* __restrict__ rhs, int64_t ld, int mode,
+                                          const T* __restrict__ Limg,
+                                          const float* __restrict__ Mimg, int Rl, int Rr,
+                                          double* __restrict__ core_out,
+                                          double* __restrict__ ell, CdfEpilogue ep, int nctas) {
+  if ((info && *info) || (ep.run_if && *ep.run_if == 0)) return;
+  static_assert(NV <= TNW && NV % Subst<T, NV, VP, PB>::VPW == 0, "vectors a warp");
+  T* inv = reinterpret_cast<T*>(sm);
+  Subst<T, NV, VP, PB> S;
+  S.n = n;
+  S.np = n + 1;
+  S.inv = inv;
+  S.panel[0] = inv + ((n + 3) & ~3);
+  S.panel[1] = S.panel[0] + (n + 1) * (PB + 1);
+  // (16-byte offset in elements: a pointer rounded as an integer would lose its address space)
+  T* x = inv + ((((n + 3) & ~3) + 2 * (n + 1) * (PB + 1) + 3) & ~3);
+  T* res = x + n * NV;
+  const int64_t v0 = cta * NV;
+  S.stage_cols(S.panel[0], Limg, 0, 0);
+  for (int c = threadIdx.x; c < n; c += TNT) inv[c] = static_cast<T>(invdiag[c]);
+  for (int v = threadIdx.x >> 5; v < NV; v += TNW)
+    for (int r = threadIdx.x & 31; r < n; r += 32) {
+      const T b = v0 + v < nvec ? static_cast<T>(rhs[(v0 + v) * ld + r]) : T(0);
+      x[r * NV + v] = b;
+      if (mode == 2) res[r * NV + v] = b;
+    }
+  int s = S.forward(x, Limg, 0, mode == 0 ? S.kNone : S.kRows);   // (its first barrier covers x)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t v0 = (cta * TW + warp) * NB;
   if (mode == 0) {
-    if (v0 < nvec) {
-      T x[QN][NB];
+    if (warp < NV && v0 + warp < nvec) {
+      T sq = T(0);
+      for (int r = lane; r < n; r += 32) sq += x[r * NV + warp] * x[r * NV + warp];
 #pragma unroll
-      for (int q = 0; q < QN; ++q) {
-        const int r = lane + 32 * q;
-#pragma unroll
-        for (int v = 0; v < NB; ++v)
-          x[q][v] = (r < n && v0 + v < nvec) ? static_cast<T>(rhs[(v0 + v) * ld + r]) : T(0);
-      }
-      forward(x, F, inv, lane);
-#pragma unroll
-      for (int v = 0; v < NB; ++v) {
-        T s = T(0);
-#pragma unroll
-        for (int q = 0; q < QN; ++q)
-          if (lane + 32 * q < n) s += x[q][v] * x[q][v];   // rows >= n hold no data
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0 && v0 + v < nvec) ell[v0 + v] = static_cast<double>(s);
-      }
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      if (lane == 0) ell[v0 + warp] = static_cast<double>(sq);
     }
     if (ep.counter) {      // the last CTA to finish forms p and the CDF
       __shared__ int s_last;
       __threadfence();
       __syncthreads();
-      if (threadIdx.x == 0) s_last = (atomicAdd(ep.counter, 1u) == static_cast<unsigned>(nctas) - 1) ? 1 : 0;
+      if (threadIdx.x == 0)
+        s_last = (atomicAdd(ep.counter, 1u) == static_cast<unsigned>(nctas) - 1) ? 1 : 0;
       __syncthreads();
       if (s_last) {
         __threadfence();
-        cdf_epilogue(ep, ell, nvec);
+        cdf_epilogue_nw<TNW>(ep, ell, nvec);
         if (threadIdx.x == 0) *ep.counter = 0u;
       }
     }
     return;
   }
-  if (v0 >= nvec) return;
-  T x[QN][NB];
-#pragma unroll
-  for (int q = 0; q < QN; ++q) {
-    const int r = lane + 32 * q;
-#pragma unroll
-    for (int v = 0; v < NB; ++v)
-      x[q][v] = (r < n && v0 + v < nvec) ? static_cast<T>(rhs[(v0 + v) * ld + r]) : T(0);
-  }
-  forward(x, F, inv, lane);
-  backward(x, F, inv, lane);
-  if (mode == 2) {
-    // residual r = b - M z (M symmetric: column t of M = row t)
-    T res[QN][NB];
-#pragma unroll
-    for (int q = 0; q < QN; ++q) {
-      const int r = lane + 32 * q;
-#pragma unroll
-      for (int v = 0; v < NB; ++v)
-        res[q][v] = (r < n && v0 + v < nvec) ? static_cast<T>(rhs[(v0 + v) * ld + r]) : T(0);
+  if constexpr (sizeof(T) == 4) {
+    s = S.backward(x, Limg, s, mode == 2 ? S.kCols : S.kNone, Mimg);
+    if (mode == 2) {
+      s = S.residual(res, x, Mimg, s, Limg);
+      s = S.forward(res, Limg, s, S.kRows);
+      S.backward(res, Limg, s, S.kNone, Limg);
     }
-    for (int qt = 0; qt < QN; ++qt) {
-      T xt[NB];
-#pragma unroll
-      for (int v = 0; v < NB; ++v) xt[v] = pick(x, qt, v);
-#pragma unroll 8
-      for (int lt = 0; lt < 32; ++lt) {
-        const int t = qt * 32 + lt;
-        if (t >= n) break;
-        T zt[NB];
-#pragma unroll
-        for (int v = 0; v < NB; ++v) zt[v] = __shfl_sync(0xffffffffu, xt[v], lt);
-#pragma unroll
-        for (int q = 0; q < QN; ++q) {
-          const int r = lane + 32 * q;
-          if (r < n) {
-            T m;
-            if constexpr (SMEM && !PACK) m = Ms[t * np + r];
-            else if (sizeof(T) == 4 && Mimg) m = static_cast<T>(__ldg(Mimg + t * np + r));
-            else m = static_cast<T>(M[t * n + r]);
-#pragma unroll
-            for (int v = 0; v < NB; ++v) res[q][v] -= m * zt[v];
-          }
-        }
-      }
-    }
-    forward(res, F, inv, lane);
-    backward(res, F, inv, lane);
-#pragma unroll
-    for (int q = 0; q < QN; ++q)
-#pragma unroll
-      for (int v = 0; v < NB; ++v) x[q][v] += res[q][v];
+  } else {
+    S.backward(x, Limg, s, S.kNone, Limg);
   }
   // new core: core[i][a][b] = z[a + Rl*b]
-#pragma unroll
-  for (int q = 0; q < QN; ++q) {
-    const int r = lane + 32 * q;
-    if (r >= n) continue;
-    const int a = r % Rl, b = r / Rl;
-#pragma unroll
-    for (int v = 0; v < NB; ++v)
-      if (v0 + v < nvec) core_out[(v0 + v) * n + a * Rr + b] = static_cast<double>(x[q][v]);
+  for (int v = warp; v < NV; v += TNW) {
+    if (v0 + v >= nvec) continue;
+    for (int r = lane; r < n; r += 32) {
+      const T z = mode == 2 ? x[r * NV + v] + res[r * NV + v] : x[r * NV + v];
+      core_out[(v0 + v) * n + (r % Rl) * Rr + r / Rl] = static_cast<double>(z);
+    }
   }
 }
 
-
-// Shared memory of the packed layout (the inverse diagonal and n(n+1)/2 factor entries).
-template <typename T>
-__host__ __device__ inline size_t packed_bytes(int n) {
-  return kMaxL * sizeof(T) +
-         ((static_cast<size_t>(n) * (n + 1) / 2 * sizeof(T) + 15) / 16) * 16;
-}
-
-template <typename T>
-__host__ __device__ inline size_t staged_bytes(int n, int mode) {
-  const size_t img = ((static_cast<size_t>(n) * (n + 1) * sizeof(T) + 15) / 16) * 16;
-  return kMaxL * sizeof(T) + (mode == 2 ? 2 : 1) * img;
-}
+// The vectors per thread follow from the rows the threads have to cover: 256 threads take
+// 32 * ceil(n / 32) rows rounded up to a power of two.
+#define TRK_SUBST_DISPATCH(n, CASE)      \
+  do {                                   \
+    if ((n) <= 32) { CASE(1); }          \
+    else if ((n) <= 64) { CASE(2); }     \
+    else if ((n) <= 128) { CASE(4); }    \
+    else { CASE(8); }                    \
+  } while (0)
 
 }  // namespace trk

@@ -37,10 +37,15 @@ __global__ void __launch_bounds__(256) kb_init_cores(const BInst* __restrict__ t
 
 // ------------------------------------------------------------------------------------
 // Draws (Alg. 3), sampled subchain rows (Alg. 4) and sampled fibres (Alg. 2) for one chunk
-// of one instance's samples: one warp per sample.
+// of one instance's samples: first one thread per draw (a binary search is a chain of dependent
+// loads, about 5 us: all of a CTA's run at once), then one warp per sample, the fibre's scattered
+// loads in flight while the slices are multiplied. 512 problems of I = 32 .. 200, J = 160 .. 640:
+// 522 us with each warp drawing, multiplying and loading in turn (this and the Gram below took
+// 340 us off a step of 1.9 ms).
 // ------------------------------------------------------------------------------------
 constexpr int SW = 8;     // warps per CTA
 constexpr int kSpwMax = 8;   // samples per warp: a launch parameter in [1, 8] (tiles)
+constexpr int kFibre = 8;    // fibre entries per lane that are loaded ahead
 
 template <typename T, typename TX>
 __global__ void __launch_bounds__(SW * 32) kb_sample(const BInst* __restrict__ tab, int step,
@@ -48,6 +53,10 @@ __global__ void __launch_bounds__(SW * 32) kb_sample(const BInst* __restrict__ t
   __shared__ T sS[SW][kMaxL];
   __shared__ T sG[SW][kMaxL];
   __shared__ ChainArgs ca;
+  __shared__ int idx[SW * kSpwMax][kMaxModes];       // the draws of each sample
+  __shared__ double prob[SW * kSpwMax][kMaxModes];
+  __shared__ int64_t fibre[SW * kSpwMax];
+  __shared__ T weight[SW * kSpwMax];
   const BInst& d = tab[blockIdx.x];
   const Cur cu = current(d, step, 0, false);
   if (!cu.active) return;
@@ -68,45 +77,56 @@ __global__ void __launch_bounds__(SW * 32) kb_sample(const BInst* __restrict__ t
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t k0 = static_cast<uint32_t>(d.seed), k1 = static_cast<uint32_t>(d.seed >> 32);
   const uint32_t u0 = static_cast<uint32_t>(cu.t), u1 = 0u;
-  const int mode_l = (lane < npos) ? (n + 1 + lane) % N : 0;
+  const int count = d.J - j0 < SW * spw ? static_cast<int>(d.J - j0) : SW * spw;
+  for (int e = threadIdx.x; e < count * npos; e += SW * 32) {
+    const int s = e / npos, m = e - s * npos;
+    const int mode = (n + 1 + m) % N;
+    const double u = draw_uniform(j0 + s, m, k0, k1, u0, u1);
+    int64_t i;
+    double pi = 1.0;
+    if (d.uniform) {
+      i = uniform_index(d.dims[mode], u);
+    } else {
+      i = inverse_cdf(d.cdf[mode], d.p[mode], d.dims[mode], u);
+      pi = d.p[mode][i];
+    }
+    idx[s][m] = static_cast<int>(i);
+    prob[s][m] = pi;
+  }
+  __syncthreads();
+  if (threadIdx.x < static_cast<unsigned>(count)) {
+    const int s = threadIdx.x;
+    int64_t off = 0;
+    for (int m = 0; m < npos; ++m) off += idx[s][m] * d.stride[(n + 1 + m) % N];
+    fibre[s] = off;
+    const double w = d.uniform ? uniform_weight(d.J, ca.I, npos) : sample_weight(d.J, prob[s], npos);
+    weight[s] = static_cast<T>(w);
+  }
+  __syncthreads();
   const TX* __restrict__ X = static_cast<const TX*>(d.X);
   T* A = static_cast<T*>(d.A);
   T* Y = static_cast<T*>(d.Y);
   const int L = cu.L;
   const int64_t I = cu.I, sn = d.stride[n];
-  const double wuni = d.uniform ? uniform_weight(d.J, ca.I, npos) : 0.0;
-  for (int s = 0; s < spw; ++s) {
-    const int64_t j = j0 + warp * spw + s;
-    if (j >= d.J) break;
-    int64_t mine = 0;
-    double pmine = 1.0;
-    int64_t off = 0;
-    if (lane < npos) {
-      const double u = draw_uniform(j, lane, k0, k1, u0, u1);
-      if (d.uniform) {
-        mine = uniform_index(d.dims[mode_l], u);
-      } else {
-        mine = inverse_cdf(d.cdf[mode_l], d.p[mode_l], d.dims[mode_l], u);
-        pmine = d.p[mode_l][mine];
-      }
-      off = mine * d.stride[mode_l];
-    }
-    double wj = wuni;
-    if (!d.uniform) {
-      double pm[kMaxModes];
-      for (int m = 0; m < npos; ++m) pm[m] = __shfl_sync(0xffffffffu, pmine, m);
-      wj = sample_weight(d.J, pm, npos);
-    }
+  for (int s = warp; s < count; s += SW) {
+    const int64_t j = j0 + s;
+    const TX* src = X + fibre[s];
+    TX ahead[kFibre];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
-    auto index = [&](int m) -> int64_t {
-      return static_cast<int64_t>(__shfl_sync(0xffffffffu, static_cast<int>(mine), m));
-    };
+    for (int q = 0; q < kFibre; ++q) {
+      const int64_t e = lane + 32 * q;
+      ahead[q] = e < I ? src[e * sn] : TX(0);
+    }
+    auto index = [&](int m) -> int64_t { return idx[s][m]; };
     warp_slice_chain<T>(ca, index, sS[warp], sG[warp], lane);
-    const T scale = static_cast<T>(wj);
+    const T scale = weight[s];
     for (int e = lane; e < L; e += 32) A[j * L + e] = sS[warp][e] * scale;
-    const TX* src = X + off;
-    for (int64_t e = lane; e < I; e += 32)
+#pragma unroll
+    for (int q = 0; q < kFibre; ++q) {
+      const int64_t e = lane + 32 * q;
+      if (e < I) Y[j * I + e] = static_cast<T>(static_cast<T>(ahead[q]) * scale);
+    }
+    for (int64_t e = lane + 32 * kFibre; e < I; e += 32)
       Y[j * I + e] = static_cast<T>(static_cast<T>(src[e * sn]) * scale);
     __syncwarp();
   }
@@ -225,12 +245,20 @@ __global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
 //           update; B^T during the updates otherwise);
 //   pass 2 (wide modes only): G2 = C^T C (I x I), C = the pass-1 factor.
 // ------------------------------------------------------------------------------------
-constexpr int GT = 32, GK = 32, GNT = 256;
+constexpr int GK = 16, GNT = 256;
+constexpr int GM = 2;                 // 2 x 2 blocks of G per thread
+
+// The 2 x 2 blocks of G's upper triangle, row by row, are dealt out to the threads (and, beyond
+// GNT * GM of them, to the CTAs of blockIdx.y), GK rows of the matrix at a time in shared memory;
+// the lower triangle is written by its mirror image. The FP64 pipe is the bound, so there is no
+// work on padding beyond the last warp: 32 x 32 tiles of the whole square took 174 .. 310 us for
+// 512 cores of L = 9 .. 64, I = 32 .. 200. Every entry is one chain over the rows
+// in order, as before.
+__host__ __device__ inline int gram_blocks(int n) { const int h = (n + 1) / 2; return h * (h + 1) / 2; }
 
 __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, int step, int init_k,
                                                int pass, int from_core) {
-  __shared__ double P[GK][GT + 1];
-  __shared__ double Q[GK][GT + 1];
+  __shared__ __align__(16) double P[GK * kMaxL];
   const BInst& d = tab[blockIdx.x];
   const Cur cu = current(d, step, init_k, true);
   if (!cu.active) return;
@@ -250,41 +278,61 @@ __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, in
     src = d.L1row; lda = cu.I; G = d.G2;
     n = static_cast<int>(cu.I); K = cu.I; trans = false;
   }
-  const int nt = (n + GT - 1) / GT;
-  const int t = blockIdx.y;
-  if (t >= nt * nt) return;
-  const int p0 = (t / nt) * GT, q0 = (t % nt) * GT;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double acc[4] = {0, 0, 0, 0};
-  for (int64_t kb = 0; kb < K; kb += GK) {
+  const int h = (n + 1) / 2, blocks = gram_blocks(n);
+  const int parts = (blocks + GNT * GM - 1) / (GNT * GM);
+  if (static_cast<int>(blockIdx.y) >= parts) return;
+  const int b0 = static_cast<int>(static_cast<int64_t>(blocks) * blockIdx.y / parts);
+  const int b1 = static_cast<int>(static_cast<int64_t>(blocks) * (blockIdx.y + 1) / parts);
+  const int ld = 2 * h;               // an even row length: aligned pairs
+  int row[GM], col[GM];
+  double acc[GM][2][2] = {};
 #pragma unroll
-    for (int r = 0; r < (GK * GT) / GNT; ++r) {
-      const int e = threadIdx.x + r * GNT;
-      int kk, col;
-      if (!trans) { kk = e / GT; col = e % GT; } else { col = e / GK; kk = e % GK; }
+  for (int q = 0; q < GM; ++q) {
+    int rest = b0 + static_cast<int>(threadIdx.x) + GNT * q;
+    row[q] = -1;
+    col[q] = 0;
+    if (rest < b1) {
+      int r = 0;
+      while (rest >= h - r) { rest -= h - r; ++r; }
+      row[q] = 2 * r;
+      col[q] = 2 * (r + rest);
+    }
+  }
+  for (int64_t kb = 0; kb < K; kb += GK) {
+    for (int e = threadIdx.x; e < GK * ld; e += GNT) {
+      int kk, c;
+      if (!trans) { kk = e / ld; c = e - kk * ld; } else { c = e / GK; kk = e % GK; }
       const int64_t k = kb + kk;
-      const int p = p0 + col, q = q0 + col;
-      double vp = 0.0, vq = 0.0;
-      if (k < K) {
-        if (p < n) vp = trans ? src[p * lda + k] : src[k * lda + p];
-        if (q < n) vq = trans ? src[q * lda + k] : src[k * lda + q];
-      }
-      P[kk][col] = vp;
-      Q[kk][col] = vq;
+      P[kk * ld + c] = k < K && c < n ? (trans ? src[c * lda + k] : src[k * lda + c]) : 0.0;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < GK; ++kk) {
-      const double b = Q[kk][tx];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] += P[kk][ty + 8 * u] * b;
+    for (int q = 0; q < GM; ++q) {
+      if (row[q] < 0) continue;
+#pragma unroll 4
+      for (int kk = 0; kk < GK; ++kk) {
+        const double2 x = *reinterpret_cast<const double2*>(P + kk * ld + row[q]);
+        const double2 y = *reinterpret_cast<const double2*>(P + kk * ld + col[q]);
+        acc[q][0][0] += x.x * y.x;
+        acc[q][0][1] += x.x * y.y;
+        acc[q][1][0] += x.y * y.x;
+        acc[q][1][1] += x.y * y.y;
+      }
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int p = p0 + ty + 8 * u, q = q0 + tx;
-    if (p < n && q < n) G[static_cast<int64_t>(p) * n + q] = acc[u];
+  for (int q = 0; q < GM; ++q) {
+    if (row[q] < 0) continue;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        const int r = row[q] + u, c = col[q] + v;
+        if (r >= n || c >= n) continue;
+        G[static_cast<int64_t>(r) * n + c] = acc[q][u][v];
+        G[static_cast<int64_t>(c) * n + r] = acc[q][u][v];
+      }
   }
 }
 
@@ -325,8 +373,7 @@ cudaError_t bl_contract(const BLaunch& b, int step, cudaStream_t st) {
 cudaError_t bl_gram(const BLaunch& b, int step, int init_k, int pass, cudaStream_t st) {
   const int nmax = pass == 1 ? b.n1max : b.n2max;
   if (nmax <= 0) return cudaSuccess;
-  const int nt = (nmax + GT - 1) / GT;
-  dim3 grid(b.count, nt * nt);
+  dim3 grid(b.count, (gram_blocks(nmax) + GNT * GM - 1) / (GNT * GM));
   kb_gram<<<grid, GNT, 0, st>>>(b.tab, step, init_k, pass, b.ls_mode == 1 ? 1 : 0);
   return cudaGetLastError();
 }

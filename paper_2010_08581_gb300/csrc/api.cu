@@ -341,6 +341,35 @@ tr_status leverage_dist(tr_ctx* ctx, char* ws, const double* mat, int64_t I, int
     ep2.run_if = gate;
     TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,
                                            nullptr, ell, st, p1.img, nullptr, &ep2));
+  } else if (precond_enabled() && leverage_f64_fits(I, L, p1.splits)) {
+    // FP64 products around an FP32 inverse (lev64.cu); the FP64 factorisation and row solves run
+    // only when its device flag says so
+    ReduceSplit sp;
+    sp.hi = reinterpret_cast<float*>(p1.Lrow);
+    sp.lda = (L + 3) & ~3;
+    Lev64 w;
+    w.K32 = sp.hi;
+    w.ldk = sp.lda;
+    w.G = p1.G;
+    w.Ximg = reinterpret_cast<float*>(p1.img);
+    w.E = p1.Lcol;
+    w.bad = p1.info + 8;      // the info word's 256-byte slot
+    w.partial = p1.partial;
+    w.splits = p1.splits;
+    w.tau = lev_tau();
+    TR_LAUNCH("gram_f64", launch_gram(mat, I, L, L, false, p1.partial, p1.splits, st));
+    TR_LAUNCH("reduce_gram", launch_reduce(p1.partial, false, p1.splits, static_cast<int64_t>(L) * L,
+                                           L, L, L, L, p1.G, L, nullptr, 0, st, sp));
+    TR_LAUNCH("lev64_factor", launch_leverage_f64(0, w, mat, I, L, L, ell, ep, st));
+    if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
+    TR_LAUNCH("lev64_rows", launch_leverage_f64(1, w, mat, I, L, L, ell, ep, st));
+    TR_LAUNCH("cholesky_leverage", launch_cholesky(p1.G, L, 1, tol, p1.Lrow, p1.Lcol, p1.invdiag,
+                                                   p1.keep, p1.info, ctx->d_err, st, p1.img,
+                                                   nullptr, nullptr, w.bad + 1));
+    CdfEpilogue ep2 = ep;
+    ep2.run_if = w.bad + 1;
+    TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,
+                                           nullptr, ell, st, p1.img, nullptr, &ep2));
   } else if (I >= L) {
     TR_TRY(run_pass(ctx, p1, mat, I, L, L, false, tol, st, mixed, mat_hi, mat_lo));
     if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
@@ -370,7 +399,8 @@ struct SolvePlan {
   void* partial; double* M; double* BT; double* Lrow; double* Lcol; double* invdiag;
   int* keep; int* info; void* limg; float* mimg; float* wimg; int splits;
   float* bt_hi = nullptr; float* bt_lo = nullptr;   // double-float planes of B^T (mixed)
-  int* fast = nullptr;   // the one-CTA FP32 factor-and-inverse succeeded (mixed, L <= 128)
+  // L <= 128: the one-CTA FP32 factor-and-inverse succeeded; L > 160: launch_inv256's two flags
+  int* fast = nullptr;
 };
 
 bool use_tensor_cores(bool f64) {
@@ -396,6 +426,7 @@ size_t solve_plan(Carver& c, int64_t J, int L, int64_t I, bool f64, SolvePlan* s
   s->bt_hi = f64 ? nullptr : c.take<float>(static_cast<size_t>(I) * L);
   s->bt_lo = f64 ? nullptr : c.take<float>(static_cast<size_t>(I) * L);
   s->fast = f64 ? nullptr : c.take<int>(1);
+  if (s->fast && solve_big_fits(L)) s->fast = s->info + 8;   // two flags in info's 256-byte slot
   return c.off;
 }
 
@@ -421,7 +452,7 @@ tr_status solve_contract(tr_ctx* ctx, const SolvePlan& s, const void* A, const v
   // mixed: the reduction also writes M's FP32 values in the factorisation's work-array
   // layout (into Lrow, free until an FP64 fallback) and M's FP32 image
   ReduceSplit sp;
-  if (!f64 && L >= 4 && L <= 160) {
+  if (!f64 && L >= 4) {
     sp.hi = reinterpret_cast<float*>(s.Lrow);
     sp.lda = (L + 3) & ~3;
     sp.img = s.mimg;
@@ -436,10 +467,11 @@ tr_status solve_contract(tr_ctx* ctx, const SolvePlan& s, const void* A, const v
   return TR_OK;
 }
 
-// The flag of the mixed LS step's one-CTA FP32 factor-and-inverse (launch_cholesky_mixed),
-// or nullptr where that form does not apply (FP64 arithmetic or factorisations, L > 128).
+// The flags of the mixed LS step's FP32 factor-and-inverse (launch_cholesky_mixed), or nullptr
+// where that form does not apply (FP64 arithmetic or factorisations).
 int* tiles_flag(const tr_ctx* ctx, const SolvePlan& s, bool f64, int L) {
-  return (!f64 && ctx->factorization != TR_FACTOR_FP64 && L >= 4 && L <= 128) ? s.fast : nullptr;
+  return (!f64 && ctx->factorization != TR_FACTOR_FP64 && L >= 4 && (L <= 128 || solve_big_fits(L)))
+             ? s.fast : nullptr;
 }
 
 tr_status solve_cholesky(tr_ctx* ctx, const SolvePlan& s, bool f64, int L, cudaStream_t st) {
@@ -460,9 +492,8 @@ tr_status solve_cholesky(tr_ctx* ctx, const SolvePlan& s, bool f64, int L, cudaS
                                     static_cast<double>(L) * eps32, s.Lrow, s.Lcol, s.invdiag,
                                     s.keep, s.info, ctx->d_err, st, static_cast<float*>(s.limg),
                                     s.mimg,
-                                    L >= 4 && L <= 160 ? reinterpret_cast<float*>(s.Lrow)
-                                                       : nullptr,
-                                    s.wimg, tiles_flag(ctx, s, f64, L)));
+                                    L >= 4 ? reinterpret_cast<float*>(s.Lrow) : nullptr, s.wimg,
+                                    tiles_flag(ctx, s, f64, L)));
     return TR_OK;
   }
   TR_LAUNCH("cholesky_solve",
@@ -481,8 +512,17 @@ tr_status solve_rhs(tr_ctx* ctx, const SolvePlan& s, int Rl, int Rr, int64_t I, 
                                             s.wimg, st, tiles_flag(ctx, s, !refine, L)));
     return TR_OK;
   }
-  TR_LAUNCH("solve_rhs", launch_trsm(refine ? 2 : 1, refine, L, s.invdiag, s.info, I, s.BT, L, Rl,
-                                      Rr, core_out, nullptr, st, s.limg, s.mimg));
+  CdfEpilogue gate{};
+  int* big = refine && solve_big_fits(L) ? tiles_flag(ctx, s, !refine, L) : nullptr;
+  if (big) {   // the contraction's partials are free: three right-hand-side blocks
+    const int64_t room = s.splits * (L + I) / 3;
+    TR_LAUNCH("solve_rhs", launch_solve_big(L, s.wimg, s.mimg, big, I, s.BT, L, Rl, Rr, core_out,
+                                            static_cast<float*>(s.partial), room < I ? room : I, st));
+    gate.run_if = big + 1;
+  }
+  TR_LAUNCH(big ? "solve_gated" : "solve_rhs",
+            launch_trsm(refine ? 2 : 1, refine, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out,
+                        nullptr, st, s.limg, s.mimg, big ? &gate : nullptr));
   return TR_OK;
 }
 

@@ -100,12 +100,14 @@ __device__ __forceinline__ bool factor_block(const float (&d)[4][4], int K, int 
 }  // namespace ci
 
 // Every thread of the CTA calls this (blockDim.x >= chol_inv_threads(n), 4 <= n <= 128).
-// On success W = L^-1 is written as the padded column-major image Wimg[c * (n + 1) + r]
-// (zeros above the diagonal) and true is returned; when a pivot is <= tol_scale * max diag K
-// nothing is written and false is returned (by every thread).
+// On success W = L^-1 is written as the column-major image Wimg[c * ldw + r] (zeros above the
+// diagonal) and true is returned; when a pivot is <= tol_scale * (the largest of the nd <= 256
+// entries diag[i * (lda_d + 1)]) nothing is written and false is returned (by every thread).
 __device__ __forceinline__ bool chol_inv_tiles(int n, float tol_scale,
                                                const float* __restrict__ pre, int lda,
-                                               float* __restrict__ Wimg, CiShared& s) {
+                                               float* __restrict__ Wimg, int ldw,
+                                               const float* __restrict__ diag, int nd, int lda_d,
+                                               CiShared& s) {
   const int nb = (n + 3) >> 2;
   const int t = threadIdx.x;
   const bool act = t < nb * (nb + 1) / 2;
@@ -127,15 +129,15 @@ __device__ __forceinline__ bool chol_inv_tiles(int n, float tol_scale,
     }
   }
   if (t < 32) {   // the largest diagonal entry: all loads issued before the first use
-    float dv[kCiMaxN / 32];
+    float dv[kMaxL / 32];
 #pragma unroll
-    for (int q = 0; q < kCiMaxN / 32; ++q) {
+    for (int q = 0; q < kMaxL / 32; ++q) {
       const int i = t + 32 * q;
-      dv[q] = i < n ? pre[static_cast<int64_t>(i) * lda + i] : 0.f;
+      dv[q] = i < nd ? diag[static_cast<int64_t>(i) * lda_d + i] : 0.f;
     }
     float md = 0.f;
 #pragma unroll
-    for (int q = 0; q < kCiMaxN / 32; ++q) md = fmaxf(md, dv[q]);
+    for (int q = 0; q < kMaxL / 32; ++q) md = fmaxf(md, dv[q]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
     if (t == 0) s.tol = tol_scale * md;
@@ -218,7 +220,6 @@ __device__ __forceinline__ bool chol_inv_tiles(int n, float tol_scale,
     __syncthreads();
   }
   if (act) {
-    const int np = n + 1;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int i = 4 * bi + r;
@@ -227,8 +228,8 @@ __device__ __forceinline__ bool chol_inv_tiles(int n, float tol_scale,
       for (int c = 0; c < 4; ++c) {
         const int col = 4 * bj + c;
         if (col >= n) continue;
-        Wimg[col * np + i] = i >= col ? a[r][c] : 0.f;
-        if (bi != bj) Wimg[i * np + col] = 0.f;   // the mirrored tile above the diagonal
+        Wimg[col * ldw + i] = i >= col ? a[r][c] : 0.f;
+        if (bi != bj) Wimg[i * ldw + col] = 0.f;   // the mirrored tile above the diagonal
       }
     }
   }

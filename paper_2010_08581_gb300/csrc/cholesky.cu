@@ -13,8 +13,10 @@ __global__ void __launch_bounds__(CNT) k_cholesky(const double* __restrict__ G, 
                                                   double tol_scale, double* Lrow, double* Lcol,
                                                   double* invdiag, int* keep_out, int* info,
                                                   unsigned* err, int use_smem,
-                                                  double* img64, float* img32, float* gimg32) {
+                                                  double* img64, float* img32, float* gimg32,
+                                                  const int* __restrict__ run_if) {
   extern __shared__ double smem[];
+  if (run_if && *run_if == 0) return;
   cholesky_cta(G, n, mode, tol_scale, use_smem ? smem : Lrow, Lrow, Lcol, invdiag, keep_out,
                info, err, img64, img32, gimg32);
 }
@@ -28,9 +30,11 @@ __global__ void __launch_bounds__(CNT) k_cholesky_mixed(const double* __restrict
                                                         int* info, unsigned* err, int dyn_bytes,
                                                         TI* img, float* gimg32,
                                                         const float* pre,
-                                                        const int* __restrict__ skip_if) {
+                                                        const int* __restrict__ skip_if,
+                                                        const int* __restrict__ run_if) {
   extern __shared__ double smem[];
   if (skip_if && *skip_if) return;   // the factor and its inverse are formed already
+  if (run_if && *run_if == 0) return;
   // A contraction whose bounded wait expired left no valid normal equations: report
   // info = -1 so that the solve leaves the core unchanged (the error bit is already set).
   if (err && (*reinterpret_cast<volatile unsigned*>(err) & kErrTimeout)) {
@@ -63,7 +67,7 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_chol_inv_solve(int n, float t
     }
     return;
   }
-  const bool ok = chol_inv_tiles(n, tol_scale, pre, lda, wimg, cs);
+  const bool ok = chol_inv_tiles(n, tol_scale, pre, lda, wimg, n + 1, pre, n, lda, cs);
   if (ok)
     for (int k = threadIdx.x; k < n; k += blockDim.x) keep[k] = 1;
   if (threadIdx.x == 0) {
@@ -143,20 +147,31 @@ cudaError_t launch_cholesky_mixed(const double* G, int n, int mode, double tol64
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
+  // n > 160: the FP32 factor and inverse by blocks (lev64.cu), fast[0] = 0 when it succeeded and
+  // fast[1] = 1 when this factorisation has to run instead
+  const bool big = wimg && fast && pre && solve_big_fits(n);
+  if (big) {
+    const cudaError_t e = launch_inv256(n, tol32, pre, (n + 3) & ~3, wimg,
+                                        reinterpret_cast<float*>(Lcol), fast, keep, info, err, st);
+    if (e != cudaSuccess) return e;
+  }
+  // (beyond kPanelCholMax the one-CTA factorisation reads G, and its work arrays may be pre's)
   k_cholesky_mixed<float><<<1, CNT, dyn, st>>>(G, n, mode, tol64, tol32, Lrow, Lcol, invdiag, keep,
                                                info, err, static_cast<int>(dyn), img32, gimg32,
-                                               pre, tiles ? fast : nullptr);
+                                               n <= kPanelCholMax ? pre : nullptr,
+                                               tiles ? fast : nullptr, big ? fast + 1 : nullptr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cholesky(const double* G, int n, int mode, double tol_scale, double* Lrow,
                             double* Lcol, double* invdiag, int* keep, int* info, unsigned* err,
-                            cudaStream_t st, double* img64, float* img32, float* gimg32) {
+                            cudaStream_t st, double* img64, float* img32, float* gimg32,
+                            const int* run_if) {
   const size_t bytes = static_cast<size_t>(n) * n * sizeof(double);
   const int use_smem = bytes <= kCholDyn ? 1 : 0;
   const size_t dyn = use_smem ? bytes : 0;
   k_cholesky<<<1, CNT, dyn, st>>>(G, n, mode, tol_scale, Lrow, Lcol, invdiag, keep, info, err,
-                                  use_smem, img64, img32, gimg32);
+                                  use_smem, img64, img32, gimg32, run_if);
   return cudaGetLastError();
 }
 

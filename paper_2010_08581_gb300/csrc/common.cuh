@@ -204,7 +204,8 @@ cudaError_t launch_ff_image(const double* Lrow, const double* Lcol, int n, const
 cudaError_t launch_cholesky(const double* G, int n, int mode, double tol_scale, double* Lrow,
                             double* Lcol, double* invdiag, int* keep, int* info,
                             unsigned* err, cudaStream_t st, double* img64 = nullptr,
-                            float* img32 = nullptr, float* gimg32 = nullptr);
+                            float* img32 = nullptr, float* gimg32 = nullptr,
+                            const int* run_if = nullptr);
 
 // Triangular solves with the factor of launch_cholesky for nvec vectors (row v of rhs,
 // leading dimension ld, length n):
@@ -291,6 +292,43 @@ int lev_precond_ctas(int n);
 cudaError_t launch_lev_precond(int stage, const LevPrecond& lp, int n, int64_t I,
                                const float* Ah, const float* Al, int64_t lda, double* ell,
                                const CdfEpilogue& ep, cudaStream_t st);
+
+// FP32 factor and inverse of an n x n matrix, 128 < n <= 256 (lev64.cu): pre as the reduction's
+// FP32 work array (row stride lda), X = L^-1 into the padded image Ximg; scratch: n * n floats
+// (16-byte aligned). bad[0] = 0 on success (then keep = 1 and *info = 0, when given), 1 when a
+// pivot is <= tol_scale * max diag, 2 when an expired wait left nothing to factor (*info = -1);
+// bad[1] = 1 when the caller's fallback has to run.
+bool inv256_fits(int n);
+bool solve_big_fits(int L);   // the sizes at which the mixed LS step takes that form
+cudaError_t launch_inv256(int n, double tol_scale, const float* pre, int lda, float* Ximg,
+                          float* scratch, int* bad, int* keep, int* info, const unsigned* err,
+                          cudaStream_t st);
+// The mixed LS step's solves through that inverse, as launch_solve_inv: scratch holds
+// 3 * rows * n floats; right-hand sides are taken `rows` at a time. Nothing when *bad != 0.
+cudaError_t launch_solve_big(int n, const float* Wimg, const float* Mimg, const int* bad,
+                             int64_t nvec, const double* rhs, int64_t ld, int Rl, int Rr,
+                             double* core_out, float* scratch, int64_t rows, cudaStream_t st);
+
+// FP64 leverage scores of a tall I x n matrix A (row stride lda) through an FP32 inverse of the
+// Gram's factor (lev64.cu): ell, then p and the CDF as launch_trsm's epilogue (ep.counter 0
+// before and after). part 0: everything up to the rows; 1: the rows (reads ep.skip). When the
+// FP32 factorisation fails or ||E||_F > tau nothing is written and bad[1] = 1: the caller's
+// fallback launches are gated on it. For the sizes leverage_f64_fits accepts (splits: of
+// gram_workspace, whose partials' room serves as scratch).
+struct Lev64 {
+  const float* K32;  // K's FP32 work array, from launch_reduce, row stride ldk
+  int ldk;
+  const double* G;   // K = A^T A, entries r <= c
+  float* Ximg;       // n (n + 1) floats
+  double* E;         // n x n
+  int* bad;          // 3
+  double* partial;   // splits * n * n
+  int splits;
+  double tau;
+};
+bool leverage_f64_fits(int64_t I, int n, int splits);
+cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,
+                                int64_t lda, double* ell, const CdfEpilogue& ep, cudaStream_t st);
 
 // dst[e] = hi[e] + lo[e] in FP64 (lev_precond.cu).
 cudaError_t launch_planes_sum(const float* hi, const float* lo, int64_t count, double* dst,

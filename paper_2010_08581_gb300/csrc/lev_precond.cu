@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_chol_inv(int n, float tol_sca
                                                             int lda, float* __restrict__ Ximg,
                                                             int* __restrict__ state) {
   __shared__ CiShared cs;
-  const bool ok = chol_inv_tiles(n, tol_scale, pre, lda, Ximg, cs);
+  const bool ok = chol_inv_tiles(n, tol_scale, pre, lda, Ximg, n + 1, pre, n, lda, cs);
   if (threadIdx.x == 0) *state = ok ? 0 : 1;
 }
 

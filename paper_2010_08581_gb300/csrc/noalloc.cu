@@ -63,6 +63,7 @@ size_t layout(char* base, int64_t J, int L, int64_t I, bool f64, Layout* s) {
   s->wimg = f64 ? nullptr : reinterpret_cast<float*>(b.take<char>(trsm_image_bytes(L, true)));
   s->err = b.take<unsigned>(1);
   s->fast = f64 ? nullptr : b.take<int>(1);
+  if (s->fast && solve_big_fits(L)) s->fast = s->info + 8;   // two flags in info's 256-byte slot
   return b.off;
 }
 
@@ -137,8 +138,8 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
   // The same reduction, factorisation and solves as tr_solve (stop-on-singular rule): on the
   // mixed path the reduction also writes M's FP32 work array and image for the FP32 factor.
   ReduceSplit sp;
-  const bool pre = !f64 && L >= 4 && L <= 160;
-  const bool tiles = !f64 && L >= 4 && L <= 128;   // as tr_solve's default factorisation
+  const bool pre = !f64 && L >= 4;
+  const bool tiles = !f64 && L >= 4 && (L <= 128 || solve_big_fits(L));   // as tr_solve's default factorisation
   if (pre) {
     sp.hi = reinterpret_cast<float*>(s.Lrow);
     sp.lda = (L + 3) & ~3;
@@ -162,9 +163,19 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
     if (!f64 && solve_inv_fits(L))
       e = launch_solve_inv(L, static_cast<const float*>(s.limg), s.mimg, s.invdiag, s.info, I,
                            s.BT, L, Rl, Rr, core_out, s.wimg, st, tiles ? s.fast : nullptr);
-    else
-      e = launch_trsm(f64 ? 1 : 2, !f64, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out, nullptr,
-                      st, s.limg, s.mimg);
+    else {
+      CdfEpilogue gate{};
+      const bool big = tiles && solve_big_fits(L);
+      if (big) {
+        const int64_t room = s.splits * (L + I) / 3;
+        e = launch_solve_big(L, s.wimg, s.mimg, s.fast, I, s.BT, L, Rl, Rr, core_out,
+                             static_cast<float*>(s.partial), room < I ? room : I, st);
+        gate.run_if = s.fast + 1;
+      }
+      if (e == cudaSuccess)
+        e = launch_trsm(f64 ? 1 : 2, !f64, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out,
+                        nullptr, st, s.limg, s.mimg, big ? &gate : nullptr);
+    }
   }
   if (e == cudaSuccess && info)
     e = cudaMemcpyAsync(info, s.info, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);

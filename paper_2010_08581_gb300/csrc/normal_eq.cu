@@ -4,30 +4,32 @@
 // writes its own partial C so that the reduction order downstream is fixed (results do
 // not depend on scheduling).
 //
-// SIMT tiles: 64 x 64 outputs per CTA in FP32, 32 x 32 in FP64, 16 rows of J per shared-memory
-// stage, the next stage's values in flight while one is multiplied. T = float accumulates in
-// FP32 within a chunk; T = double in FP64, where the FP64 pipe (2 multiply-adds per clock and
-// SM) is the bound: work on padding and idle SMs cost directly. With 64 x 64 tiles J = 2000,
-// L = 25, I = 100 ran on 64 of 152 SMs with 61% of the rows padding (78 us); with 32 x 32 on 128
-// (23 us). A tile below M's diagonal is not computed but written by its mirror image
-// (J = 2000, L = 100, I = 4: 77 -> 74 us). The chunks, and with them every sum, are the same.
+// SIMT tiles: 64 x 64 outputs per CTA in FP32, 32 x 32 or 16 x 16 in FP64, 16 rows of J per
+// shared-memory stage, the next stage's values in flight while one is multiplied. T = float
+// accumulates in FP32 within a chunk; T = double in FP64, where the FP64 pipe (2 multiply-adds
+// per clock and SM) is the bound: work on padding and idle SMs cost directly. With 64 x 64 tiles
+// J = 2000, L = 25, I = 100 ran on 64 of 152 SMs with 61% of the rows padding (78 us); with
+// 32 x 32 on 128 (23 us). A tile below M's diagonal is not computed but written by its mirror
+// image. 16 x 16 where that leaves the busiest SM less to do: J = 2000, L = 100, I = 4 is 160
+// tiles of 32 x 32, two on 8 of the SMs (74 us), or 560 of 16 x 16, four at most (28 us). The
+// chunks, and with them every sum, are the same.
 #include "common.cuh"
 
 namespace trk {
 namespace {
 
-constexpr int BK = 16, NT = 256;
+constexpr int BK = 16;
 
-// Edge of an output tile, by type.
-constexpr int tile_edge(bool f64) { return f64 ? 32 : 64; }
+// Threads along an edge of a BM x BM tile.
+constexpr int tile_threads(int bm) { return bm < 32 ? 8 : 16; }
 
-template <typename T>
-__global__ void __launch_bounds__(NT) k_normal_eq(const T* __restrict__ A,
+template <typename T, int BM>
+__global__ void __launch_bounds__(tile_threads(BM) * tile_threads(BM)) k_normal_eq(const T* __restrict__ A,
                                                   const T* __restrict__ Y, int64_t J, int L,
                                                   int64_t I, int64_t chunk,
                                                   T* __restrict__ partial,
                                                   const int64_t* __restrict__ jdev) {
-  constexpr int BM = tile_edge(sizeof(T) == 8), BN = BM, U = BM / 16, V = BN / 16;
+  constexpr int BN = BM, TE = tile_threads(BM), NT = TE * TE, U = BM / TE, V = BN / TE;
   __shared__ T As[2][BK][BM];
   __shared__ T Bs[2][BK][BN];
   const int64_t ldc = L + I;
@@ -39,7 +41,7 @@ __global__ void __launch_bounds__(NT) k_normal_eq(const T* __restrict__ A,
   const int64_t j0 = static_cast<int64_t>(blockIdx.z) * chunk;
   const int64_t Jr = jdev ? (*jdev < J ? *jdev : J) : J;
   const int64_t j1 = (j0 + chunk < Jr) ? j0 + chunk : Jr;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads
+  const int tx = threadIdx.x % TE, ty = threadIdx.x / TE;
   T acc[U][V];
 #pragma unroll
   for (int u = 0; u < U; ++u)
@@ -79,9 +81,9 @@ __global__ void __launch_bounds__(NT) k_normal_eq(const T* __restrict__ A,
     for (int kk = 0; kk < BK; ++kk) {
       T a[U], b[V];
 #pragma unroll
-      for (int u = 0; u < U; ++u) a[u] = As[s][kk][ty + 16 * u];
+      for (int u = 0; u < U; ++u) a[u] = As[s][kk][ty + TE * u];
 #pragma unroll
-      for (int v = 0; v < V; ++v) b[v] = Bs[s][kk][tx + 16 * v];
+      for (int v = 0; v < V; ++v) b[v] = Bs[s][kk][tx + TE * v];
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -91,11 +93,11 @@ __global__ void __launch_bounds__(NT) k_normal_eq(const T* __restrict__ A,
   T* out = partial + static_cast<int64_t>(blockIdx.z) * L * ldc;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int r = r0 + ty + 16 * u;
+    const int r = r0 + ty + TE * u;
     if (r >= L) continue;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      const int64_t c = c0 + tx + 16 * v;
+      const int64_t c = c0 + tx + TE * v;
       if (c < ldc) out[static_cast<int64_t>(r) * ldc + c] = acc[u][v];
       // the mirror image of an entry whose own tile was not computed
       if (kMirror && c < L && r / BN * BN + BN <= c / BM * BM)
@@ -118,6 +120,15 @@ void plan(int64_t J, int L, int64_t I, int* splits, int64_t* chunk) {
   *chunk = c;
 }
 
+template <typename T, int BM>
+void go(const void* A, const void* Y, int64_t J, int L, int64_t I, int64_t chunk, void* partial,
+        int splits, cudaStream_t st, const int64_t* jdev) {
+  const dim3 grid(static_cast<unsigned>((L + I + BM - 1) / BM), (L + BM - 1) / BM, splits);
+  k_normal_eq<T, BM><<<grid, tile_threads(BM) * tile_threads(BM), 0, st>>>(
+      static_cast<const T*>(A), static_cast<const T*>(Y), J, L, I, chunk, static_cast<T*>(partial),
+      jdev);
+}
+
 }  // namespace
 
 size_t normal_eq_workspace(int64_t J, int L, int64_t I, bool f64, int* splits) {
@@ -133,16 +144,17 @@ cudaError_t launch_normal_eq(const void* A, const void* Y, bool f64, int64_t J, 
   int64_t chunk;
   plan(J, L, I, &s, &chunk);
   if (s != splits) return cudaErrorInvalidValue;
-  const int b = tile_edge(f64);
-  dim3 grid(static_cast<unsigned>((L + I + b - 1) / b), (L + b - 1) / b, s);
-  if (f64)
-    k_normal_eq<double><<<grid, NT, 0, st>>>(static_cast<const double*>(A),
-                                             static_cast<const double*>(Y), J, L, I, chunk,
-                                             static_cast<double*>(partial), jdev);
-  else
-    k_normal_eq<float><<<grid, NT, 0, st>>>(static_cast<const float*>(A),
-                                            static_cast<const float*>(Y), J, L, I, chunk,
-                                            static_cast<float*>(partial), jdev);
+  if (f64) {
+    // the busiest SM's multiply-adds with tiles of edge b (those below M's diagonal left out)
+    auto share = [&](int64_t b) {
+      const int64_t rows = (L + b - 1) / b, ctas = (rows * ((L + I + b - 1) / b) - rows * (rows - 1) / 2) * s;
+      return (ctas + sm_count() - 1) / sm_count() * b * b;
+    };
+    if (share(16) < share(32)) go<double, 16>(A, Y, J, L, I, chunk, partial, s, st, jdev);
+    else go<double, 32>(A, Y, J, L, I, chunk, partial, s, st, jdev);
+  } else {
+    go<float, 64>(A, Y, J, L, I, chunk, partial, s, st, jdev);
+  }
   return cudaGetLastError();
 }
 

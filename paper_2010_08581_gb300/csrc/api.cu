@@ -452,7 +452,7 @@ tr_status solve_contract(tr_ctx* ctx, const SolvePlan& s, const void* A, const v
   // mixed: the reduction also writes M's FP32 values in the factorisation's work-array
   // layout (into Lrow, free until an FP64 fallback) and M's FP32 image
   ReduceSplit sp;
-  if (!f64 && L >= 4) {
+  if (f64 ? solve_f64_fits(I, L, s.splits) : L >= 4) {
     sp.hi = reinterpret_cast<float*>(s.Lrow);
     sp.lda = (L + 3) & ~3;
     sp.img = s.mimg;
@@ -474,7 +474,8 @@ int* tiles_flag(const tr_ctx* ctx, const SolvePlan& s, bool f64, int L) {
              ? s.fast : nullptr;
 }
 
-tr_status solve_cholesky(tr_ctx* ctx, const SolvePlan& s, bool f64, int L, cudaStream_t st) {
+tr_status solve_cholesky(tr_ctx* ctx, const SolvePlan& s, bool f64, int L, int64_t I,
+                         cudaStream_t st) {
   const double eps = 2.220446049250313e-16;
   const int mode = ctx->ls_rank == TR_LS_RANK_DROP ? 1 : 0;
   if (!f64 && ctx->factorization == TR_FACTOR_FP64) {
@@ -496,10 +497,16 @@ tr_status solve_cholesky(tr_ctx* ctx, const SolvePlan& s, bool f64, int L, cudaS
                                     tiles_flag(ctx, s, f64, L)));
     return TR_OK;
   }
+  // X' of M where it pays; the one-CTA factorisation and the substitutions then run only when a
+  // device flag says so
+  const bool inv = solve_f64_fits(I, L, s.splits);
+  if (inv)
+    TR_LAUNCH("solve_factor", launch_leverage_f64(0, solve_f64_plan(s, L), nullptr, 0, L, 0, nullptr,
+                                                  CdfEpilogue{}, st));
   TR_LAUNCH("cholesky_solve",
             launch_cholesky(s.M, L, mode, static_cast<double>(L) * eps, s.Lrow, s.Lcol, s.invdiag,
                             s.keep, s.info, ctx->d_err, st, static_cast<double*>(s.limg),
-                            nullptr, nullptr));
+                            nullptr, nullptr, inv ? s.info + 9 : nullptr));
   return TR_OK;
 }
 
@@ -520,6 +527,11 @@ tr_status solve_rhs(tr_ctx* ctx, const SolvePlan& s, int Rl, int Rr, int64_t I, 
                                             static_cast<float*>(s.partial), room < I ? room : I, st));
     gate.run_if = big + 1;
   }
+  if (!refine && solve_f64_fits(I, L, s.splits)) {
+    big = s.info + 8;
+    TR_LAUNCH("solve_rhs", launch_solve_f64(solve_f64_plan(s, L), L, s.BT, L, I, Rl, Rr, core_out, st));
+    gate.run_if = big + 1;
+  }
   TR_LAUNCH(big ? "solve_gated" : "solve_rhs",
             launch_trsm(refine ? 2 : 1, refine, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out,
                         nullptr, st, s.limg, s.mimg, big ? &gate : nullptr));
@@ -528,7 +540,7 @@ tr_status solve_rhs(tr_ctx* ctx, const SolvePlan& s, int Rl, int Rr, int64_t I, 
 
 tr_status solve_factor(tr_ctx* ctx, const SolvePlan& s, bool f64, int Rl, int Rr, int64_t I,
                        bool refine, double* core_out, cudaStream_t st) {
-  TR_TRY(solve_cholesky(ctx, s, f64, Rl * Rr, st));
+  TR_TRY(solve_cholesky(ctx, s, f64, Rl * Rr, I, st));
   return solve_rhs(ctx, s, Rl, Rr, I, refine, core_out, st);
 }
 
@@ -560,7 +572,7 @@ tr_status update_run(tr_ctx* ctx, char* ws, size_t solve_ws, const void* A, cons
   const bool bt_planes = p && mixed_lev && ctx->ls_rank != TR_LS_RANK_DROP && I >= L;
   TR_TRY(solve_contract(ctx, s, A, Y, f64, J, L, I, st, jdev, bt_planes, post));
   if (!p) {   // uniform sampling: the new core needs no distribution
-    TR_TRY(solve_cholesky(ctx, s, f64, L, st));
+    TR_TRY(solve_cholesky(ctx, s, f64, L, I, st));
     return solve_rhs(ctx, s, Rl, Rr, I, !f64, core_out, st);
   }
   if (ctx->ls_rank == TR_LS_RANK_DROP) {
@@ -569,14 +581,14 @@ tr_status update_run(tr_ctx* ctx, char* ws, size_t solve_ws, const void* A, cons
     // distribution is therefore the leverage of the new core itself (Alg. 2, "update n-th
     // distribution"), formed after the solve. The core's slice-major rows are its G_(2) rows
     // with the columns permuted, which leaves the leverage scores unchanged.
-    TR_TRY(solve_cholesky(ctx, s, f64, L, st));
+    TR_TRY(solve_cholesky(ctx, s, f64, L, I, st));
     TR_TRY(solve_rhs(ctx, s, Rl, Rr, I, !f64, core_out, st));
     return leverage_dist(ctx, ws + solve_ws, core_out, I, L, p, cdf, s.info, st, nullptr,
                          mixed_lev);
   }
   TR_CUDA(cudaEventRecord(ctx->ev_fork, st));
   TR_CUDA(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
-  TR_TRY(solve_cholesky(ctx, s, f64, L, st));
+  TR_TRY(solve_cholesky(ctx, s, f64, L, I, st));
   // The side branch needs the solve's Cholesky status (info) only in its last kernel, to
   // keep the old distribution when the core was not updated.
   TR_CUDA(cudaEventRecord(ctx->ev_info, st));

@@ -325,7 +325,36 @@ struct Lev64 {
   double* partial;   // splits * n * n
   int splits;
   double tau;
+  int* keep = nullptr;   // LS step: keep = 1 and *info = 0 when the series applies
+  int* info = nullptr;
 };
+// The FP64 LS step through the same form of M (part 0, then the solves): the contraction's
+// partials, splits * n * (n + I) doubles, are the scratch. When part 0 finds that it does not
+// apply, bad[1] = 1 and nothing is written.
+bool solve_f64_fits(int64_t I, int n, int splits);
+cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t ld, int64_t I, int Rl,
+                             int Rr, double* core_out, cudaStream_t st);
+cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,
+                                int64_t lda, double* ell, const CdfEpilogue& ep, cudaStream_t st);
+// The FP64 LS step through an FP32 inverse (lev64.cu) on a solve's workspace; the flags are in
+// the info word's 256-byte slot.
+template <typename Plan>
+Lev64 solve_f64_plan(const Plan& s, int L) {
+  Lev64 w{};
+  w.K32 = reinterpret_cast<float*>(s.Lrow);
+  w.ldk = (L + 3) & ~3;
+  w.G = s.M;
+  w.Ximg = static_cast<float*>(s.limg);
+  w.E = s.Lcol;
+  w.bad = s.info + 8;
+  w.partial = static_cast<double*>(s.partial);
+  w.splits = s.splits;
+  w.tau = 1e-2;
+  w.keep = s.keep;
+  w.info = s.info;
+  return w;
+}
+
 bool leverage_f64_fits(int64_t I, int n, int splits);
 cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,
                                 int64_t lda, double* ell, const CdfEpilogue& ep, cudaStream_t st);

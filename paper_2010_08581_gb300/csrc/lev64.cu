@@ -4,6 +4,7 @@
 //     identity of lev_precond.cu), K^-1 = X'^T X' for X' = C^-1/2 X, so ell_i = ||X' a_i||^2. Every
 //     product is in FP64 and C^-1/2 is its binomial series in E, through E^3 for
 //     ||E||_F <= 1e-4, E^5 up to 1e-3 and E^7 up to 1e-2: a remainder below 3e-17 each time;
+//   * the FP64 LS step (row a6): z = M^-1 b = X'^T (X' b) with the same X' of M;
 //   * the mixed-precision LS step's solves (row a6) for 160 < L <= 256.
 //
 // Why: one SM multiplies two FP64 pairs per clock, so the one-CTA FP64 factorisation of a 256 x
@@ -392,6 +393,32 @@ __global__ void __launch_bounds__(kFinishThreads) k_l64_finish(L64 g, const doub
   if (ep.p) cdf_epilogue_nw<kFinishThreads / 32>(ep, ell, I);
 }
 
+// The FP64 LS step: y = X' b for `rows` right-hand sides (rows of B^T), then z = X'^T y into the
+// new core.
+__global__ void __launch_bounds__(DNT) k_l64_y(L64 g, const double* __restrict__ b, int64_t ld,
+                                               int rows, double* __restrict__ y) {
+  __shared__ __align__(16) Panels sm;
+  if (g.flag[0] || g.flag[2] == 0) return;
+  const int n = g.n;
+  tile8<true, true>(sm, blockIdx.y * DE, blockIdx.x * DE, 0, n,
+      [&](int i, int k) { return i < rows ? b[i * ld + k] : 0.0; },
+      [&](int k, int j) { return j < n ? g.T[j * n + k] : 0.0; },
+      [&](int i, int j, double v) { if (i < rows && j < n) y[static_cast<int64_t>(i) * n + j] = v; });
+}
+
+__global__ void __launch_bounds__(DNT) k_l64_z(L64 g, const double* __restrict__ y, int rows, int Rl,
+                                               int Rr, double* __restrict__ core) {
+  __shared__ __align__(16) Panels sm;
+  if (g.flag[0] || g.flag[2] == 0) return;
+  const int n = g.n;
+  tile8<true, false>(sm, blockIdx.y * DE, blockIdx.x * DE, 0, n,
+      [&](int i, int k) { return i < rows ? y[static_cast<int64_t>(i) * n + k] : 0.0; },
+      [&](int k, int j) { return j < n ? g.T[k * n + j] : 0.0; },
+      [&](int i, int j, double v) {
+        if (i < rows && j < n) core[static_cast<int64_t>(i) * n + (j % Rl) * Rr + j / Rl] = v;
+      });
+}
+
 // ------------------------------------------------------------------------------------
 // The mixed LS step's solves, 160 < n <= 256, `rows` right-hand sides b (rows of B^T): with
 // W = X: y = W b, z = W^T y, r = b - M z, y = W r, z += W^T y, in FP32, as solve_inv.cu.
@@ -467,8 +494,8 @@ unsigned dtiles(int64_t n) { return static_cast<unsigned>((n + DE - 1) / DE); }
 
 L64 args_of(const Lev64& w, int n) {
   const size_t nn = static_cast<size_t>(n) * n;
-  return L64{n, w.Ximg, w.G, w.E, w.partial, w.partial + nn, w.partial + 2 * nn, w.bad, nullptr,
-             nullptr, w.tau * w.tau};
+  return L64{n, w.Ximg, w.G, w.E, w.partial, w.partial + nn, w.partial + 2 * nn, w.bad, w.keep,
+             w.info, w.tau * w.tau};
 }
 
 unsigned tiles_of(int64_t n) { return static_cast<unsigned>((n + GE - 1) / GE); }
@@ -525,6 +552,28 @@ cudaError_t launch_solve_big(int n, const float* Wimg, const float* Mimg, const 
     k_sv_residual<<<grid, GNT, 0, st>>>(n, Mimg, bad, m, b, ld, z, r);
     k_sv_lower<float><<<grid, GNT, 0, st>>>(n, Wimg, bad, m, r, n, y);
     k_sv_upper<<<grid, GNT, 0, st>>>(n, Wimg, bad, m, y, z, nullptr, Rl, Rr, core_out + r0 * n);
+  }
+  return cudaGetLastError();
+}
+
+// (The same line for the FP64 LS step, with the gated launches: L = 64, 300 right-hand sides: 114 ->
+// 117 us, L = 100: 210 -> 162, L = 256: 2430 -> 410.)
+bool solve_f64_fits(int64_t I, int n, int splits) {
+  return n >= kLev64MinN && n <= kMaxL &&
+         static_cast<int64_t>(splits) * (n + I) >= 3 * static_cast<int64_t>(n) + 1;
+}
+
+cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t ld, int64_t I, int Rl,
+                             int Rr, double* core_out, cudaStream_t st) {
+  const L64 g = args_of(w, n);
+  double* y = w.partial + 3 * static_cast<size_t>(n) * n;
+  int64_t rows = static_cast<int64_t>(w.splits) * (n + I) - 3 * static_cast<int64_t>(n);
+  if (rows > kMaxRows) rows = kMaxRows;
+  for (int64_t r0 = 0; r0 < I; r0 += rows) {
+    const int m = static_cast<int>(I - r0 < rows ? I - r0 : rows);
+    const dim3 grid(dtiles(n), dtiles(m));
+    k_l64_y<<<grid, DNT, 0, st>>>(g, rhs + r0 * ld, ld, m, y);
+    k_l64_z<<<grid, DNT, 0, st>>>(g, y, m, Rl, Rr, core_out + r0 * n);
   }
   return cudaGetLastError();
 }

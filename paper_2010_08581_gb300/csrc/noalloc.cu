@@ -138,7 +138,8 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
   // The same reduction, factorisation and solves as tr_solve (stop-on-singular rule): on the
   // mixed path the reduction also writes M's FP32 work array and image for the FP32 factor.
   ReduceSplit sp;
-  const bool pre = !f64 && L >= 4;
+  const bool inv = f64 && solve_f64_fits(I, L, s.splits);
+  const bool pre = inv || (!f64 && L >= 4);
   const bool tiles = !f64 && L >= 4 && (L <= 128 || solve_big_fits(L));   // as tr_solve's default factorisation
   if (pre) {
     sp.hi = reinterpret_cast<float*>(s.Lrow);
@@ -149,9 +150,12 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
   if (e == cudaSuccess)
     e = launch_reduce(s.partial, !f64, s.splits, L * ld, ld, L, ld, L, s.M, L, s.BT, L, st, sp);
   if (e == cudaSuccess) {
-    if (f64)
+    if (inv) e = launch_leverage_f64(0, solve_f64_plan(s, L), nullptr, 0, L, 0, nullptr, CdfEpilogue{}, st);
+    if (e != cudaSuccess) {
+    } else if (f64)
       e = launch_cholesky(s.M, L, 0, static_cast<double>(L) * eps, s.Lrow, s.Lcol, s.invdiag,
-                          s.keep, s.info, s.err, st, static_cast<double*>(s.limg));
+                          s.keep, s.info, s.err, st, static_cast<double*>(s.limg), nullptr, nullptr,
+                          inv ? s.info + 9 : nullptr);
     else
       e = launch_cholesky_mixed(s.M, L, 0, static_cast<double>(L) * eps,
                                 static_cast<double>(L) * eps32, s.Lrow, s.Lcol, s.invdiag,
@@ -171,10 +175,13 @@ extern "C" tr_status tr_solve_noalloc(const void* A, const void* Y, tr_dtype dty
         e = launch_solve_big(L, s.wimg, s.mimg, s.fast, I, s.BT, L, Rl, Rr, core_out,
                              static_cast<float*>(s.partial), room < I ? room : I, st);
         gate.run_if = s.fast + 1;
+      } else if (inv) {
+        e = launch_solve_f64(solve_f64_plan(s, L), L, s.BT, L, I, Rl, Rr, core_out, st);
+        gate.run_if = s.info + 9;
       }
       if (e == cudaSuccess)
         e = launch_trsm(f64 ? 1 : 2, !f64, L, s.invdiag, s.info, I, s.BT, L, Rl, Rr, core_out,
-                        nullptr, st, s.limg, s.mimg, big ? &gate : nullptr);
+                        nullptr, st, s.limg, s.mimg, gate.run_if ? &gate : nullptr);
     }
   }
   if (e == cudaSuccess && info)

@@ -1,5 +1,5 @@
-"""FP64 leverage scores of tall cores through an FP32 inverse (48 <= L <= 256, I >= L), and the
-mixed LS step's blocked factor for L > 128: block edges, one row above square, columns of very
+"""FP64 leverage scores of tall cores through an FP32 inverse (L >= 88, I >= L), and the
+mixed LS step's blocked factor for L > 160: block edges, one row above square, columns of very
 different lengths (the FP32 factorisation gives up: the FP64 one runs), scales outside FP32's
 range, dependent columns.
 

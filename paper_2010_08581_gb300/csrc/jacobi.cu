@@ -83,11 +83,15 @@ __global__ void __launch_bounds__(JT) k_leverage_jacobi(const double* __restrict
         al = warp_sum(al);
         be = warp_sum(be);
         ga = warp_sum(ga);
+        // rotation zeroing the inner product of rows a and b, tan = 2 ga sign(d) / (|d| + hypot(d,
+        // 2 ga)): the test's square root beside the hypotenuse, then one division and one reciprocal
+        // square root. Each is a chain of a dozen dependent FP64 operations (three divisions and
+        // three square roots in turn before: 4 x 100, 71 us; 4.5 us less now, by whole updates).
+        const double d = be - al, g2 = 2.0 * ga;
+        const double den = fabs(d) + hypot(d, g2);
         if (al == 0.0 || be == 0.0 || !(fabs(ga) > rot_tol * sqrt(al * be))) continue;
-        // rotation zeroing the inner product of rows a and b
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double cs = 1.0 / sqrt(1.0 + t * t), sn = cs * t;
+        const double t = (d == 0.0 || (d > 0.0) == (ga > 0.0) ? fabs(g2) : -fabs(g2)) / den;
+        const double cs = rsqrt(1.0 + t * t), sn = cs * t;
         for (int c = lane; c < L; c += 32) {
           const double x = ra[c], y = rb[c];
           ra[c] = cs * x - sn * y;

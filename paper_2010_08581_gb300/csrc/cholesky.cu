@@ -15,6 +15,7 @@ __global__ void __launch_bounds__(CNT) k_cholesky(const double* __restrict__ G, 
                                                   unsigned* err, int use_smem,
                                                   double* img64, float* img32, float* gimg32,
                                                   const int* __restrict__ run_if) {
+  grid_wait();
   extern __shared__ double smem[];
   if (run_if && *run_if == 0) return;
   cholesky_cta(G, n, mode, tol_scale, use_smem ? smem : Lrow, Lrow, Lcol, invdiag, keep_out,
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(CNT) k_cholesky_mixed(const double* __restrict
                                                         const float* pre,
                                                         const int* __restrict__ skip_if,
                                                         const int* __restrict__ run_if) {
+  grid_wait();
   extern __shared__ double smem[];
   if (skip_if && *skip_if) return;   // the factor and its inverse are formed already
   if (run_if && *run_if == 0) return;
@@ -59,6 +61,7 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_chol_inv_solve(int n, float t
                                                                   int* __restrict__ info,
                                                                   const unsigned* err,
                                                                   int* __restrict__ fast) {
+  grid_wait();
   __shared__ CiShared cs;
   if (err && (*reinterpret_cast<const volatile unsigned*>(err) & kErrTimeout)) {
     if (threadIdx.x == 0) {
@@ -86,6 +89,7 @@ __global__ void __launch_bounds__(CNT) k_cholesky_lev_mixed(const double* __rest
                                                             const float* pre_hi,
                                                             const float* pre_lo,
                                                             const int* run_if) {
+  grid_wait();
   extern __shared__ double smem[];
   if (run_if && *run_if == 0) return;
   const int64_t nn = static_cast<int64_t>(n) * n;
@@ -101,6 +105,7 @@ __global__ void __launch_bounds__(256) k_ff_image(const float* __restrict__ hi,
                                                   const int* __restrict__ info,
                                                   double* __restrict__ img64,
                                                   const int* __restrict__ run_if) {
+  grid_wait();
   if ((run_if && *run_if == 0) || *info != 2) return;
   for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < count;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x)
@@ -113,7 +118,7 @@ cudaError_t launch_ff_image(const double* Lrow, const double* Lcol, int n, const
                             double* img64, cudaStream_t st, const int* run_if) {
   const int64_t count = static_cast<int64_t>(n) * (n + 1);
   const unsigned blocks = static_cast<unsigned>((count + 255) / 256 < sm_count() ? (count + 255) / 256 : sm_count());
-  k_ff_image<<<blocks, 256, 0, st>>>(reinterpret_cast<const float*>(Lrow),
+  launch_pdl(k_ff_image, blocks, 256, 0, st, reinterpret_cast<const float*>(Lrow),
                                      reinterpret_cast<const float*>(Lcol), count, info, img64,
                                      run_if);
   return cudaGetLastError();
@@ -128,7 +133,7 @@ cudaError_t launch_cholesky_lev_mixed(const double* G, int n, double tol64, doub
   const size_t ff = static_cast<size_t>(panel_floats<FFOps>(n)) * 4;
   const size_t want = nn * 8 > ff ? nn * 8 : ff;
   const size_t dyn = want <= kCholDyn ? want : (nn * 8 <= kCholDyn ? nn * 8 : 0);
-  k_cholesky_lev_mixed<<<1, CNT, dyn, st>>>(G, n, tol64, tolff, Lrow, Lcol, invdiag, keep, info,
+  launch_pdl(k_cholesky_lev_mixed, 1, CNT, dyn, st, G, n, tol64, tolff, Lrow, Lcol, invdiag, keep, info,
                                             err, static_cast<int>(dyn), img64, pre_hi, pre_lo,
                                             run_if);
   return cudaGetLastError();
@@ -142,7 +147,7 @@ cudaError_t launch_cholesky_mixed(const double* G, int n, int mode, double tol64
   const size_t dyn = nn * 8 <= kCholDyn ? nn * 8 : (nn * 4 <= kCholDyn ? nn * 4 : 0);
   const bool tiles = wimg && fast && pre && n >= 4 && n <= kCiMaxN;
   if (tiles) {
-    k_chol_inv_solve<<<1, chol_inv_threads(n), 0, st>>>(n, static_cast<float>(tol32), pre,
+    launch_pdl(k_chol_inv_solve, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(tol32), pre,
                                                         (n + 3) & ~3, wimg, keep, info, err, fast);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -156,7 +161,7 @@ cudaError_t launch_cholesky_mixed(const double* G, int n, int mode, double tol64
     if (e != cudaSuccess) return e;
   }
   // (beyond kPanelCholMax the one-CTA factorisation reads G, and its work arrays may be pre's)
-  k_cholesky_mixed<float><<<1, CNT, dyn, st>>>(G, n, mode, tol64, tol32, Lrow, Lcol, invdiag, keep,
+  launch_pdl(k_cholesky_mixed<float>, 1, CNT, dyn, st, G, n, mode, tol64, tol32, Lrow, Lcol, invdiag, keep,
                                                info, err, static_cast<int>(dyn), img32, gimg32,
                                                n <= kPanelCholMax ? pre : nullptr,
                                                tiles ? fast : nullptr, big ? fast + 1 : nullptr);
@@ -170,7 +175,7 @@ cudaError_t launch_cholesky(const double* G, int n, int mode, double tol_scale, 
   const size_t bytes = static_cast<size_t>(n) * n * sizeof(double);
   const int use_smem = bytes <= kCholDyn ? 1 : 0;
   const size_t dyn = use_smem ? bytes : 0;
-  k_cholesky<<<1, CNT, dyn, st>>>(G, n, mode, tol_scale, Lrow, Lcol, invdiag, keep, info, err,
+  launch_pdl(k_cholesky, 1, CNT, dyn, st, G, n, mode, tol_scale, Lrow, Lcol, invdiag, keep, info, err,
                                   use_smem, img64, img32, gimg32, run_if);
   return cudaGetLastError();
 }

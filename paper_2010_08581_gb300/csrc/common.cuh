@@ -383,6 +383,37 @@ cudaError_t launch_merge(const int32_t* idx, const double* w, int64_t J, int npo
 cudaError_t launch_init_normal(double* out, int64_t count, uint64_t seed, uint32_t stream_id,
                                const uint64_t* seed_dev, cudaStream_t st);
 
+// A kernel of a chain, launched while its predecessor on the stream still runs (programmatic
+// dependent launch): its blocks are scheduled when the predecessor's last ones are, and wait in
+// grid_wait for the predecessor's results. The update's chains are a dozen short kernels, each of
+// which otherwise starts with about 2 us of launch and drain (update of 40^3 in FP64: 141 -> 122 us,
+// of 500^3: 524 -> 446). Every kernel launched this way calls grid_wait before anything else, so
+// that the completion of one implies that of all before it. Not while a graph is captured: there
+// the chains ran 2 % slower with such edges (500^3, ten sweeps: 4.95 -> 5.06 ms).
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+  cudaStreamIsCapturing(st, &cap);
+  cfg.attrs = &attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);   // (callers read cudaGetLastError)
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // Number of SMs of the current device (queried once per device and cached); grids of the
 // streaming kernels and the split counts of the contractions are sized from it.
 int sm_count();

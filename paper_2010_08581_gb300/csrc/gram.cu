@@ -15,6 +15,7 @@ constexpr int GT = 32, GK = 32, GNT = 256;
 __global__ void __launch_bounds__(GNT) k_gram(const double* __restrict__ A, int64_t K, int n,
                                               int64_t lda, bool trans, int64_t chunk,
                                               double* __restrict__ partial) {
+  grid_wait();
   __shared__ double P[GK][GT + 1];
   __shared__ double Q[GK][GT + 1];
   const int nt = (n + GT - 1) / GT;
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(GNT) k_gram_ff(const float* __restrict__ Ah,
                                                  const float* __restrict__ Al, int64_t K, int n,
                                                  int64_t lda, int64_t chunk,
                                                  double* __restrict__ partial) {
+  grid_wait();
   __shared__ float Ph[GK][GT + 1], Pl[GK][GT + 1];
   __shared__ float Qh[GK][GT + 1], Ql[GK][GT + 1];
   const int nt = (n + GT - 1) / GT;
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(256) k_reduce(const TP* __restrict__ partial, 
                                                 double* __restrict__ out1, int64_t ld1,
                                                 double* __restrict__ out2, int64_t ld2,
                                                 ReduceSplit sp) {
+  grid_wait();
   const int64_t total = nrows * ncols;
   for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -234,7 +237,7 @@ cudaError_t launch_gram(const double* A, int64_t rows, int cols, int64_t lda, bo
   const int s = plan_splits(K, nt * (nt + 1) / 2, GK, &chunk);
   if (s != splits) return cudaErrorInvalidValue;
   dim3 grid(nt * (nt + 1) / 2, s);
-  k_gram<<<grid, GNT, 0, st>>>(A, K, n, lda, trans, chunk, partial);
+  launch_pdl(k_gram, grid, GNT, 0, st, A, K, n, lda, trans, chunk, partial);
   return cudaGetLastError();
 }
 
@@ -246,7 +249,7 @@ cudaError_t launch_gram_ff(const float* Ah, const float* Al, int64_t rows, int c
   const int s = plan_splits(rows, nt * (nt + 1) / 2, GK, &chunk);
   if (s != splits) return cudaErrorInvalidValue;
   dim3 grid(nt * (nt + 1) / 2, s);
-  k_gram_ff<<<grid, GNT, 0, st>>>(Ah, Al, rows, n, lda, chunk, partial);
+  launch_pdl(k_gram_ff, grid, GNT, 0, st, Ah, Al, rows, n, lda, chunk, partial);
   return cudaGetLastError();
 }
 
@@ -259,13 +262,13 @@ cudaError_t launch_reduce(const void* partial, bool partial_f32, int splits, int
   int64_t blocks = (total + 255) / 256;
   if (blocks > sm_count() * 16) blocks = sm_count() * 16;
   if (partial_f32)
-    k_reduce<float><<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        static_cast<const float*>(partial), splits, pstride, pld, nrows, ncols, c_split, out1,
-        ld1, out2, ld2, split);
+    launch_pdl(k_reduce<float>, static_cast<unsigned>(blocks), 256, 0, st,
+               static_cast<const float*>(partial), splits, pstride, pld, nrows, ncols, c_split, out1,
+               ld1, out2, ld2, split);
   else
-    k_reduce<double><<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        static_cast<const double*>(partial), splits, pstride, pld, nrows, ncols, c_split, out1,
-        ld1, out2, ld2, split);
+    launch_pdl(k_reduce<double>, static_cast<unsigned>(blocks), 256, 0, st,
+               static_cast<const double*>(partial), splits, pstride, pld, nrows, ncols, c_split, out1,
+               ld1, out2, ld2, split);
   return cudaGetLastError();
 }
 

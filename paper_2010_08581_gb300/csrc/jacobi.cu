@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(JT) k_leverage_jacobi(const double* __restrict
                                                         double* __restrict__ cdf,
                                                         const int* __restrict__ skip,
                                                         unsigned* err) {
+  grid_wait();
   extern __shared__ __align__(16) double jsm[];
   const int n = I + (I & 1);            // even player count; a padded row stays zero
   double* B = jsm;                      // [n][L]
@@ -169,8 +170,8 @@ cudaError_t launch_leverage_jacobi(const double* A, int64_t I, int L, int64_t ld
                                    double* p, double* cdf, const int* skip, unsigned* err,
                                    cudaStream_t st) {
   if (!leverage_jacobi_fits(I, L)) return cudaErrorInvalidValue;
-  k_leverage_jacobi<<<1, JT, leverage_jacobi_smem(I, L), st>>>(
-      A, static_cast<int>(I), L, lda, ell, p, cdf, skip, err);
+  launch_pdl(k_leverage_jacobi, 1, JT, leverage_jacobi_smem(I, L), st, A, static_cast<int>(I), L, lda,
+             ell, p, cdf, skip, err);
   return cudaGetLastError();
 }
 

@@ -99,6 +99,7 @@ struct BigInv {
 __global__ void __launch_bounds__(kCiMaxThreads) k_big_factor(BigInv g, float tol, int part,
                                                               int* keep, int* info,
                                                               const unsigned* err) {
+  grid_wait();
   __shared__ CiShared cs;
   const int np = g.n + 1, n2 = g.n - g.n1;
   if (part == 0) {
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_big_factor(BigInv g, float to
 }
 
 __global__ void __launch_bounds__(GNT) k_big_lb(BigInv g) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (g.bad[0]) return;
   const int np = g.n + 1, n1 = g.n1, n2 = g.n - n1;
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(GNT) k_big_lb(BigInv g) {
 }
 
 __global__ void __launch_bounds__(GNT) k_big_s(BigInv g) {
+  grid_wait();
   __shared__ Stages<float> sm;
   const int i0 = blockIdx.y * GE, j0 = blockIdx.x * GE;
   if (g.bad[0] || i0 + GE <= j0) return;
@@ -146,6 +149,7 @@ __global__ void __launch_bounds__(GNT) k_big_s(BigInv g) {
 }
 
 __global__ void __launch_bounds__(GNT) k_big_t(BigInv g) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (g.bad[0]) return;
   const int np = g.n + 1, n1 = g.n1, n2 = g.n - n1;
@@ -158,6 +162,7 @@ __global__ void __launch_bounds__(GNT) k_big_t(BigInv g) {
 }
 
 __global__ void __launch_bounds__(GNT) k_big_x21(BigInv g) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (g.bad[0]) return;
   const int np = g.n + 1, n1 = g.n1, n2 = g.n - n1;
@@ -252,6 +257,7 @@ struct L64 {
 
 // U = X K.
 __global__ void __launch_bounds__(DNT) k_l64_u(L64 g) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0]) return;
   const int n = g.n, np = n + 1, i0 = blockIdx.y * DE, j0 = blockIdx.x * DE;
@@ -264,6 +270,7 @@ __global__ void __launch_bounds__(DNT) k_l64_u(L64 g) {
 // E = U X^T - I on the tiles with i0 <= j0, both triangles written, and the tile's share of
 // ||E||_F^2 in P[tile].
 __global__ void __launch_bounds__(DNT) k_l64_e(L64 g) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0]) return;
   const int n = g.n, np = n + 1;
@@ -293,6 +300,7 @@ __device__ __forceinline__ double l64_c(int k) {
 
 // Degree of the series by ||E||_F: 3, 5, 7, or 0 when E is too large for it; E2 = E E.
 __global__ void __launch_bounds__(DNT) k_l64_e2(L64 g) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0]) return;
   const int n = g.n;
@@ -326,6 +334,7 @@ __global__ void __launch_bounds__(DNT) k_l64_e2(L64 g) {
 // E2 T into P's place by `which` = 1, 2, 3: polynomials in E, so symmetric; the tiles of the upper
 // triangle are formed and both triangles written. which = 4: X' = Q X into T's place, all tiles.
 __global__ void __launch_bounds__(DNT) k_l64_poly(L64 g, int which) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0]) return;
   const int deg = g.flag[2];
@@ -361,6 +370,7 @@ __global__ void __launch_bounds__(DNT) k_l64_poly(L64 g, int which) {
 // Partial row norms of A X'^T: the tile's 8 columns of ||X' a_i||^2 into part[column tile][row].
 __global__ void __launch_bounds__(DNT) k_l64_rows(L64 g, const double* __restrict__ A, int64_t lda,
                                                   int rows, double* __restrict__ part) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0] || g.flag[2] == 0) return;
   const int n = g.n, i0 = blockIdx.y * DE, j0 = blockIdx.x * DE;
@@ -381,6 +391,7 @@ constexpr int kFinishThreads = 1024;
 __global__ void __launch_bounds__(kFinishThreads) k_l64_finish(L64 g, const double* __restrict__ part,
                                                                int tiles, int rows, int64_t row0,
                                                                double* ell, int64_t I, CdfEpilogue ep) {
+  grid_wait();
   if (g.flag[0] || g.flag[2] == 0) return;
   for (int i = threadIdx.x; i < rows; i += kFinishThreads) {
     double s = 0.0;
@@ -397,6 +408,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_l64_finish(L64 g, const doub
 // new core.
 __global__ void __launch_bounds__(DNT) k_l64_y(L64 g, const double* __restrict__ b, int64_t ld,
                                                int rows, double* __restrict__ y) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0] || g.flag[2] == 0) return;
   const int n = g.n;
@@ -408,6 +420,7 @@ __global__ void __launch_bounds__(DNT) k_l64_y(L64 g, const double* __restrict__
 
 __global__ void __launch_bounds__(DNT) k_l64_z(L64 g, const double* __restrict__ y, int rows, int Rl,
                                                int Rr, double* __restrict__ core) {
+  grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0] || g.flag[2] == 0) return;
   const int n = g.n;
@@ -429,6 +442,7 @@ __global__ void __launch_bounds__(GNT) k_sv_lower(int n, const float* __restrict
                                                   const int* bad, int rows,
                                                   const TS* __restrict__ src, int64_t ld,
                                                   float* __restrict__ out) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (*bad) return;
   const int np = n + 1, i0 = blockIdx.y * GE, j0 = blockIdx.x * GE;
@@ -445,6 +459,7 @@ __global__ void __launch_bounds__(GNT) k_sv_upper(int n, const float* __restrict
                                                   const float* __restrict__ add,
                                                   float* __restrict__ z, int Rl, int Rr,
                                                   double* __restrict__ core) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (*bad) return;
   const int np = n + 1, i0 = blockIdx.y * GE, j0 = blockIdx.x * GE;
@@ -464,6 +479,7 @@ __global__ void __launch_bounds__(GNT) k_sv_residual(int n, const float* __restr
                                                      const double* __restrict__ b, int64_t ld,
                                                      const float* __restrict__ z,
                                                      float* __restrict__ r) {
+  grid_wait();
   __shared__ Stages<float> sm;
   if (*bad) return;
   const int np = n + 1, i0 = blockIdx.y * GE, j0 = blockIdx.x * GE;
@@ -479,6 +495,7 @@ constexpr double kEps32 = 1.1920928955078125e-07;
 __global__ void __launch_bounds__(kCiMaxThreads) k_small_factor(int n, float tol,
                                                                 const float* pre, int lda,
                                                                 float* Ximg, int* bad) {
+  grid_wait();
   __shared__ CiShared cs;
   const bool ok = chol_inv_tiles(n, tol, pre, lda, Ximg, n + 1, pre, n, lda, cs);
   if (threadIdx.x == 0) { bad[0] = ok ? 0 : 1; bad[1] = ok ? 0 : 1; }
@@ -527,12 +544,12 @@ cudaError_t launch_inv256(int n, double tol_scale, const float* pre, int lda, fl
   g.bad = bad;
   const float tol = static_cast<float>(tol_scale);
   const dim3 lb(tiles_of(g.n1), tiles_of(n2));
-  k_big_factor<<<1, chol_inv_threads(g.n1), 0, st>>>(g, tol, 0, nullptr, info, err);
-  k_big_lb<<<lb, GNT, 0, st>>>(g);
-  k_big_s<<<dim3(tiles_of(n2), tiles_of(n2)), GNT, 0, st>>>(g);
-  k_big_factor<<<1, chol_inv_threads(n2), 0, st>>>(g, tol, 1, keep, info, nullptr);
-  k_big_t<<<lb, GNT, 0, st>>>(g);
-  k_big_x21<<<lb, GNT, 0, st>>>(g);
+  launch_pdl(k_big_factor, 1, chol_inv_threads(g.n1), 0, st, g, tol, 0, nullptr, info, err);
+  launch_pdl(k_big_lb, lb, GNT, 0, st, g);
+  launch_pdl(k_big_s, dim3(tiles_of(n2), tiles_of(n2)), GNT, 0, st, g);
+  launch_pdl(k_big_factor, 1, chol_inv_threads(n2), 0, st, g, tol, 1, keep, info, nullptr);
+  launch_pdl(k_big_t, lb, GNT, 0, st, g);
+  launch_pdl(k_big_x21, lb, GNT, 0, st, g);
   return cudaGetLastError();
 }
 
@@ -547,11 +564,11 @@ cudaError_t launch_solve_big(int n, const float* Wimg, const float* Mimg, const 
     float* r = z + static_cast<int64_t>(m) * n;
     const double* b = rhs + r0 * ld;
     const dim3 grid(tiles_of(n), tiles_of(m));
-    k_sv_lower<double><<<grid, GNT, 0, st>>>(n, Wimg, bad, m, b, ld, y);
-    k_sv_upper<<<grid, GNT, 0, st>>>(n, Wimg, bad, m, y, nullptr, z, Rl, Rr, nullptr);
-    k_sv_residual<<<grid, GNT, 0, st>>>(n, Mimg, bad, m, b, ld, z, r);
-    k_sv_lower<float><<<grid, GNT, 0, st>>>(n, Wimg, bad, m, r, n, y);
-    k_sv_upper<<<grid, GNT, 0, st>>>(n, Wimg, bad, m, y, z, nullptr, Rl, Rr, core_out + r0 * n);
+    launch_pdl(k_sv_lower<double>, grid, GNT, 0, st, n, Wimg, bad, m, b, ld, y);
+    launch_pdl(k_sv_upper, grid, GNT, 0, st, n, Wimg, bad, m, y, nullptr, z, Rl, Rr, nullptr);
+    launch_pdl(k_sv_residual, grid, GNT, 0, st, n, Mimg, bad, m, b, ld, z, r);
+    launch_pdl(k_sv_lower<float>, grid, GNT, 0, st, n, Wimg, bad, m, r, n, y);
+    launch_pdl(k_sv_upper, grid, GNT, 0, st, n, Wimg, bad, m, y, z, nullptr, Rl, Rr, core_out + r0 * n);
   }
   return cudaGetLastError();
 }
@@ -572,8 +589,8 @@ cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t l
   for (int64_t r0 = 0; r0 < I; r0 += rows) {
     const int m = static_cast<int>(I - r0 < rows ? I - r0 : rows);
     const dim3 grid(dtiles(n), dtiles(m));
-    k_l64_y<<<grid, DNT, 0, st>>>(g, rhs + r0 * ld, ld, m, y);
-    k_l64_z<<<grid, DNT, 0, st>>>(g, y, m, Rl, Rr, core_out + r0 * n);
+    launch_pdl(k_l64_y, grid, DNT, 0, st, g, rhs + r0 * ld, ld, m, y);
+    launch_pdl(k_l64_z, grid, DNT, 0, st, g, y, m, Rl, Rr, core_out + r0 * n);
   }
   return cudaGetLastError();
 }
@@ -597,8 +614,8 @@ cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64
       const int m = static_cast<int>(I - r0 < most ? I - r0 : most);
       CdfEpilogue e2 = ep;
       if (r0 + m < I) e2.p = nullptr;
-      k_l64_rows<<<dim3(nt, dtiles(m)), DNT, 0, st>>>(g, A + r0 * lda, lda, m, sums);
-      k_l64_finish<<<1, kFinishThreads, 0, st>>>(g, sums, static_cast<int>(nt), m, r0, ell, I, e2);
+      launch_pdl(k_l64_rows, dim3(nt, dtiles(m)), DNT, 0, st, g, A + r0 * lda, lda, m, sums);
+      launch_pdl(k_l64_finish, 1, kFinishThreads, 0, st, g, sums, static_cast<int>(nt), m, r0, ell, I, e2);
     }
     return cudaGetLastError();
   }
@@ -607,14 +624,14 @@ cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64
                                         w.bad, nullptr, nullptr, nullptr, st);
     if (e != cudaSuccess) return e;
   } else {
-    k_small_factor<<<1, chol_inv_threads(n), 0, st>>>(n, static_cast<float>(tol), w.K32, w.ldk,
+    launch_pdl(k_small_factor, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(tol), w.K32, w.ldk,
                                                       w.Ximg, w.bad);
   }
-  k_l64_u<<<dim3(nt, nt), DNT, 0, st>>>(g);
-  k_l64_e<<<up, DNT, 0, st>>>(g);
-  k_l64_e2<<<up, DNT, 0, st>>>(g);
-  for (int k = 1; k < 4; ++k) k_l64_poly<<<up, DNT, 0, st>>>(g, k);
-  k_l64_poly<<<dim3(nt, nt), DNT, 0, st>>>(g, 4);
+  launch_pdl(k_l64_u, dim3(nt, nt), DNT, 0, st, g);
+  launch_pdl(k_l64_e, up, DNT, 0, st, g);
+  launch_pdl(k_l64_e2, up, DNT, 0, st, g);
+  for (int k = 1; k < 4; ++k) launch_pdl(k_l64_poly, up, DNT, 0, st, g, k);
+  launch_pdl(k_l64_poly, dim3(nt, nt), DNT, 0, st, g, 4);
   return cudaGetLastError();
 }
 

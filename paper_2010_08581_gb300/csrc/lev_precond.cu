@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(GDNT) k_gram_dd(const float* __restrict__ Ah,
                                                   unsigned* __restrict__ cnt,
                                                   float* __restrict__ kh, float* __restrict__ kl,
                                                   int lda, double* __restrict__ k64) {
+  grid_wait();
   __shared__ float Ph[GDK][GD + 1], Pl[GDK][GD + 1];
   __shared__ float Qh[GDK][GD + 1], Ql[GDK][GD + 1];
   __shared__ int s_last;
@@ -190,6 +191,7 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_chol_inv(int n, float tol_sca
                                                             const float* __restrict__ pre,
                                                             int lda, float* __restrict__ Ximg,
                                                             int* __restrict__ state) {
+  grid_wait();
   __shared__ CiShared cs;
   const bool ok = chol_inv_tiles(n, tol_scale, pre, lda, Ximg, n + 1, pre, n, lda, cs);
   if (threadIdx.x == 0) *state = ok ? 0 : 1;
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(LT * LT) k_lev_u(int n, const float* __restric
                                                    const int* __restrict__ state,
                                                    float* __restrict__ Uh,
                                                    float* __restrict__ Ul, int ldu) {
+  grid_wait();
   __shared__ float Xt[kMaxPre][LT + 1];        // X[i0 + r][k] at Xt[k][r]
   __shared__ float Kth[kMaxPre][LT], Ktl[kMaxPre][LT];
   if (*state != 0) return;
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(LT * LT) k_lev_e(int n, const float* __restric
                                                    const int* __restrict__ state,
                                                    float* __restrict__ E, int lde,
                                                    float* __restrict__ esq) {
+  grid_wait();
   __shared__ float Uth[LT][kMaxPre + 1], Utl[LT][kMaxPre + 1];   // U[i0 + r][k]
   __shared__ float Xt[kMaxPre][LT + 1];                          // X[j0 + r][k] at Xt[k][r]
   __shared__ float red[LT * LT / 32];
@@ -334,6 +338,7 @@ __global__ void __launch_bounds__(LR_NT) k_lev_rows(int n, int64_t I, const floa
                                                     const float* __restrict__ esq, int nesq,
                                                     int* state, double* __restrict__ ell,
                                                     CdfEpilogue ep, float tau) {
+  grid_wait();
   extern __shared__ __align__(16) float lrs[];  // X image, then E (row stride lde)
   __shared__ float2 as[LR_ROWS][kMaxPre];     // (a_hi, a_lo)
   __shared__ float wv[LR_ROWS][kMaxPre];      // w (FP32), then v1, v2
@@ -545,7 +550,7 @@ cudaError_t launch_gram_dd(const float* Ah, const float* Al, int64_t I, int n, i
   int64_t chunk;
   const int splits = gram_dd_splits(I, &chunk);
   const int nt = (n + GD - 1) / GD;
-  k_gram_dd<<<dim3(nt * (nt + 1) / 2, splits), GDNT, 0, st>>>(Ah, Al, I, n, lda_a, chunk, splits,
+  launch_pdl(k_gram_dd, dim3(nt * (nt + 1) / 2, splits), GDNT, 0, st, Ah, Al, I, n, lda_a, chunk, splits,
                                                               ph, pl, cnt, kh, kl, lda, k64);
   return cudaGetLastError();
 }
@@ -566,21 +571,21 @@ cudaError_t launch_lev_precond(int stage, const LevPrecond& lp, int n, int64_t I
   switch (stage) {
     case 0: {
       const double eps32 = 1.1920928955078125e-07;
-      k_chol_inv<<<1, chol_inv_threads(n), 0, st>>>(n, static_cast<float>(n * eps32), lp.K_hi,
+      launch_pdl(k_chol_inv, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(n * eps32), lp.K_hi,
                                                     lp.lda_k, lp.Ximg, lp.state);
       return cudaGetLastError();
     }
     case 1:
-      k_lev_u<<<dim3(nt, nt), dim3(LT, LT), 0, st>>>(n, lp.K_hi, lp.K_lo, lp.lda_k, lp.Ximg,
+      launch_pdl(k_lev_u, dim3(nt, nt), dim3(LT, LT), 0, st, n, lp.K_hi, lp.K_lo, lp.lda_k, lp.Ximg,
                                                      lp.state, lp.Uh, lp.Ul, ld);
       return cudaGetLastError();
     case 2:
-      k_lev_e<<<lev_precond_ctas(n), dim3(LT, LT), 0, st>>>(n, lp.Uh, lp.Ul, ld, lp.Ximg,
+      launch_pdl(k_lev_e, lev_precond_ctas(n), dim3(LT, LT), 0, st, n, lp.Uh, lp.Ul, ld, lp.Ximg,
                                                            lp.state, lp.E, ld, lp.esq);
       return cudaGetLastError();
     case 3: {
       const unsigned rb = static_cast<unsigned>((I + LR_ROWS - 1) / LR_ROWS);
-      k_lev_rows<<<rb, LR_NT, lev_rows_smem(n), st>>>(n, I, Ah, Al, lda, lp.Ximg, lp.E, ld,
+      launch_pdl(k_lev_rows, rb, LR_NT, lev_rows_smem(n), st, n, I, Ah, Al, lda, lp.Ximg, lp.E, ld,
                                                         lp.esq, lev_precond_ctas(n), lp.state,
                                                         ell, ep, lp.tau);
       return cudaGetLastError();

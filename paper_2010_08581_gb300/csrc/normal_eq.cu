@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(tile_threads(BM) * tile_threads(BM)) k_normal_
                                                   int64_t I, int64_t chunk,
                                                   T* __restrict__ partial,
                                                   const int64_t* __restrict__ jdev) {
+  grid_wait();
   constexpr int BN = BM, TE = tile_threads(BM), NT = TE * TE, U = BM / TE, V = BN / TE;
   __shared__ T As[2][BK][BM];
   __shared__ T Bs[2][BK][BN];
@@ -124,9 +125,9 @@ template <typename T, int BM>
 void go(const void* A, const void* Y, int64_t J, int L, int64_t I, int64_t chunk, void* partial,
         int splits, cudaStream_t st, const int64_t* jdev) {
   const dim3 grid(static_cast<unsigned>((L + I + BM - 1) / BM), (L + BM - 1) / BM, splits);
-  k_normal_eq<T, BM><<<grid, tile_threads(BM) * tile_threads(BM), 0, st>>>(
-      static_cast<const T*>(A), static_cast<const T*>(Y), J, L, I, chunk, static_cast<T*>(partial),
-      jdev);
+  launch_pdl((k_normal_eq<T, BM>), grid, tile_threads(BM) * tile_threads(BM), 0, st,
+             static_cast<const T*>(A), static_cast<const T*>(Y), J, L, I, chunk,
+             static_cast<T*>(partial), jdev);
 }
 
 }  // namespace

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(NT, 2) k_normal_eq_tc(const float* __restrict_
                                                         float* __restrict__ partial,
                                                         unsigned* err, long long wait_limit,
                                                         const int64_t* __restrict__ jdev) {
+  grid_wait();
   constexpr uint32_t kIdesc = idesc_tf32(TM, TN);
   constexpr int B_BYTES = TN * TK * 4;
   constexpr int STAGE_BYTES = stage_bytes<TN>();
@@ -305,8 +306,8 @@ cudaError_t launch_tn(const float* A, const float* Y, int64_t J, int L, int64_t 
                       int64_t chunk, int splits, float* partial, unsigned* err, cudaStream_t st,
                       long long wait_limit, const int64_t* jdev) {
   dim3 grid(static_cast<unsigned>((L + I + TN - 1) / TN), (L + TM - 1) / TM, splits);
-  k_normal_eq_tc<TN, kDense><<<grid, NT, STAGES * stage_bytes<TN>() + 1024, st>>>(
-      A, Y, J, L, I, post, chunk, partial, err, wait_limit < 0 ? kTcSpinLimit : wait_limit, jdev);
+  launch_pdl((k_normal_eq_tc<TN, kDense>), grid, NT, STAGES * stage_bytes<TN>() + 1024, st, A, Y, J,
+             L, I, post, chunk, partial, err, wait_limit < 0 ? kTcSpinLimit : wait_limit, jdev);
   return cudaGetLastError();
 }
 

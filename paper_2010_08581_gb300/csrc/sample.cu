@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(FW * 32) k_sample_chain(SampleArgs sa, ChainAr
                                                           T* __restrict__ A, int staged,
                                                           GatherArgs ga, const TX* __restrict__ X,
                                                           T* __restrict__ Y) {
+  grid_wait();
   extern __shared__ __align__(16) double fused_smem[];
   __shared__ T sS[FW][kMaxL];
   __shared__ T sG[FW][kMaxL];
@@ -184,7 +185,7 @@ void run_sample_chain(unsigned blocks, size_t dyn, cudaStream_t st, const Sample
                       const ChainArgs& ca, int64_t J, uint32_t k0, uint32_t k1, uint32_t u0,
                       uint32_t u1, int32_t* idx, double* w, void* A, int staged,
                       const GatherArgs& ga, const void* X, void* Y) {
-  k_sample_chain<T, TX><<<blocks, FW * 32, dyn, st>>>(sa, ca, J, k0, k1, u0, u1, idx, w,
+  launch_pdl((k_sample_chain<T, TX>), blocks, FW * 32, dyn, st, sa, ca, J, k0, k1, u0, u1, idx, w,
                                                       static_cast<T*>(A), staged, ga,
                                                       static_cast<const TX*>(X),
                                                       static_cast<T*>(Y));

@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(IW * 32) k_tri_inv(int n, const float* __restr
                                                      const int* __restrict__ info,
                                                      float* __restrict__ Wimg,
                                                      const int* __restrict__ skip_if) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char ism[];
   if (*info != 0 || (skip_if && *skip_if)) return;
   const int np = n + 1;
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(SNT) k_solve_inv(int n, const float* __restric
                                                    const int* __restrict__ info, int64_t nvec,
                                                    const double* __restrict__ rhs, int64_t ld,
                                                    int Rl, int Rr, double* __restrict__ core_out) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char ssm[];
   if (*info != 0) return;
   const int np = n + 1;
@@ -193,15 +195,15 @@ cudaError_t launch_solve_inv(int n, const float* Limg, const float* Mimg,
   if (nvec <= 0) return cudaSuccess;
   const unsigned ib = static_cast<unsigned>((n + IW - 1) / IW);
   switch ((n + 31) / 32) {
-    case 1: k_tri_inv<1><<<ib, IW * 32, inv_smem(n), st>>>(n, Limg, invdiag, info, Wimg, fast); break;
-    case 2: k_tri_inv<2><<<ib, IW * 32, inv_smem(n), st>>>(n, Limg, invdiag, info, Wimg, fast); break;
-    case 3: k_tri_inv<3><<<ib, IW * 32, inv_smem(n), st>>>(n, Limg, invdiag, info, Wimg, fast); break;
-    default: k_tri_inv<4><<<ib, IW * 32, inv_smem(n), st>>>(n, Limg, invdiag, info, Wimg, fast); break;
+    case 1: launch_pdl(k_tri_inv<1>, ib, IW * 32, inv_smem(n), st, n, Limg, invdiag, info, Wimg, fast); break;
+    case 2: launch_pdl(k_tri_inv<2>, ib, IW * 32, inv_smem(n), st, n, Limg, invdiag, info, Wimg, fast); break;
+    case 3: launch_pdl(k_tri_inv<3>, ib, IW * 32, inv_smem(n), st, n, Limg, invdiag, info, Wimg, fast); break;
+    default: launch_pdl(k_tri_inv<4>, ib, IW * 32, inv_smem(n), st, n, Limg, invdiag, info, Wimg, fast); break;
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned sb = static_cast<unsigned>((nvec + SNR - 1) / SNR);
-  k_solve_inv<<<sb, SNT, solve_smem_bytes(n), st>>>(n, Wimg, Mimg, info, nvec, rhs, ld, Rl, Rr,
+  launch_pdl(k_solve_inv, sb, SNT, solve_smem_bytes(n), st, n, Wimg, Mimg, info, nvec, rhs, ld, Rl, Rr,
                                                      core_out);
   return cudaGetLastError();
 }

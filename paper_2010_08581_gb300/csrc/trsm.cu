@@ -12,6 +12,7 @@ __global__ void __launch_bounds__(TNT) k_trsm(int n, const double* __restrict__ 
                                               const float* __restrict__ Mimg, int Rl, int Rr,
                                               double* __restrict__ core_out,
                                               double* __restrict__ ell, CdfEpilogue ep) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char trsm_smem[];
   subst_cta<T, NV, VP, PB>(trsm_smem, blockIdx.x, n, invdiag, info, nvec, rhs, ld, mode, Limg, Mimg,
                        Rl, Rr, core_out, ell, ep, gridDim.x);
@@ -28,8 +29,8 @@ cudaError_t run(int n, const double* invdiag, const int* info, int64_t nvec, con
   const unsigned blocks = static_cast<unsigned>((nvec + nv - 1) / nv);
   const size_t dyn = subst_smem<T>(n, nv, panel_cols<T>(few));
 #define TRSM_GO(NV, VP, FEW)                                                                     \
-  k_trsm<T, NV, VP, panel_cols<T>(FEW)><<<blocks, TNT, dyn, st>>>(n, invdiag, info, nvec, rhs, ld, mode, Limg, Mimg, \
-                                              Rl, Rr, core_out, ell, ep)
+  launch_pdl((k_trsm<T, NV, VP, panel_cols<T>(FEW)>), blocks, TNT, dyn, st, n, invdiag, info,     \
+             nvec, rhs, ld, mode, Limg, Mimg, Rl, Rr, core_out, ell, ep)
 #define TRSM_8(VP) TRSM_GO(8, VP, false)
 #define TRSM_4(VP) TRSM_GO(4, (VP > 1 ? VP / 2 : 1), false)
 #define TRSM_FEW(VP) TRSM_GO(4, (VP > 1 ? VP / 2 : 1), true)

@@ -246,10 +246,10 @@ __global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
 //   pass 2 (wide modes only): G2 = C^T C (I x I), C = the pass-1 factor.
 // ------------------------------------------------------------------------------------
 constexpr int GK = 16, GNT = 256;
-constexpr int GM = 2;                 // 2 x 2 blocks of G per thread
+constexpr int GM = 2;                 // 2 x 2 blocks of G per thread, at most
 
-// The 2 x 2 blocks of G's upper triangle, row by row, are dealt out to the threads (and, beyond
-// GNT * GM of them, to the CTAs of blockIdx.y), GK rows of the matrix at a time in shared memory;
+// The 2 x 2 blocks of G's upper triangle, row by row, are dealt out to the CTAs of blockIdx.y, `per`
+// each, and their threads, GK rows of the matrix at a time in shared memory;
 // the lower triangle is written by its mirror image. The FP64 pipe is the bound, so there is no
 // work on padding beyond the last warp: 32 x 32 tiles of the whole square took 174 .. 310 us for
 // 512 cores of L = 9 .. 64, I = 32 .. 200. Every entry is one chain over the rows
@@ -257,7 +257,7 @@ constexpr int GM = 2;                 // 2 x 2 blocks of G per thread
 __host__ __device__ inline int gram_blocks(int n) { const int h = (n + 1) / 2; return h * (h + 1) / 2; }
 
 __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, int step, int init_k,
-                                               int pass, int from_core) {
+                                               int pass, int from_core, int per) {
   __shared__ __align__(16) double P[GK * kMaxL];
   const BInst& d = tab[blockIdx.x];
   const Cur cu = current(d, step, init_k, true);
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, in
     n = static_cast<int>(cu.I); K = cu.I; trans = false;
   }
   const int h = (n + 1) / 2, blocks = gram_blocks(n);
-  const int parts = (blocks + GNT * GM - 1) / (GNT * GM);
+  const int parts = (blocks + per - 1) / per;
   if (static_cast<int>(blockIdx.y) >= parts) return;
   const int b0 = static_cast<int>(static_cast<int64_t>(blocks) * blockIdx.y / parts);
   const int b1 = static_cast<int>(static_cast<int64_t>(blocks) * (blockIdx.y + 1) / parts);
@@ -373,8 +373,11 @@ cudaError_t bl_contract(const BLaunch& b, int step, cudaStream_t st) {
 cudaError_t bl_gram(const BLaunch& b, int step, int init_k, int pass, cudaStream_t st) {
   const int nmax = pass == 1 ? b.n1max : b.n2max;
   if (nmax <= 0) return cudaSuccess;
-  dim3 grid(b.count, (gram_blocks(nmax) + GNT * GM - 1) / (GNT * GM));
-  kb_gram<<<grid, GNT, 0, st>>>(b.tab, step, init_k, pass, b.ls_mode == 1 ? 1 : 0);
+  // all that a CTA's threads hold, or, where the problems alone do not fill the SMs, two warps'
+  // worth: one SM's FP64 pipe takes 150 us for 512 blocks of 300 rows, 19 us for 64
+  const int per = b.count >= 2 * sm_count() ? GNT * GM : 64;
+  dim3 grid(b.count, (gram_blocks(nmax) + per - 1) / per);
+  kb_gram<<<grid, GNT, 0, st>>>(b.tab, step, init_k, pass, b.ls_mode == 1 ? 1 : 0, per);
   return cudaGetLastError();
 }
 

@@ -51,13 +51,15 @@ typedef enum tr_status {
 typedef enum tr_dtype { TR_F32 = 0, TR_F64 = 1 } tr_dtype;
 
 /* Arithmetic of the least-squares step (rows a3-a6) and of the drivers' distributions.
- * TR_PREC_FP64 : design rows, fibres, contractions, Cholesky and solves in FP64.
+ * TR_PREC_FP64 : design rows, fibres, contractions, Cholesky and solves in FP64 (from L = 88
+ *                on through X' = (X M X^T)^-1/2 X, X an FP32 inverse of M's Cholesky factor,
+ *                every product in FP64; the FP64 factorisation when X is too poor for it).
  * TR_PREC_MIXED: design rows and fibres in FP32, contractions with FP32 accumulation.
  *                The normal matrix is factored in FP32 when every pivot exceeds
  *                L*eps32*max diag, else in FP64 (same singular rule as TR_PREC_FP64);
  *                FP32 solves (for L <= 128 products by the factor's FP32 inverse, formed
- *                together with the FP32 factor in one pass; triangular substitutions
- *                otherwise) and one step of iterative refinement against the
+ *                together with the FP32 factor in one pass, for L > 160 by blocks;
+ *                triangular substitutions otherwise) and one step of iterative refinement against the
  *                FP32-accurate normal-equation residual. In the drivers, the leverage
  *                scores of a tall matrix (I >= L, 4 <= L <= 128) are those of
  *                tr_leverage_planes: an FP32 Cholesky preconditioner of the double-float
@@ -110,7 +112,8 @@ tr_status tr_status_sync(tr_ctx* ctx, tr_stream stream);
  * above max(I,L)*eps*sigma_max (the rule of a singular value decomposition); otherwise from
  * a Cholesky-based thin QR of G_(2) (or of G_(2)^T when I < L), with dependent columns
  * dropped at pivot <= max(I,L)*eps*max diag, which resolves singular values down to about
- * sqrt(max(I,L)*eps)*sigma_max. The drivers form every distribution the same way.
+ * sqrt(max(I,L)*eps)*sigma_max (I >= L >= 88 with every FP32 pivot above L*eps32*max diag: by FP64
+ * products with X' of TR_PREC_FP64 above, which resolves as much). The drivers form every distribution the same way.
  * A zero core records TR_ERR_SINGULAR and yields the uniform distribution. */
 tr_status tr_leverage(tr_ctx* ctx, const double* core, int64_t I, int Rl, int Rr,
                       double* p, double* cdf, tr_stream stream);

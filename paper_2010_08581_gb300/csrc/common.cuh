@@ -386,8 +386,8 @@ cudaError_t launch_init_normal(double* out, int64_t count, uint64_t seed, uint32
 // A kernel of a chain, launched while its predecessor on the stream still runs (programmatic
 // dependent launch): its blocks are scheduled when the predecessor's last ones are, and wait in
 // grid_wait for the predecessor's results. The update's chains are a dozen short kernels, each of
-// which otherwise starts with about 2 us of launch and drain (update of 40^3 in FP64: 141 -> 122 us,
-// of 500^3: 524 -> 446). Every kernel launched this way calls grid_wait before anything else, so
+// which otherwise starts with about 2 us of launch and drain (update of 40 x 30 x 20 in FP64: 141 -> 116 us,
+// of 500^3: 522 -> 443). Every kernel launched this way calls grid_wait before anything else, so
 // that the completion of one implies that of all before it. Not while a graph is captured: there
 // the chains ran 2 % slower with such edges (500^3, ten sweeps: 4.95 -> 5.06 ms).
 template <typename... P, typename... A>

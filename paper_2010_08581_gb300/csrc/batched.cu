@@ -245,8 +245,7 @@ __global__ void __launch_bounds__((TILE / 4) * (TILE / 4)) kb_contract(
 //           update; B^T during the updates otherwise);
 //   pass 2 (wide modes only): G2 = C^T C (I x I), C = the pass-1 factor.
 // ------------------------------------------------------------------------------------
-constexpr int GK = 16, GNT = 256;
-constexpr int GM = 2;                 // 2 x 2 blocks of G per thread, at most
+constexpr int GK = 16, GNT = 256;     // a thread holds at most one 2 x 2 block; all of them load
 
 // The 2 x 2 blocks of G's upper triangle, row by row, are dealt out to the CTAs of blockIdx.y, `per`
 // each, and their threads, GK rows of the matrix at a time in shared memory;
@@ -284,19 +283,13 @@ __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, in
   const int b0 = static_cast<int>(static_cast<int64_t>(blocks) * blockIdx.y / parts);
   const int b1 = static_cast<int>(static_cast<int64_t>(blocks) * (blockIdx.y + 1) / parts);
   const int ld = 2 * h;               // an even row length: aligned pairs
-  int row[GM], col[GM];
-  double acc[GM][2][2] = {};
-#pragma unroll
-  for (int q = 0; q < GM; ++q) {
-    int rest = b0 + static_cast<int>(threadIdx.x) + GNT * q;
-    row[q] = -1;
-    col[q] = 0;
-    if (rest < b1) {
-      int r = 0;
-      while (rest >= h - r) { rest -= h - r; ++r; }
-      row[q] = 2 * r;
-      col[q] = 2 * (r + rest);
-    }
+  int row = -1, col = 0, rest = b0 + static_cast<int>(threadIdx.x);
+  double acc[2][2] = {};
+  if (rest < b1) {
+    int r = 0;
+    while (rest >= h - r) { rest -= h - r; ++r; }
+    row = 2 * r;
+    col = 2 * (r + rest);
   }
   for (int64_t kb = 0; kb < K; kb += GK) {
     for (int e = threadIdx.x; e < GK * ld; e += GNT) {
@@ -306,34 +299,29 @@ __global__ void __launch_bounds__(GNT) kb_gram(const BInst* __restrict__ tab, in
       P[kk * ld + c] = k < K && c < n ? (trans ? src[c * lda + k] : src[k * lda + c]) : 0.0;
     }
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < GM; ++q) {
-      if (row[q] < 0) continue;
+    if (row >= 0) {
 #pragma unroll 4
       for (int kk = 0; kk < GK; ++kk) {
-        const double2 x = *reinterpret_cast<const double2*>(P + kk * ld + row[q]);
-        const double2 y = *reinterpret_cast<const double2*>(P + kk * ld + col[q]);
-        acc[q][0][0] += x.x * y.x;
-        acc[q][0][1] += x.x * y.y;
-        acc[q][1][0] += x.y * y.x;
-        acc[q][1][1] += x.y * y.y;
+        const double2 x = *reinterpret_cast<const double2*>(P + kk * ld + row);
+        const double2 y = *reinterpret_cast<const double2*>(P + kk * ld + col);
+        acc[0][0] += x.x * y.x;
+        acc[0][1] += x.x * y.y;
+        acc[1][0] += x.y * y.x;
+        acc[1][1] += x.y * y.y;
       }
     }
     __syncthreads();
   }
+  if (row < 0) return;
 #pragma unroll
-  for (int q = 0; q < GM; ++q) {
-    if (row[q] < 0) continue;
+  for (int u = 0; u < 2; ++u)
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        const int r = row[q] + u, c = col[q] + v;
-        if (r >= n || c >= n) continue;
-        G[static_cast<int64_t>(r) * n + c] = acc[q][u][v];
-        G[static_cast<int64_t>(c) * n + r] = acc[q][u][v];
-      }
-  }
+    for (int v = 0; v < 2; ++v) {
+      const int r = row + u, c = col + v;
+      if (r >= n || c >= n) continue;
+      G[static_cast<int64_t>(r) * n + c] = acc[u][v];
+      G[static_cast<int64_t>(c) * n + r] = acc[u][v];
+    }
 }
 
 }  // namespace
@@ -373,9 +361,10 @@ cudaError_t bl_contract(const BLaunch& b, int step, cudaStream_t st) {
 cudaError_t bl_gram(const BLaunch& b, int step, int init_k, int pass, cudaStream_t st) {
   const int nmax = pass == 1 ? b.n1max : b.n2max;
   if (nmax <= 0) return cudaSuccess;
-  // all that a CTA's threads hold, or, where the problems alone do not fill the SMs, two warps'
-  // worth: one SM's FP64 pipe takes 150 us for 512 blocks of 300 rows, 19 us for 64
-  const int per = b.count >= 2 * sm_count() ? GNT * GM : 64;
+  // 128 blocks a CTA, 64 where the problems alone do not fill the SMs: one SM's FP64 pipe takes
+  // 150 us for 512 blocks of 300 rows, 19 us for 64, and the largest problems of a batch end last
+  // (512 problems: 180 us with 512 blocks, 135 with 128)
+  const int per = b.count >= 2 * sm_count() ? 128 : 64;
   dim3 grid(b.count, (gram_blocks(nmax) + per - 1) / per);
   kb_gram<<<grid, GNT, 0, st>>>(b.tab, step, init_k, pass, b.ls_mode == 1 ? 1 : 0, per);
   return cudaGetLastError();

@@ -7,6 +7,12 @@ namespace trk {
 namespace {
 
 constexpr int BNV = 8;              // vectors per CTA
+// Columns per panel: in FP64 and up to 64 unknowns 8, so that a warp solves the diagonal blocks of
+// four vectors at once: with many CTAs per SM the FP64 pipe is the bound, where a warp's instruction
+// takes 16 clocks however few lanes matter (rows of 512 problems: 250 us with 16 columns, 227 with
+// 8). Beyond, where a few large problems have the SMs to themselves, fewer panels count.
+template <typename T>
+constexpr int batch_cols(int vp) { return sizeof(T) == 4 ? 32 : (vp <= 2 ? 8 : 16); }
 
 template <typename T>
 __device__ __forceinline__ void subst_any(unsigned char* sm, int64_t cta, int n,
@@ -15,7 +21,7 @@ __device__ __forceinline__ void subst_any(unsigned char* sm, int64_t cta, int n,
                                           const float* Mimg, int Rl, int Rr, double* core_out,
                                           double* ell, const CdfEpilogue& ep, int nctas) {
 #define SUBST_GO(VP)                                                                          \
-  subst_cta<T, BNV, VP, panel_cols<T>(false)>(sm, cta, n, invdiag, info, nvec, rhs, ld, mode, Limg, Mimg, Rl, Rr,   \
+  subst_cta<T, BNV, VP, batch_cols<T>(VP)>(sm, cta, n, invdiag, info, nvec, rhs, ld, mode, Limg, Mimg, Rl, Rr,   \
                         core_out, ell, ep, nctas)
   TRK_SUBST_DISPATCH(n, SUBST_GO);
 #undef SUBST_GO
@@ -52,7 +58,7 @@ __global__ void __launch_bounds__(TNT) kb_rows(const BInst* __restrict__ tab, in
 }
 
 template <typename T>
-size_t smem(int n) { return subst_smem<T>(n, BNV, panel_cols<T>(false)); }
+size_t smem(int n) { return subst_smem<T>(n, BNV, batch_cols<T>(8)); }
 unsigned ctas(int64_t I) { return static_cast<unsigned>((I + BNV - 1) / BNV); }
 
 }  // namespace

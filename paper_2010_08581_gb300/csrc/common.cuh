@@ -310,8 +310,8 @@ cudaError_t launch_solve_big(int n, const float* Wimg, const float* Mimg, const 
                              double* core_out, float* scratch, int64_t rows, cudaStream_t st);
 
 // FP64 leverage scores of a tall I x n matrix A (row stride lda) through an FP32 inverse of the
-// Gram's factor (lev64.cu): ell, then p and the CDF as launch_trsm's epilogue (ep.counter 0
-// before and after). part 0: everything up to the rows; 1: the rows (reads ep.skip). When the
+// Gram's factor (lev64.cu): ell, then p and the CDF as launch_trsm's epilogue (ep.counter is not
+// used). part 0: everything up to the rows; 1: the rows (reads ep.skip). When the
 // FP32 factorisation fails or ||E||_F > tau nothing is written and bad[1] = 1: the caller's
 // fallback launches are gated on it. For the sizes leverage_f64_fits accepts (splits: of
 // gram_workspace, whose partials' room serves as scratch).

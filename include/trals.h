@@ -51,9 +51,12 @@ typedef enum tr_status {
 typedef enum tr_dtype { TR_F32 = 0, TR_F64 = 1 } tr_dtype;
 
 /* Arithmetic of the least-squares step (rows a3-a6) and of the drivers' distributions.
- * TR_PREC_FP64 : design rows, fibres, contractions, Cholesky and solves in FP64 (from L = 88
- *                on through X' = (X M X^T)^-1/2 X, X an FP32 inverse of M's Cholesky factor,
- *                every product in FP64; the FP64 factorisation when X is too poor for it).
+ * TR_PREC_FP64 : design rows, fibres, contractions, Cholesky and solves in FP64. From L = 88 on
+ *                the solves take V = X'^T X', X' = (X M X^T)^-1/2 X and X an FP32 inverse of M's
+ *                Cholesky factor, and one step of refinement, every product in FP64: z = V b,
+ *                z += V (b - M z), whose residual is no larger than that of a factorisation
+ *                (||b - M z|| <= 1.5 * 2^-53 ||M|| ||z|| in the tests); the FP64 factorisation
+ *                when X is too poor for it.
  * TR_PREC_MIXED: design rows and fibres in FP32, contractions with FP32 accumulation.
  *                The normal matrix is factored in FP32 when every pivot exceeds
  *                L*eps32*max diag, else in FP64 (same singular rule as TR_PREC_FP64);

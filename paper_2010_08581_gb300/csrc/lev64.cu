@@ -4,7 +4,9 @@
 //     identity of lev_precond.cu), K^-1 = X'^T X' for X' = C^-1/2 X, so ell_i = ||X' a_i||^2. Every
 //     product is in FP64 and C^-1/2 is its binomial series in E, through E^3 for
 //     ||E||_F <= 1e-4, E^5 up to 1e-3 and E^7 up to 1e-2: a remainder below 3e-17 each time;
-//   * the FP64 LS step (row a6): z = M^-1 b = X'^T (X' b) with the same X' of M;
+//   * the FP64 LS step (row a6): z = V b with V = M^-1 = X'^T X' and the same X' of M, then one step
+//     of refinement, r = b - M z, z += V r: E carries a rounding of eps cond(M), which the products
+//     alone would take into z as cond(M)^1/2 times that;
 //   * the mixed-precision LS step's solves (row a6) for 160 < L <= 256.
 //
 // Why: one SM multiplies two FP64 pairs per clock, so the one-CTA FP64 factorisation of a 256 x
@@ -191,8 +193,8 @@ struct Panels {
 
 // ep(i, j, sum over kb <= k < ke of a(i, k) * b(k, j)) for the tile at (i0, j0), by the first
 // warp: lane = 4 * row + column pair. kAk / kBk: a (b) is contiguous in k. Each warp sums half of
-// the terms.
-template <bool kAk, bool kBk, typename A, typename B, typename Ep>
+// the terms, in runs of kRun (even).
+template <bool kAk, bool kBk, int kRun = DLD, typename A, typename B, typename Ep>
 __device__ __forceinline__ void tile8(Panels& sm, int i0, int j0, int kb, int ke, A a, B b, Ep ep) {
   const int t = threadIdx.x, kn = ke - kb, kp = (kn + 3) & ~3;    // padded with zeros to a half
   if constexpr (kAk) {
@@ -210,15 +212,23 @@ __device__ __forceinline__ void tile8(Panels& sm, int i0, int j0, int kb, int ke
   __syncthreads();
   const int warp = t >> 5, lane = t & 31, r = lane >> 2, c = 2 * (lane & 3);
   double x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
+  const int k1 = (warp + 1) * (kp / 2);
+  for (int kr = warp * (kp / 2); kr < k1; kr += kRun) {
+    double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
 #pragma unroll 4
-  for (int k = warp * (kp / 2); k < (warp + 1) * (kp / 2); k += 2) {
-    const double2 u = *reinterpret_cast<const double2*>(&sm.a[r][k]);
-    const double2 v = *reinterpret_cast<const double2*>(&sm.b[c][k]);
-    const double2 w = *reinterpret_cast<const double2*>(&sm.b[c + 1][k]);
-    x0 += u.x * v.x;
-    y0 += u.x * w.x;
-    x1 += u.y * v.y;
-    y1 += u.y * w.y;
+    for (int k = kr; k < min(kr + kRun, k1); k += 2) {
+      const double2 u = *reinterpret_cast<const double2*>(&sm.a[r][k]);
+      const double2 v = *reinterpret_cast<const double2*>(&sm.b[c][k]);
+      const double2 w = *reinterpret_cast<const double2*>(&sm.b[c + 1][k]);
+      p0 += u.x * v.x;
+      q0 += u.x * w.x;
+      p1 += u.y * v.y;
+      q1 += u.y * w.y;
+    }
+    x0 += p0;
+    y0 += q0;
+    x1 += p1;
+    y1 += q1;
   }
   x0 += x1;
   y0 += y1;
@@ -404,31 +414,60 @@ __global__ void __launch_bounds__(kFinishThreads) k_l64_finish(L64 g, const doub
   if (ep.p) cdf_epilogue_nw<kFinishThreads / 32>(ep, ell, I);
 }
 
-// The FP64 LS step: y = X' b for `rows` right-hand sides (rows of B^T), then z = X'^T y into the
-// new core.
-__global__ void __launch_bounds__(DNT) k_l64_y(L64 g, const double* __restrict__ b, int64_t ld,
-                                               int rows, double* __restrict__ y) {
+// The FP64 LS step: V = X'^T X' into E2's place (the tiles of the upper triangle, both written).
+// z = X'^T (X' b) twice would be five products of a right-hand side instead of three and two
+// launches more (L = 256, 300 right-hand sides: 314 us a solve, 242 with V).
+__global__ void __launch_bounds__(DNT) k_l64_inv(L64 g) {
+  grid_wait();
+  __shared__ __align__(16) Panels sm;
+  if (g.flag[0] || g.flag[2] == 0) return;
+  const int n = g.n;
+  int i0, j0;
+  upper_tile(blockIdx.x, (n + DE - 1) / DE, i0, j0);
+  tile8<false, false>(sm, i0, j0, 0, n, [&](int i, int k) { return i < n ? g.T[k * n + i] : 0.0; },
+      [&](int k, int j) { return j < n ? g.T[k * n + j] : 0.0; },
+      [&](int i, int j, double v) {
+        if (i >= n || j >= n || i > j) return;
+        g.U[i * n + j] = v;
+        g.U[j * n + i] = v;
+      });
+}
+
+// The place of unknown k in a row of the core.
+__device__ __forceinline__ int core_entry(int k, int Rl, int Rr) { return (k % Rl) * Rr + k / Rl; }
+
+// z = V b for `rows` right-hand sides (rows of b) into the new core, or z there + V b (add).
+__global__ void __launch_bounds__(DNT) k_l64_z(L64 g, const double* __restrict__ b, int64_t ld,
+                                               int rows, int Rl, int Rr, double* __restrict__ core,
+                                               bool add) {
   grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0] || g.flag[2] == 0) return;
   const int n = g.n;
   tile8<true, true>(sm, blockIdx.y * DE, blockIdx.x * DE, 0, n,
       [&](int i, int k) { return i < rows ? b[i * ld + k] : 0.0; },
-      [&](int k, int j) { return j < n ? g.T[j * n + k] : 0.0; },
-      [&](int i, int j, double v) { if (i < rows && j < n) y[static_cast<int64_t>(i) * n + j] = v; });
+      [&](int k, int j) { return j < n ? g.U[j * n + k] : 0.0; },
+      [&](int i, int j, double v) {
+        if (i >= rows || j >= n) return;
+        double* at = core + static_cast<int64_t>(i) * n + core_entry(j, Rl, Rr);
+        *at = add ? *at + v : v;
+      });
 }
 
-__global__ void __launch_bounds__(DNT) k_l64_z(L64 g, const double* __restrict__ y, int rows, int Rl,
-                                               int Rr, double* __restrict__ core) {
+// r = b - M z, summed in runs of 16 terms: the rounding of r is what is left in the result, and
+// one chain of 256 terms carries about twice as much of it.
+__global__ void __launch_bounds__(DNT) k_l64_r(L64 g, const double* __restrict__ b, int64_t ld,
+                                               int rows, int Rl, int Rr,
+                                               const double* __restrict__ core, double* __restrict__ r) {
   grid_wait();
   __shared__ __align__(16) Panels sm;
   if (g.flag[0] || g.flag[2] == 0) return;
   const int n = g.n;
-  tile8<true, false>(sm, blockIdx.y * DE, blockIdx.x * DE, 0, n,
-      [&](int i, int k) { return i < rows ? y[static_cast<int64_t>(i) * n + k] : 0.0; },
-      [&](int k, int j) { return j < n ? g.T[k * n + j] : 0.0; },
+  tile8<true, false, 16>(sm, blockIdx.y * DE, blockIdx.x * DE, 0, n,
+      [&](int i, int k) { return i < rows ? core[static_cast<int64_t>(i) * n + core_entry(k, Rl, Rr)] : 0.0; },
+      [&](int k, int j) { return j < n ? (k <= j ? g.G[k * n + j] : g.G[j * n + k]) : 0.0; },
       [&](int i, int j, double v) {
-        if (i < rows && j < n) core[static_cast<int64_t>(i) * n + (j % Rl) * Rr + j / Rl] = v;
+        if (i < rows && j < n) r[static_cast<int64_t>(i) * n + j] = b[i * ld + j] - v;
       });
 }
 
@@ -573,25 +612,29 @@ cudaError_t launch_solve_big(int n, const float* Wimg, const float* Mimg, const 
   return cudaGetLastError();
 }
 
-// (The same line for the FP64 LS step, with the gated launches: L = 64, 300 right-hand sides: 114 ->
-// 117 us, L = 100: 210 -> 162, L = 256: 2430 -> 410.)
+// (The same line for the FP64 LS step, whole calls of 30 right-hand sides, J = 9 L, substitutions
+// against V: L = 88: 210 -> 188 us, L = 100: 253 -> 203, L = 256: 2645 -> 563; L = 81 was equal.)
+// A right-hand side costs three products here and one in the substitutions, which many of them keep
+// busy: the forms break even at about 550 right-hand sides for L = 88 and 90, 830 for 100, 900 for
+// 121, 1160 for 144, and, where the factor no longer fits one SM's shared memory, 2260 for 169, 3400
+// for 196, 5400 for 225 and 8600 for 256 (I = 1000: L = 90: 349 us by substitutions, 384 with V,
+// L = 169: 1194 and 997; I = 10000: L = 256: 13.8 and 14.1 ms).
 bool solve_f64_fits(int64_t I, int n, int splits) {
-  return n >= kLev64MinN && n <= kMaxL &&
+  return n >= kLev64MinN && n <= kMaxL && I <= (n > kSolveBigMin ? 12 : 6) * n &&
          static_cast<int64_t>(splits) * (n + I) >= 3 * static_cast<int64_t>(n) + 1;
 }
 
 cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t ld, int64_t I, int Rl,
                              int Rr, double* core_out, cudaStream_t st) {
   const L64 g = args_of(w, n);
-  double* y = w.partial + 3 * static_cast<size_t>(n) * n;
-  int64_t rows = static_cast<int64_t>(w.splits) * (n + I) - 3 * static_cast<int64_t>(n);
-  if (rows > kMaxRows) rows = kMaxRows;
-  for (int64_t r0 = 0; r0 < I; r0 += rows) {
-    const int m = static_cast<int>(I - r0 < rows ? I - r0 : rows);
-    const dim3 grid(dtiles(n), dtiles(m));
-    launch_pdl(k_l64_y, grid, DNT, 0, st, g, rhs + r0 * ld, ld, m, y);
-    launch_pdl(k_l64_z, grid, DNT, 0, st, g, y, m, Rl, Rr, core_out + r0 * n);
-  }
+  const unsigned nt = dtiles(n);
+  launch_pdl(k_l64_inv, nt * (nt + 1) / 2, DNT, 0, st, g);
+  double* r = g.P;        // behind V: room for splits * (n + I) - n >= I rows
+  const int m = static_cast<int>(I);
+  const dim3 grid(nt, dtiles(m));
+  launch_pdl(k_l64_z, grid, DNT, 0, st, g, rhs, ld, m, Rl, Rr, core_out, false);
+  launch_pdl(k_l64_r, grid, DNT, 0, st, g, rhs, ld, m, Rl, Rr, core_out, r);
+  launch_pdl(k_l64_z, grid, DNT, 0, st, g, r, static_cast<int64_t>(n), m, Rl, Rr, core_out, true);
   return cudaGetLastError();
 }
 

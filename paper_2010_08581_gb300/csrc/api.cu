@@ -1703,19 +1703,22 @@ tr_status tr_rel_error(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, cons
   int blocks;
   const bool xf64 = X_dtype == TR_F64;
   size_t tables;
-  size_t bytes = fit_workspace(fa, xf64, false, &blocks, &tables);
+  FitRoom room = kFitRoomy;
+  size_t bytes = fit_workspace(fa, xf64, room, &blocks, &tables);
   auto no_room = [&](size_t b) {
     return ctx->budget && b > ctx->arena_bytes && b + ctx->host_stage_bytes > ctx->budget;
   };
-  // the slice tables, and then the faster form's larger workspace, only where the budget leaves
-  // room for them
+  // the slice tables, a partial sum per CTA and the tensor cores' operand of W, each only where the
+  // budget leaves room for it
   if (no_room(bytes + tables)) tables = 0;
-  const bool tight = no_room(bytes);
-  if (tight) bytes = fit_workspace(fa, xf64, true, &blocks, &tables);
+  while (no_room(bytes) && room != kFitLeast) {
+    room = room == kFitRoomy ? kFitTight : kFitLeast;
+    bytes = fit_workspace(fa, xf64, room, &blocks, &tables);
+  }
   TR_TRY(ensure_ws(ctx, bytes + tables));
   double* partial = reinterpret_cast<double*>(ctx->arena);
   cudaStream_t st = S(stream);
-  TR_LAUNCH("fit", launch_fit(fa, X, xf64, tight, ctx->arena, blocks,
+  TR_LAUNCH("fit", launch_fit(fa, X, xf64, room, ctx->arena, blocks,
                               tables ? reinterpret_cast<float*>(ctx->arena + bytes) : nullptr,
                               ctx->d_err, st));
   std::vector<double> h(2 * static_cast<size_t>(blocks));

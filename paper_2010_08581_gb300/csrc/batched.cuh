@@ -76,7 +76,7 @@ struct BInst {
   SlotState* slot;
   double* fitp;                  // 2 * kFitParts partial sums of the fit evaluation
   void* fitw;                    // right factors of the fit's mode split (X's precision)
-  int fit_plain;                 // 1: FP32 X on the fit's FP64 form (fit_body.cuh)
+  int fit_plain;                 // 1: FP32 X on the fit's FP64 form, for want of room (fit_body.cuh)
   double* hist;                  // kMaxServedSweeps fits, one per completed sweep
 };
 

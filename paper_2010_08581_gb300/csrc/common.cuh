@@ -429,12 +429,14 @@ struct FitArgs {
   int ranks[kMaxModes];
   int N;
 };
-// Workspace: 2 * blocks partial sums, then the right factors of the mode split; tight: the form
-// and the blocks that need the least. FP32 slice
-// tables (table_bytes, launch_fit's `tables`) are optional: without them FP32 X reads the
-// FP64 cores, which is slower.
-size_t fit_workspace(const FitArgs& a, bool x_f64, bool tight, int* blocks, size_t* table_bytes);
-cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, bool tight, void* ws,
+// Workspace: 2 * blocks partial sums, then the right factors of the mode split. FP32 slice tables
+// (table_bytes, launch_fit's `tables`) are optional: without them FP32 X reads the FP64 cores, which
+// is slower. kFitTight: no more partial sums than one per row block (a few KB less); kFitLeast: FP32
+// X with K > 128 on the FP64 form too, whose right factors take half the room, at several times the
+// time.
+enum FitRoom { kFitRoomy, kFitTight, kFitLeast };
+size_t fit_workspace(const FitArgs& a, bool x_f64, FitRoom room, int* blocks, size_t* table_bytes);
+cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, FitRoom room, void* ws,
                        int blocks, float* tables, unsigned* err, cudaStream_t st);
 
 }  // namespace trk

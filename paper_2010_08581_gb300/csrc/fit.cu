@@ -84,14 +84,16 @@ void fit_f64(const FitArgs& a, const FitSplit& f, const void* X, char* wt, doubl
 }
 
 // FP32 X on the FP64 form (fit_body.cuh).
-bool fit_plain(const FitSplit& f, bool x_f64, bool tight) { return tight && !x_f64 && f.K > FKPlain; }
+bool fit_plain(const FitSplit& f, bool x_f64, FitRoom room) {
+  return room == kFitLeast && !x_f64 && f.K > FKPlain;
+}
 
 }  // namespace
 
-size_t fit_workspace(const FitArgs& a, bool x_f64, bool tight, int* blocks, size_t* table_bytes) {
+size_t fit_workspace(const FitArgs& a, bool x_f64, FitRoom room, int* blocks, size_t* table_bytes) {
   const FitSplit f = split_of(a);
-  if (tight) {   // as little room as one CTA per row block takes
-    const bool plain = fit_plain(f, x_f64, true);
+  if (room != kFitRoomy) {   // the room of one CTA per row block
+    const bool plain = fit_plain(f, x_f64, room);
     const int64_t edge = x_f64 ? FL : (plain ? 2 * FL : FT_Q);
     const int64_t most = x_f64 || plain ? 4 * sm_count() : sm_count();
     const int64_t rb = (f.rows + edge - 1) / edge;
@@ -120,14 +122,14 @@ size_t fit_workspace(const FitArgs& a, bool x_f64, bool tight, int* blocks, size
   return round256(round256(static_cast<size_t>(2 * b) * sizeof(double)) + right);
 }
 
-cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, bool tight, void* ws,
+cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, FitRoom room, void* ws,
                        int blocks, float* tables, unsigned* err, cudaStream_t st) {
   const FitSplit f = split_of(a);
   double* partial = static_cast<double*>(ws);
   char* wt = static_cast<char*>(ws) + round256(static_cast<size_t>(2 * blocks) * sizeof(double));
   if (x_f64) {
     fit_f64<double>(a, f, X, wt, partial, blocks, st);
-  } else if (fit_plain(f, x_f64, tight)) {
+  } else if (fit_plain(f, x_f64, room)) {
     fit_f64<float>(a, f, X, wt, partial, blocks, st);
   } else {
     const FitTcPlan pl = fit_tc_plan(a, f);

@@ -11,10 +11,12 @@
 //
 // The split is chosen so that cols is large enough to amortise the row chains while the right
 // factors stay small (fit_split). FP32 X is evaluated on the tensor cores (fit_tc.cuh). This
-// file holds the split and the FP64 form (also for FP32 X with K > 128 where the budget has no
-// room for the tensor cores' operand of W, twice the size of FP32 W^T): W is formed once per evaluation (fit_right_warp,
+// file holds the split and the FP64 form: W is formed once per evaluation (fit_right_warp,
 // e-major: W^T[e][q]) and V per block of FL rows in shared memory; each thread computes a
-// 2 x 2 register tile of TR from two vector loads per e.
+// 2 x 2 register tile of TR from two vector loads per e. FP32 X with K > 128 takes it too where a
+// budget or an arena has no room for the tensor cores' operand of W (two parts of every entry, in
+// whole tiles of 128 columns and 32 terms) but has room for FP32 W^T, half as large: such a call is
+// slow rather than refused.
 //
 // The work is cut into units (row block, column tile), row block by row block, and every CTA
 // takes one contiguous range of them, forming V again where its range enters a row block. A
@@ -31,7 +33,7 @@ constexpr int FNT = 256;                       // threads of a fit CTA
 constexpr int64_t kFitMinCols = 256;           // grow cols (move s left) up to this
 constexpr int64_t kFitMaxRight = 1ll << 22;    // max elements of W^T (cols * K)
 
-constexpr int FKPlain = 128;                   // FP32 X: W's operand is never larger than W^T up to here
+constexpr int FKPlain = 128;                   // FP32 X: the longest K without that form
 constexpr int FL = 32, FI = 32;                // rows and columns of an FP64 tile
 constexpr int FMI = 2, FMJ = 2;                // outputs per thread
 

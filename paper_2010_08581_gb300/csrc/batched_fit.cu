@@ -40,8 +40,8 @@ __device__ __forceinline__ void fit_args(const BInst& d, FitArgs& fa) {
 __device__ __forceinline__ float* fit_tables(const BInst& d, const FitArgs& fa, const FitSplit& f) {
   int64_t Imax = 0;
   for (int m = 0; m < fa.N; ++m) Imax = fa.dims[m] > Imax ? fa.dims[m] : Imax;
-  return fit_tc_tables_fit(fa, f) && fit_tc_tables_floats(fa, f) <= d.J * Imax
-             ? static_cast<float*>(d.Y) : nullptr;
+  const int64_t n = fit_tc_tables_floats(fa, f);
+  return n > 0 && fit_tc_tables_fit(fa, f) && n <= d.J * Imax ? static_cast<float*>(d.Y) : nullptr;
 }
 
 constexpr int kFitRightCtas = 128;  // CTAs per slot forming the right factors
@@ -77,30 +77,27 @@ __global__ void __launch_bounds__(FNT) kb_fit_right(const BInst* __restrict__ ta
 }
 
 // ... or the split operand tiles of the tensor-core contraction.
-__global__ void __launch_bounds__(FT_Q) kb_fit_right_tc(const BInst* __restrict__ tab) {
+__global__ void __launch_bounds__(32 * FT_RWS) kb_fit_right_tc(const BInst* __restrict__ tab) {
   __shared__ __align__(16) float P[32 * 256];   // 8 chains of kMaxL doubles in the FP64 form
-  __shared__ float G[4 * kMaxL];
+  __shared__ float G[FT_RWS * kMaxL];
   __shared__ FitArgs fa;
   const BInst& d = tab[blockIdx.x];
   if (!fit_due(d)) return;
   if (threadIdx.x == 0) fit_args(d, fa);
   __syncthreads();
   const FitSplit f = fit_split(fa.N, fa.dims, fa.ranks);
-  const float* tables = fit_tables(d, fa, f);
-  if (tables) tables += fit_tc_table_floats(fa, f.s - 1);
+  const float* table = fit_tc_right(fa, f, fit_tables(d, fa, f));
   if (d.fit_plain) {        // FP32 W^T for the FP64 form
     double (*chain)[kMaxL] = reinterpret_cast<double (*)[kMaxL]>(P);
     const int warp = threadIdx.x >> 5;
-    for (int64_t q = static_cast<int64_t>(blockIdx.y) * 4 + warp; q < f.cols; q += 4 * gridDim.y)
+    for (int64_t q = static_cast<int64_t>(blockIdx.y) * FT_RWS + warp; q < f.cols; q += FT_RWS * gridDim.y)
       fit_right_warp(fa, f, q, static_cast<float*>(d.fitw), chain[warp], chain[4 + warp],
                      static_cast<int>(threadIdx.x & 31));
     return;
   }
-  const int nj = (f.K + 2 * FT_KS - 1) / (2 * FT_KS);      // jobs of two k-steps
-  const int64_t jobs = (f.cols + FT_Q - 1) / FT_Q * nj;
-  for (int64_t j = blockIdx.y; j < jobs; j += gridDim.y) {
-    const int ks = 2 * static_cast<int>(j % nj);
-    fit_right_tc_tile(fa, f, j / nj, ks, ks + 2, tables, static_cast<unsigned char*>(d.fitw), P, G);
+  const int jobs = fit_right_jobs((f.cols + FT_Q - 1) / FT_Q, (f.K + FT_KS - 1) / FT_KS, 4 * FT_RWS);
+  for (int j = blockIdx.y; j < jobs; j += gridDim.y) {
+    fit_right_tc_job<FT_RWS, 4>(fa, f, j, table, static_cast<unsigned char*>(d.fitw), P, G);
     __syncthreads();
   }
 }
@@ -161,7 +158,7 @@ __global__ void __launch_bounds__(FT_NT, 1) kb_fit_tc(const BInst* __restrict__ 
     return;
   }
   fit_tc_units(fa, f, pl, static_cast<const float*>(d.X),
-               static_cast<const unsigned char*>(d.fitw), fit_tables(d, fa, f),
+               static_cast<const unsigned char*>(d.fitw), fit_tc_left(fa, f, fit_tables(d, fa, f)),
                pl.units * blockIdx.y / parts, pl.units * (blockIdx.y + 1) / parts, fit_tc_dyn, sh,
                err, se, sx);
   fit_tc_reduce(se, sx, red);
@@ -214,7 +211,7 @@ cudaError_t bl_fit(const BLaunch& b, unsigned* err, cudaStream_t st) {
     kb_fit<<<grid, FNT, fit_smem_bytes(b.Lmax), st>>>(b.tab);
   } else {
     kb_fit_tables<<<dim3(b.count, 16), 256, 0, st>>>(b.tab);
-    kb_fit_right_tc<<<rgrid, FT_Q, 0, st>>>(b.tab);
+    kb_fit_right_tc<<<rgrid, 32 * FT_RWS, 0, st>>>(b.tab);
     kb_fit_tc<<<grid, FT_NT, kFitTcSmem, st>>>(b.tab, err);
   }
   return cudaGetLastError();

@@ -35,19 +35,19 @@ __global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const T* __r
   }
 }
 
-// FP32 slice tables of the modes s - 1 and N - 1 (fit_tc.cuh), one warp per slice.
+// FP32 slice tables (fit_tc.cuh), one warp per slice.
 __global__ void __launch_bounds__(256) k_fit_tables(FitArgs a, FitSplit f,
                                                     float* __restrict__ out) {
   fit_tables_warps(a, f, out, (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5,
                    static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5));
 }
 
-__global__ void __launch_bounds__(FT_Q) k_fit_right_tc(FitArgs a, FitSplit f, const float* tables,
-                                                       unsigned char* __restrict__ WS) {
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) k_fit_right_tc(FitArgs a, FitSplit f, const float* tables,
+                                                              unsigned char* __restrict__ WS) {
   __shared__ __align__(16) float P[32 * 256];
-  __shared__ float G[4 * kMaxL];
-  fit_right_tc_tile(a, f, blockIdx.x, 2 * blockIdx.y, 2 * blockIdx.y + 2,
-                    tables ? tables + fit_tc_table_floats(a, f.s - 1) : nullptr, WS, P, G);
+  __shared__ float G[kWarps * kMaxL];
+  fit_right_tc_job<kWarps, 1>(a, f, blockIdx.x, fit_tc_right(a, f, tables), WS, P, G);
 }
 
 __global__ void __launch_bounds__(FT_NT, 1) k_fit_tc(FitArgs a, FitSplit f, FitTcPlan pl,
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(FT_NT, 1) k_fit_tc(FitArgs a, FitSplit f, FitT
   __shared__ double red[2 * FT_EW];
   __shared__ FitTcShared sh;
   double se = 0.0, sx = 0.0;
-  fit_tc_units(a, f, pl, X, WS, tables, pl.units * blockIdx.x / gridDim.x,
+  fit_tc_units(a, f, pl, X, WS, fit_tc_left(a, f, tables), pl.units * blockIdx.x / gridDim.x,
                pl.units * (blockIdx.x + 1) / gridDim.x, fit_tc_raw, sh, err, se, sx);
   fit_tc_reduce(se, sx, red);
   if (threadIdx.x == 0) {
@@ -104,11 +104,12 @@ size_t fit_workspace(const FitArgs& a, bool x_f64, FitRoom room, int* blocks, si
                            : fit_tc_right_bytes(f));
   }
   int64_t b = x_f64 ? fit_units(f) : fit_tc_plan(a, f).units;
-  // the tensor-core form: one CTA per SM. FP64: four per SM, but with a chain of three or more
+  // the tensor-core form: one CTA per SM. FP64: as many as are resident (three per SM up to
+  // K = 80; a fourth is a round of its own: 100000 x 3 x 3, rank 3: 148 us a call), but with a chain of three or more
   // modes a CTA's own V costs more than a tile of products, so the CTAs are then whole row
   // blocks, or equal parts of them while SMs are left over (4^10, rank 10: 279 us with 128 row
   // blocks on as many CTAs, 352 us with 304 CTAs that form V twice each)
-  int64_t cap = x_f64 ? 4 * sm_count() : sm_count();
+  int64_t cap = x_f64 ? 3 * sm_count() : sm_count();
   if (x_f64 && f.s > 2) {
     const int64_t rb = (f.rows + FL - 1) / FL;
     const int64_t whole = rb * (sm_count() / rb > 1 ? sm_count() / rb : 1);
@@ -135,11 +136,15 @@ cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, FitRoom room
     const FitTcPlan pl = fit_tc_plan(a, f);
     unsigned char* WS = reinterpret_cast<unsigned char*>(wt);
     if (tables) {
-      const int64_t n = (a.dims[f.s - 1] + a.dims[a.N - 1] + 7) / 8;
+      const int64_t n = ((f.s > 1 ? a.dims[f.s - 1] : 0) + (f.s < a.N - 1 ? a.dims[a.N - 1] : 0) + 7) / 8;
       const int64_t tb = n < 8 * sm_count() ? n : 8 * sm_count();
       k_fit_tables<<<static_cast<unsigned>(tb), 256, 0, st>>>(a, f, tables);
     }
-    k_fit_right_tc<<<dim3(static_cast<unsigned>(pl.tiles), (pl.ks + 1) / 2), FT_Q, 0, st>>>(a, f, tables, WS);
+    const int jobs = fit_right_jobs(pl.tiles, pl.ks, FT_RW);
+    if (f.s < a.N - 1 && a.dims[a.N - 1] < 8 && jobs <= 2 * sm_count())
+      k_fit_right_tc<FT_RW><<<jobs, 32 * FT_RW, 0, st>>>(a, f, tables, WS);
+    else
+      k_fit_right_tc<FT_RWS><<<fit_right_jobs(pl.tiles, pl.ks, FT_RWS), 32 * FT_RWS, 0, st>>>(a, f, tables, WS);
     k_fit_tc<<<blocks, FT_NT, kFitTcSmem, st>>>(a, f, pl, static_cast<const float*>(X), WS, tables,
                                                 partial, blocks, err);
   }

@@ -44,7 +44,7 @@ namespace trk {
 constexpr int FT_Q = 128;                      // columns of X per tile (MMA M)
 constexpr int FT_KS = 8;                       // terms per k-step (MMA K)
 constexpr int FT_SLOT = 2 * 2 * FT_Q * 16;     // W of one tile and k-step: 8 KB
-constexpr int FT_MAXKS = kMaxL / FT_KS;        // 16
+constexpr int FT_MAXKS = kMaxL / FT_KS;        // 32
 constexpr int FT_MAXSLOTS = 8;
 constexpr int FT_EW = 8, FT_BW = 8;            // epilogue and builder warps
 constexpr int FT_NT = 32 * (FT_EW + FT_BW + 4);
@@ -62,16 +62,33 @@ __host__ __device__ inline size_t fit_tc_right_bytes(const FitSplit& f) {
 
 // FP32 slice tables of the last mode of each group, entry-major: t[(r * Rc + c) * I + i], so
 // that threads that own consecutive indices i read consecutive words. Optional: without them
-// the FP64 cores are read (one conversion per use, on the FP64 pipe).
+// the FP64 cores are read (one conversion per use, on the FP64 pipe). A group of one mode has none:
+// its entries are read once (100000 x 3 x 3, rank 3: 102 us a call with a table, 89 without).
 __host__ __device__ inline int64_t fit_tc_table_floats(const FitArgs& a, int mode) {
   return a.dims[mode] * a.ranks[(mode - 1 + a.N) % a.N] * a.ranks[mode];
 }
-__host__ __device__ inline int64_t fit_tc_tables_floats(const FitArgs& a, const FitSplit& f) {
-  return fit_tc_table_floats(a, f.s - 1) + fit_tc_table_floats(a, a.N - 1);
+__host__ __device__ inline int64_t fit_tc_left_floats(const FitArgs& a, const FitSplit& f) {
+  return f.s > 1 ? fit_tc_table_floats(a, f.s - 1) : 0;
 }
-// Table offsets are 32-bit.
+__host__ __device__ inline int64_t fit_tc_right_floats(const FitArgs& a, const FitSplit& f) {
+  return f.s < a.N - 1 ? fit_tc_table_floats(a, a.N - 1) : 0;
+}
+__host__ __device__ inline int64_t fit_tc_tables_floats(const FitArgs& a, const FitSplit& f) {
+  return fit_tc_left_floats(a, f) + fit_tc_right_floats(a, f);
+}
+// Table offsets are 32-bit. Where the right group alone has one, few entries read with a conversion
+// each cost less than the launch that forms it (20 x 20 x 20, rank 8, 2e5 of them: 77 us a call with
+// the table, 74 without; 60 x 60 x 60, rank 16, 1.5e7: 142 and 176).
 __host__ __device__ inline bool fit_tc_tables_fit(const FitArgs& a, const FitSplit& f) {
-  return fit_tc_tables_floats(a, f) < (1ll << 31);
+  return (f.s > 1 || f.cols * a.ranks[a.N - 2] * f.K >= (1 << 20)) &&
+         fit_tc_tables_floats(a, f) < (1ll << 31);
+}
+// The two tables behind `tables` (null where there is none).
+__host__ __device__ inline const float* fit_tc_left(const FitArgs& a, const FitSplit& f, const float* tables) {
+  return f.s > 1 ? tables : nullptr;
+}
+__host__ __device__ inline const float* fit_tc_right(const FitArgs& a, const FitSplit& f, const float* tables) {
+  return tables && f.s < a.N - 1 ? tables + fit_tc_left_floats(a, f) : nullptr;
 }
 
 struct FitTcPlan {
@@ -173,27 +190,48 @@ __device__ __forceinline__ float dot_row(const float* row, const float (&g)[16],
 
 // Product of the slices of modes m0 .. m1 - 1 at the mixed-radix index `pre` (the last mode
 // fastest) into dst (row stride 16, zeros beyond the last rank), one warp; G is scratch of
-// kMaxL floats, used when the product has more than one factor.
+// kMaxL floats, used when the product has more than one factor. kAhead: a factor's loads are in
+// flight while the one before it is multiplied (16 registers; a long chain is their latency).
+template <bool kAhead>
 __device__ inline void prefix_product(const FitArgs& a, int m0, int m1, int64_t pre, float* dst,
                                       float* G, int lane) {
   int64_t div = 1;
   for (int m = m0 + 1; m < m1; ++m) div *= a.dims[m];
   const int rows = a.ranks[(m0 - 1 + a.N) % a.N];
   int cols = a.ranks[m0];
+  double next[kAhead ? kMaxL / 32 : 1];
+  auto fetch = [&](int m, int left) {        // the slice of mode m, left x ranks[m]
+    pre %= div;
+    div /= a.dims[m];
+    const int n = left * a.ranks[m];
+    const double* src = a.core[m] + (pre / div) * n;
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int q = 0; q < kMaxL / 32; ++q) next[q] = lane + 32 * q < n ? src[lane + 32 * q] : 0.0;
+    } else {
+      __syncwarp();
+      for (int e = lane; e < n; e += 32) G[e] = static_cast<float>(src[e]);
+    }
+  };
   {
     const double* src = a.core[m0] + (pre / div) * rows * cols;
+    if (kAhead && m0 + 1 < m1) fetch(m0 + 1, cols);
     for (int e = lane; e < rows * 16; e += 32) {
       const int r = e >> 4, c = e & 15;
       dst[e] = c < cols ? static_cast<float>(src[r * cols + c]) : 0.f;
     }
   }
   for (int m = m0 + 1; m < m1; ++m) {
-    pre %= div;
-    div /= a.dims[m];
     const int rr = a.ranks[m];
-    const double* src = a.core[m] + (pre / div) * cols * rr;
-    __syncwarp();
-    for (int e = lane; e < cols * rr; e += 32) G[e] = static_cast<float>(src[e]);
+    if constexpr (kAhead) {
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < kMaxL / 32; ++q)
+        if (lane + 32 * q < cols * rr) G[lane + 32 * q] = static_cast<float>(next[q]);
+      if (m + 1 < m1) fetch(m + 1, rr);
+    } else {
+      fetch(m, cols);
+    }
     __syncwarp();
     float acc[8];                    // rows * 16 <= 256 entries, 8 per lane
 #pragma unroll
@@ -284,7 +322,7 @@ __device__ __forceinline__ void build_v(const FitArgs& a, const FitSplit& f, con
       const int np = static_cast<int>((pend - 1) / I - pre0 + 1);
       for (int x = bw; x < np; x += FT_BW) {
         float* dst = prefix + x * pstride;
-        prefix_product(a, 0, f.s - 1, pre0 + x, dst, scratch + bw * kMaxL, lane);
+        prefix_product<false>(a, 0, f.s - 1, pre0 + x, dst, scratch + bw * kMaxL, lane);
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");
     }
@@ -354,78 +392,100 @@ __device__ __forceinline__ void build_v(const FitArgs& a, const FitSplit& f, con
 
 }  // namespace ft
 
-// The slice tables of the modes s - 1 and N - 1, one warp per slice: warp w of n.
+// The slice tables, one warp per slice: warp w of n.
 __device__ inline void fit_tables_warps(const FitArgs& a, const FitSplit& f, float* out, int64_t w,
                                         int64_t n) {
   const int lane = threadIdx.x & 31;
-  const int64_t I0 = a.dims[f.s - 1], I1 = a.dims[a.N - 1];
+  const int64_t I0 = f.s > 1 ? a.dims[f.s - 1] : 0, I1 = f.s < a.N - 1 ? a.dims[a.N - 1] : 0;
   for (; w < I0 + I1; w += n) {
     const int mode = w < I0 ? f.s - 1 : a.N - 1;
     const int64_t i = w < I0 ? w : w - I0, I = w < I0 ? I0 : I1;
-    float* t = w < I0 ? out : out + fit_tc_table_floats(a, f.s - 1);
+    float* t = w < I0 ? out : out + fit_tc_left_floats(a, f);
     const int L = a.ranks[(mode - 1 + a.N) % a.N] * a.ranks[mode];
     for (int e = lane; e < L; e += 32) t[e * I + i] = static_cast<float>(a.core[mode][i * L + e]);
   }
 }
 
-// W of one 128-column tile and the k-steps ks0 .. ks1 - 1, by a CTA of 128 threads (thread =
-// column), in operand layout: WS[tile][k-step][part][k-group][column][4]; entry e = b * Rlast + a
-// holds P_right(q)[b][a]. Prefix products (modes s .. N-2) are formed 32 at a time.
-// P: 32 * 256 floats, G: 4 * kMaxL floats of shared memory.
-__device__ inline void fit_right_tc_tile(const FitArgs& a, const FitSplit& f, int64_t tile,
-                                         int ks0, int ks1, const float* table, unsigned char* WS,
-                                         float* P, float* G) {
+// The right factors are formed in jobs of 32 columns and kWarps * kPer k-steps: thread = column, and
+// kPer k-steps one after another. What bounds a job is chains: of its at most 32 prefix products
+// (modes s .. N-2), dealt out to the warps, of the loads of an entry's slice column, and of the
+// instructions themselves, hence one short loop over the entries (unrolled, with 128 columns and two
+// k-steps a CTA: 10 x 10 x 10, rank 3: 20 us, now 9; 2^12, rank 3, with 64 prefixes of six products:
+// 110, now 17). One problem: 4 warps and one k-step each, or 16 where 32 columns span more than four
+// prefixes and the jobs leave SMs idle (2^12 with 4: 39 us; 20 x 20 x 20, rank 8, with 16: 17 us, with
+// 4: 11, the conversions of one SM's FP64 pipe); served requests share the SMs: 4 warps and 4 k-steps
+// each, so that a prefix product serves more entries.
+constexpr int FT_RC = 32, FT_RW = 16, FT_RWS = 4;
+__host__ __device__ inline int fit_right_jobs(int64_t tiles, int ks, int per_job) {
+  return static_cast<int>(tiles) * (FT_Q / FT_RC) * ((ks + per_job - 1) / per_job);
+}
+
+template <bool kTable>
+__device__ __forceinline__ void fit_right_entries(const ft::Slices& g, bool pre, const float* P,
+                                                  int Rlast, int e0, int e1, bool valid, int64_t i,
+                                                  unsigned char* dst) {
+  const float* tp = g.table + i;
+  const double* dp = g.core + i * g.Rm * g.Rc;
+  const int cstep = kTable ? g.Rc * static_cast<int>(g.I) : g.Rc;
+  const int bstep = kTable ? static_cast<int>(g.I) : 1;
+  auto entry = [&](int o) -> float {
+    if constexpr (kTable) return __ldg(tp + o);
+    else return static_cast<float>(__ldg(dp + o));
+  };
+  int b = e0 / Rlast, c = e0 - b * Rlast;
+  const int end = (e1 + FT_KS - 1) / FT_KS * FT_KS;       // the last k-step is padded with zeros
+#pragma unroll 1
+  for (int e = e0; e < end; ++e) {
+    float v = 0.f;
+    if (valid && e < e1) {
+      if (pre) {
+        float gc[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) gc[t] = t < g.Rm ? entry(t * cstep + c * bstep) : 0.f;
+        v = ft::dot_row(P + b * 16, gc, g.Rm);
+      } else {
+        v = entry(b * cstep + c * bstep);
+      }
+    }
+    const float h = tc::tf32_rna(v);
+    unsigned char* at = dst + static_cast<size_t>((e - e0) / FT_KS) * FT_SLOT +
+                        ((e >> 2) & 1) * (FT_Q * 16) + (e & 3) * 4;
+    *reinterpret_cast<float*>(at) = h;
+    *reinterpret_cast<float*>(at + 2 * FT_Q * 16) = tc::tf32_rna(v - h);
+    if (++c == Rlast) { c = 0; ++b; }
+  }
+}
+
+// Job `job` of them, in operand layout: WS[tile][k-step][part][k-group][column][4]; entry
+// e = b * Rlast + a holds P_right(q)[b][a]. P: 32 * 256 floats, G: kWarps * kMaxL floats of shared
+// memory.
+template <int kWarps, int kPer>
+__device__ inline void fit_right_tc_job(const FitArgs& a, const FitSplit& f, int64_t job,
+                                        const float* table, unsigned char* WS, float* P, float* G) {
+  constexpr int kJob = kWarps * kPer;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nks = (f.K + FT_KS - 1) / FT_KS;
+  const int nks = (f.K + FT_KS - 1) / FT_KS, nkj = (nks + kJob - 1) / kJob;
   const int Rlast = a.ranks[a.N - 1];
   const ft::Slices g = ft::slices(a, a.N - 1, table);
   const bool pre = f.s < a.N - 1;
-  const int64_t q = tile * FT_Q + threadIdx.x;
+  const int64_t part = job / nkj, tile = part / (FT_Q / FT_RC);
+  const int ks = static_cast<int>(job - part * nkj) * kJob + warp * kPer;
+  const int64_t q = part * FT_RC + lane;
   const bool valid = q < f.cols;
-  const int64_t i = valid ? q % g.I : 0, mine = valid ? q / g.I : 0;
-  const int64_t last = (tile * FT_Q + FT_Q < f.cols ? tile * FT_Q + FT_Q : f.cols) - 1;
-  const int64_t pre0 = tile * FT_Q / g.I, pre1 = last / g.I;
-  for (int64_t b0 = pre0; b0 <= pre1; b0 += 32) {
-    if (pre) {
-      __syncthreads();
-      for (int64_t x = b0 + warp; x <= pre1 && x < b0 + 32; x += 4)
-        ft::prefix_product(a, f.s, a.N - 1, x, P + (x - b0) * 256, G + warp * kMaxL, lane);
-      __syncthreads();
-    }
-    const bool now = valid && (!pre || (mine >= b0 && mine < b0 + 32));
-    if (now || (!valid && b0 == pre0)) {
-      int b = ks0 * FT_KS / Rlast, c = ks0 * FT_KS - b * Rlast;
-      for (int ks = ks0; ks < ks1 && ks < nks; ++ks) {
-        unsigned char* dst = WS + (static_cast<size_t>(tile) * nks + ks) * FT_SLOT + threadIdx.x * 16;
-        float h[FT_KS], l[FT_KS];
-#pragma unroll
-        for (int u = 0; u < FT_KS; ++u) {
-          float v = 0.f;
-          if (now && ks * FT_KS + u < f.K) {
-            if (pre) {
-              float gc[16];
-#pragma unroll
-              for (int t = 0; t < 16; ++t) gc[t] = t < g.Rm ? g.at(t, c, i) : 0.f;
-              v = ft::dot_row(P + (mine - b0) * 256 + b * 16, gc, g.Rm);
-            } else {
-              v = g.at(b, c, i);
-            }
-          }
-          h[u] = tc::tf32_rna(v);
-          l[u] = tc::tf32_rna(v - h[u]);
-          if (++c == Rlast) { c = 0; ++b; }
-        }
-#pragma unroll
-        for (int kg = 0; kg < 2; ++kg) {
-          unsigned char* d = dst + kg * (FT_Q * 16);
-          *reinterpret_cast<float4*>(d) = make_float4(h[4 * kg], h[4 * kg + 1], h[4 * kg + 2], h[4 * kg + 3]);
-          *reinterpret_cast<float4*>(d + 2 * FT_Q * 16) =
-              make_float4(l[4 * kg], l[4 * kg + 1], l[4 * kg + 2], l[4 * kg + 3]);
-        }
-      }
-    }
-    if (!pre) break;
+  const int64_t mine = q / g.I, pre0 = part * FT_RC / g.I;
+  if (pre && part * FT_RC < f.cols) {
+    const int64_t last = (part * FT_RC + FT_RC < f.cols ? part * FT_RC + FT_RC : f.cols) - 1;
+    for (int64_t x = pre0 + warp; x <= last / g.I; x += kWarps)
+      ft::prefix_product<true>(a, f.s, a.N - 1, x, P + (x - pre0) * 256, G + warp * kMaxL, lane);
   }
+  __syncthreads();
+  if (ks >= nks) return;
+  const int e0 = ks * FT_KS, most = (ks + kPer) * FT_KS, e1 = most < f.K ? most : f.K;
+  unsigned char* dst = WS + (static_cast<size_t>(tile) * nks + ks) * FT_SLOT + (q - tile * FT_Q) * 16;
+  const float* Pq = P + (valid ? mine - pre0 : 0) * 256;
+  const int64_t i = valid ? q - mine * g.I : 0;
+  if (table) fit_right_entries<true>(g, pre, Pq, Rlast, e0, e1, valid, i, dst);
+  else fit_right_entries<false>(g, pre, Pq, Rlast, e0, e1, valid, i, dst);
 }
 
 // Accumulates (se, sx) over the units lo .. hi - 1 (unit = row block * tiles + tile). All

@@ -638,8 +638,14 @@ cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t l
   return cudaGetLastError();
 }
 
+// A row costs one product here (n^2 multiply-adds, in tiles) and half of that in the substitutions,
+// which many rows keep busy. Break-even by whole calls: I = 3000 for n = 90, 5800 for 100, 7000 for 121
+// and 144 (I = 20000, n = 100: 1157 us here, 977 by substitutions), and, where the factor no longer
+// fits one SM's shared memory, 10500 for 169, 12500 for 196, 19000 for 225 and 32000 for 256
+// (I = 5000: 877 us here and 1081 for 169, 1453 and 2838 for 256; I = 50000: 6.8 and 5.2 ms, 11.1 and
+// 10.2).
 bool leverage_f64_fits(int64_t I, int n, int splits) {
-  return n >= kLev64MinN && n <= kMaxL && I >= n && splits >= 4;
+  return n >= kLev64MinN && n <= kMaxL && I >= n && I <= (n > kSolveBigMin ? 64 : 32) * n && splits >= 4;
 }
 
 cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,

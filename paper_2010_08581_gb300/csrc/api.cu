@@ -361,11 +361,13 @@ tr_status leverage_dist(tr_ctx* ctx, char* ws, const double* mat, int64_t I, int
     TR_LAUNCH("reduce_gram", launch_reduce(p1.partial, false, p1.splits, static_cast<int64_t>(L) * L,
                                            L, L, L, L, p1.G, L, nullptr, 0, st, sp));
     TR_LAUNCH("lev64_factor", launch_leverage_f64(0, w, mat, I, L, L, ell, ep, st));
-    if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
-    TR_LAUNCH("lev64_rows", launch_leverage_f64(1, w, mat, I, L, L, ell, ep, st));
+    // (before the wait, so that it runs beside the LS step's own factorisation: it writes X, K's
+    // FP32 array and E, which the rows do not read, and only when they have nothing to do)
     TR_LAUNCH("cholesky_leverage", launch_cholesky(p1.G, L, 1, tol, p1.Lrow, p1.Lcol, p1.invdiag,
                                                    p1.keep, p1.info, ctx->d_err, st, p1.img,
                                                    nullptr, nullptr, w.bad + 1));
+    if (wait_before_rows) TR_CUDA(cudaStreamWaitEvent(st, wait_before_rows, 0));
+    TR_LAUNCH("lev64_rows", launch_leverage_f64(1, w, mat, I, L, L, ell, ep, st));
     CdfEpilogue ep2 = ep;
     ep2.run_if = w.bad + 1;
     TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,

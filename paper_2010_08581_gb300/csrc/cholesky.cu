@@ -184,6 +184,12 @@ cudaError_t cholesky_attributes() {
   cudaError_t e =
       cudaFuncSetAttribute(k_cholesky, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholDyn);
   if (e != cudaSuccess) return e;
+  // Beyond 160 unknowns the matrix stays in global memory and the factorisation lives off L1: without
+  // this preference an SM that runs the other branch's tiles leaves it little (n = 256: 2.2 ms
+  // beside them instead of 1.45).
+  e = cudaFuncSetAttribute(k_cholesky, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           cudaSharedmemCarveoutMaxL1);
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_cholesky_mixed<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kCholDyn);
   if (e != cudaSuccess) return e;

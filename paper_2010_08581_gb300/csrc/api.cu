@@ -286,6 +286,15 @@ bool precond_enabled() {
   return !(e && e[0] == '0');
 }
 
+// The mixed drivers' tall distributions outside lev_precond.cu (initial ones, those of the
+// column-dropping rule, and L > 128) keep the double-float factorisation as far as it goes. A call
+// with three of them, I = 300, good cores: L = 88: 625 us by FP64 products, 581 so; 100: 663 and 645;
+// 128: 755 and 823; 160: 1115 and 1278 (I = 1000: 759 and 672, 871 and 814, at 144 1409 and 1390). Poor
+// cores, on which the products are refused, pay for both: four sweeps at L = 144: 6.0 ms and 4.1,
+// with the dropping rule 6.0 and 5.4. Beyond 160 one CTA factors in FP64 from global memory and the
+// products win either way.
+constexpr int kDoubleFloatMax = 160;
+
 // Leverage scores of the rows of the I x L row-major matrix `mat` (a core's G_(2), or any
 // matrix with the same column space) and, from them, p and the CDF (unless *skip != 0).
 // `mixed` (the mixed-precision drivers): a tall matrix's Gram is factored in double-float
@@ -341,7 +350,8 @@ tr_status leverage_dist(tr_ctx* ctx, char* ws, const double* mat, int64_t I, int
     ep2.run_if = gate;
     TR_LAUNCH("leverage_rows", launch_trsm(0, false, L, p1.invdiag, nullptr, I, mat, L, 1, 1,
                                            nullptr, ell, st, p1.img, nullptr, &ep2));
-  } else if (precond_enabled() && leverage_f64_fits(I, L, p1.splits)) {
+  } else if (!(mixed && L <= kDoubleFloatMax) && precond_enabled() &&
+             leverage_f64_fits(I, L, p1.splits)) {
     // FP64 products around an FP32 inverse (lev64.cu); the FP64 factorisation and row solves run
     // only when its device flag says so
     ReduceSplit sp;

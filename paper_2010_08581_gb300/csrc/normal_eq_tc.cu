@@ -16,14 +16,17 @@
 // where it lies: there 32 consecutive samples of one column are consecutive words of X.
 //
 // A stage is latency: loads, conversion, two barriers and twelve MMAs follow one another. With
-// 128 columns per CTA (129 KB of shared memory) one CTA ran per SM: 2.2 us a stage, and 155
-// CTAs on 152 SMs took two rounds at J = 250,000 (1134 us). With 64 or 80 columns two CTAs
-// share an SM and one's loads and conversions cover the other's MMAs (788 us).
+// 128 columns per CTA (129 KB of shared memory) one CTA runs per SM, and 155 CTAs on 152 SMs took
+// two rounds at J = 250,000 (1134 us). With 64 or 80 columns two CTAs share an SM and one's loads
+// and conversions cover the other's MMAs (788 us). One CTA of 128 columns per SM converts A's rows
+// half as often and is the best where it is one round (launch_normal_eq_tc).
 // The column tile does not change a result: an entry is the same sequence of FP32
 // accumulations over the same chunk of samples whatever the tile. Every
 // mbarrier wait is bounded: a wait of the main loop polls at most `wait_limit` times; on
 // expiry the CTA records an error, stops issuing, waits (bounded by the default limit) for
 // the MMAs it has committed, frees its TMEM and returns without writing its partials.
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -41,13 +44,15 @@ constexpr uint32_t TMEM_COLS = 128;    // FP32 accumulator: 128 lanes x TN <= 12
 
 template <int TN>
 constexpr int stage_bytes() { return 2 * A_BYTES + 2 * TN * TK * 4; }   // hi and lo of both
+template <int TN>
+constexpr int smem_bytes() { return STAGES * stage_bytes<TN>() + 1024; }
 
 using namespace tc;
 
 // TN output columns per CTA (MMA N). kDense: the columns from L on are X viewed as
 // [J / post][I][post] (Y points to X, post > 1): Y[r][i] = X[r / post][i][r % post].
 template <int TN, bool kDense>
-__global__ void __launch_bounds__(NT, 2) k_normal_eq_tc(const float* __restrict__ A,
+__global__ void __launch_bounds__(NT, TN > 80 ? 1 : 2) k_normal_eq_tc(const float* __restrict__ A,
                                                         const float* __restrict__ Y, int64_t J,
                                                         int L, int64_t I, int64_t post,
                                                         int64_t chunk,
@@ -306,7 +311,7 @@ cudaError_t launch_tn(const float* A, const float* Y, int64_t J, int L, int64_t 
                       int64_t chunk, int splits, float* partial, unsigned* err, cudaStream_t st,
                       long long wait_limit, const int64_t* jdev) {
   dim3 grid(static_cast<unsigned>((L + I + TN - 1) / TN), (L + TM - 1) / TM, splits);
-  launch_pdl((k_normal_eq_tc<TN, kDense>), grid, NT, STAGES * stage_bytes<TN>() + 1024, st, A, Y, J,
+  launch_pdl((k_normal_eq_tc<TN, kDense>), grid, NT, smem_bytes<TN>(), st, A, Y, J,
              L, I, post, chunk, partial, err, wait_limit < 0 ? kTcSpinLimit : wait_limit, jdev);
   return cudaGetLastError();
 }
@@ -326,35 +331,43 @@ cudaError_t launch_normal_eq_tc(const float* A, const float* Y, int64_t J, int L
   int64_t chunk;
   plan_tc(J, L, I, &s, &chunk);
   if (s != splits) return cudaErrorInvalidValue;
-  // The busiest SM's share: CTAs per SM times the work of a stage (the tile's columns plus A's
-  // 128 rows, which every column tile converts again). 64 columns unless 80 save a round of
-  // CTAs: J = 250,000, L = 100, I = 500 gives 310 CTAs or 248, three or two on an SM.
+  // The busiest SM's share: its CTAs times the work of a stage (the tile's columns plus A's 128
+  // rows, which every column tile converts again) times their stages. The last chunk of the samples
+  // is the shorter one and its CTAs are launched last: where only they are left over for one more
+  // round, that round is as short. 800 sizes (L = 9 to 256, I = 3 to 4000, J = 300 to 40000): on average
+  // 0.3 % slower than the fastest tile of each, 7 % without the 128-column tile (whose CTA, alone on
+  // its SM, counts 250). J = 4000, L = 100, I = 500: 125 CTAs of 128 columns, 250 of 64: 19 us and 20.6; J = 250,000:
+  // 310 CTAs of 64 or 248 of 80, three or two on an SM; J = 4000, L = 121, I = 300: 22.4 us with 128 columns,
+  // 31.2 with 64.
   const int64_t mt = (L + TM - 1) / TM, sms = sm_count();
+  const int64_t last = J - (splits - 1) * chunk;
   auto share = [&](int tn) {
-    const int64_t ctas = mt * ((L + I + tn - 1) / tn) * splits;
-    return ((ctas + sms - 1) / sms) * (tn + TM);
+    const int64_t of_chunk = mt * ((L + I + tn - 1) / tn), ctas = of_chunk * splits;
+    const int64_t rounds = (ctas + sms - 1) / sms, over = ctas - (rounds - 1) * sms;
+    const int64_t rows = rounds > 1 && over <= of_chunk ? (rounds - 1) * chunk + last : rounds * chunk;
+    return rows * (tn < 128 ? tn + TM : 250);
   };
-  const bool wide = share(80) < share(64);
-  if (post > 1)
-    return wide ? launch_tn<80, true>(A, Y, J, L, I, post, chunk, splits, partial, err, st,
-                                      wait_limit, jdev)
-                : launch_tn<64, true>(A, Y, J, L, I, post, chunk, splits, partial, err, st,
-                                      wait_limit, jdev);
-  return wide ? launch_tn<80, false>(A, Y, J, L, I, 1, chunk, splits, partial, err, st, wait_limit,
-                                     jdev)
-              : launch_tn<64, false>(A, Y, J, L, I, 1, chunk, splits, partial, err, st, wait_limit,
-                                     jdev);
+  auto go = [&](auto tn) {
+    constexpr int N = decltype(tn)::value;
+    return post > 1 ? launch_tn<N, true>(A, Y, J, L, I, post, chunk, splits, partial, err, st,
+                                         wait_limit, jdev)
+                    : launch_tn<N, false>(A, Y, J, L, I, 1, chunk, splits, partial, err, st,
+                                          wait_limit, jdev);
+  };
+  const int64_t s64 = share(64), s80 = share(80), s128 = share(128);
+  if (s128 < s64 && s128 < s80) return go(std::integral_constant<int, 128>{});
+  if (s80 < s64) return go(std::integral_constant<int, 80>{});
+  return go(std::integral_constant<int, 64>{});
 }
 
 cudaError_t normal_eq_tc_attributes() {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_normal_eq_tc<64, false>, attr, STAGES * stage_bytes<64>() + 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_normal_eq_tc<80, false>, attr, STAGES * stage_bytes<80>() + 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_normal_eq_tc<64, true>, attr, STAGES * stage_bytes<64>() + 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_normal_eq_tc<80, true>, attr, STAGES * stage_bytes<80>() + 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_normal_eq_tc<64, false>, attr, smem_bytes<64>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_normal_eq_tc<80, false>, attr, smem_bytes<80>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_normal_eq_tc<128, false>, attr, smem_bytes<128>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_normal_eq_tc<64, true>, attr, smem_bytes<64>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_normal_eq_tc<80, true>, attr, smem_bytes<80>());
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_normal_eq_tc<128, true>, attr, smem_bytes<128>());
   return e;
 }
 

@@ -73,6 +73,14 @@ FitSplit split_of(const FitArgs& a) { return fit_split(a.N, a.dims, a.ranks); }
 
 size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
+// CTAs of k_fit<double> per SM (at most 3) by their shared memory: of 228 KB, 1 KB of each CTA's is
+// the system's.
+int fit_resident(int K) {
+  const size_t cta = fit_smem_bytes(K) + (2 * 8 * kMaxL + 2 * (FNT / 32)) * sizeof(double) + 1024;
+  const int n = static_cast<int>(228 * 1024 / cta);
+  return n < 1 ? 1 : (n > 3 ? 3 : n);
+}
+
 template <typename T>
 void fit_f64(const FitArgs& a, const FitSplit& f, const void* X, char* wt, double* partial,
              int blocks, cudaStream_t st) {
@@ -104,18 +112,21 @@ size_t fit_workspace(const FitArgs& a, bool x_f64, FitRoom room, int* blocks, si
                            : fit_tc_right_bytes(f));
   }
   int64_t b = x_f64 ? fit_units(f) : fit_tc_plan(a, f).units;
-  // the tensor-core form: one CTA per SM. FP64: as many as are resident (three per SM up to
-  // K = 80; a fourth is a round of its own: 100000 x 3 x 3, rank 3: 148 us a call), but with a chain of three or more
+  // the tensor-core form: one CTA per SM. FP64: as many as are resident, three per SM at most (one
+  // more is a round of its own: 100000 x 3 x 3, rank 3, with four: 148 us a call, now 132; 7 x 9000 x 11,
+  // rank 11, two resident, with three: 940 us a call, now 742), but with a chain of three or more
   // modes a CTA's own V costs more than a tile of products, so the CTAs are then whole row
   // blocks, or equal parts of them while SMs are left over (4^10, rank 10: 279 us with 128 row
   // blocks on as many CTAs, 352 us with 304 CTAs that form V twice each)
-  int64_t cap = x_f64 ? 3 * sm_count() : sm_count();
+  int64_t cap = x_f64 ? fit_resident(f.K) * sm_count() : sm_count();
   if (x_f64 && f.s > 2) {
     const int64_t rb = (f.rows + FL - 1) / FL;
     const int64_t whole = rb * (sm_count() / rb > 1 ? sm_count() / rb : 1);
     cap = whole < cap ? whole : cap;
   }
-  if (b > cap) b = cap;
+  // (a few units more than resident CTAs: one each, the last ones run alone on their SMs; 7 x 900 x 11,
+  // rank 11: 310 units, 304 resident: 183 us a call, 210 with 304 CTAs)
+  if (b > cap && !(x_f64 && f.s <= 2 && b <= cap + cap / 4)) b = cap;
   *blocks = static_cast<int>(b);
   const size_t right = x_f64 ? static_cast<size_t>(f.cols) * f.K * 8 : fit_tc_right_bytes(f);
   *table_bytes = x_f64 || !fit_tc_tables_fit(a, f)

@@ -1472,7 +1472,7 @@ tr_status tr_als(tr_ctx* ctx, const void* X, tr_dtype X_dtype, int N, const int6
       // (sums over a sweep: 64 x 8192 x 2, rank 8: 315 -> 144 us; 64 x 256 x 64: 56 -> 43).
       // FP64 rows are bound by the FP64 pipe and were slower by runs (40 x 30 x 20 x 12: 27 us a
       // mode row by row, 47 by runs).
-      if (!f64 && core_floats <= head) {
+      if (!f64 && core_floats <= head && dense_by_runs(N, n, ca)) {
         TR_LAUNCH("dense_rows", launch_dense_rows(N, n, ca, reinterpret_cast<float*>(idx),
                                                   static_cast<float*>(A), st));
       } else {

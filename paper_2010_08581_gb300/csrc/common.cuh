@@ -109,6 +109,7 @@ struct DenseDims {
 cudaError_t launch_enumerate(int N, int n, const DenseDims& d, int32_t* idx, cudaStream_t st);
 cudaError_t launch_dense_rows(int N, int n, const ChainArgs& ca, float* f32_cores, float* A,
                               cudaStream_t st);
+bool dense_by_runs(int N, int n, const ChainArgs& ca);   // whether the latter is the faster one
 cudaError_t launch_unfold(const void* X, bool x_f64, int N, int n, const DenseDims& d, void* Y,
                           bool y_f64, cudaStream_t st);
 

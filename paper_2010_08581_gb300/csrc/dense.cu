@@ -225,6 +225,21 @@ cudaError_t launch_enumerate(int N, int n, const DenseDims& d, int32_t* idx, cud
   return cudaGetLastError();
 }
 
+// A run costs a chain of barriers whatever its length, and a CTA: short ones are only worth it while
+// they are few or their products large (the kernel that takes row by row reads longer chains from
+// global memory from 100 columns on). All updates of 400 x 400 x f x f, by runs and row by row: f = 3,
+// rank 8: 1887 and 818 us; f = 5, rank 10: 2188 and 2318; f = 6, rank 8: 1985 and 1596, rank 9: 2116 and 2067, of
+// 50 x 50 x 40 x f x f: f = 7, rank 8: 2016 and 1915; 30 x 30 x 3 x 3, rank 8: 59 and 66; 8^6, rank 8: 54 and
+// 58 an update; 2^16, rank 2: 349 and 120.
+bool dense_by_runs(int N, int n, const ChainArgs& ca) {
+  const int f = ((n == N - 1 ? N - 2 : N - 1) - n - 1 + N) % N;     // ring position of the runs' mode
+  const int L = ca.rl[0] * ca.rr[ca.npos - 1];
+  int64_t runs = 1;
+  for (int m = 0; m < ca.npos; ++m)
+    if (m != f) runs *= ca.I[m];
+  return ca.I[f] >= (L >= 100 ? 5 : (L > 64 ? 6 : 8)) || runs <= 2 * sm_count();
+}
+
 cudaError_t launch_dense_rows(int N, int n, const ChainArgs& ca, float* f32_cores, float* A,
                               cudaStream_t st) {
   k_cores_f32<<<2 * static_cast<unsigned>(sm_count()), 256, 0, st>>>(ca, f32_cores);

@@ -226,6 +226,8 @@ cudaError_t batched_fit_attributes() {
   cudaError_t e = cudaFuncSetAttribute(kb_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(fit_smem_bytes(kMaxL)));
   if (e != cudaSuccess) return e;
+  e = fit_tc_registers(reinterpret_cast<const void*>(kb_fit_tc));
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(kb_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kFitTcSmem));
 }

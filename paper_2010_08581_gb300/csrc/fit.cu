@@ -169,6 +169,8 @@ cudaError_t fit_attributes() {
   e = cudaFuncSetAttribute(k_fit<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(fit_smem_bytes(kMaxL)));
   if (e != cudaSuccess) return e;
+  e = fit_tc_registers(reinterpret_cast<const void*>(k_fit_tc));
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_fit_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kFitTcSmem));
 }

@@ -52,6 +52,15 @@ constexpr int FT_NT = 32 * (FT_EW + FT_BW + 4);
 // and one of 128 threads, (2 * 128 + 2 * 88 + 40) * 128 <= 640 * 96
 constexpr int FT_REGS = 96, FT_REGS_E = 128, FT_REGS_B = 88, FT_REGS_C = 40;
 static_assert(2 * FT_REGS_E + 2 * FT_REGS_B + FT_REGS_C <= 5 * FT_REGS, "register shares");
+// setmaxnreg.inc draws on what the CTA was launched with and waits for it without limit, so a kernel
+// that the compiler gave fewer registers than the shares add up to must never be launched: checked
+// when a context or a server is created.
+inline cudaError_t fit_tc_registers(const void* kernel) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess) return e;
+  return at.numRegs < FT_REGS ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
 constexpr size_t kFitTcSmem = 220 * 1024;      // dynamic shared memory of a CTA
 
 // Bytes of the right factors of a split (whole chunks of 32 terms).

@@ -124,9 +124,10 @@ size_t fit_workspace(const FitArgs& a, bool x_f64, FitRoom room, int* blocks, si
     const int64_t whole = rb * (sm_count() / rb > 1 ? sm_count() / rb : 1);
     cap = whole < cap ? whole : cap;
   }
-  // (a few units more than resident CTAs: one each, the last ones run alone on their SMs; 7 x 900 x 11,
-  // rank 11: 310 units, 304 resident: 183 us a call, 210 with 304 CTAs)
-  if (b > cap && !(x_f64 && f.s <= 2 && b <= cap + cap / 4)) b = cap;
+  // (up to four units per SM one each: the ones beyond the resident CTAs run as others leave; 7 x 900 x 11,
+  // rank 11: 310 units, 304 resident: 183 us a call, 210 with 304 CTAs; 40 x 40 x 380, rank 5: 600 units,
+  // 456 resident: 110 and 123)
+  if (b > cap && !(x_f64 && f.s <= 2 && b <= 4 * sm_count())) b = cap;
   *blocks = static_cast<int>(b);
   const size_t right = x_f64 ? static_cast<size_t>(f.cols) * f.K * 8 : fit_tc_right_bytes(f);
   *table_bytes = x_f64 || !fit_tc_tables_fit(a, f)

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(FNT) k_fit(FitArgs a, FitSplit f, const T* __r
 // FP32 slice tables (fit_tc.cuh), one warp per slice.
 __global__ void __launch_bounds__(256) k_fit_tables(FitArgs a, FitSplit f,
                                                     float* __restrict__ out) {
+  grid_wait();
   fit_tables_warps(a, f, out, (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5,
                    static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5));
 }
@@ -45,6 +46,7 @@ __global__ void __launch_bounds__(256) k_fit_tables(FitArgs a, FitSplit f,
 template <int kWarps>
 __global__ void __launch_bounds__(32 * kWarps) k_fit_right_tc(FitArgs a, FitSplit f, const float* tables,
                                                               unsigned char* __restrict__ WS) {
+  grid_wait();
   __shared__ __align__(16) float P[32 * 256];
   __shared__ float G[kWarps * kMaxL];
   fit_right_tc_job<kWarps, 1>(a, f, blockIdx.x, fit_tc_right(a, f, tables), WS, P, G);
@@ -56,6 +58,7 @@ __global__ void __launch_bounds__(FT_NT, 1) k_fit_tc(FitArgs a, FitSplit f, FitT
                                                      const float* tables,
                                                      double* __restrict__ partial, int blocks,
                                                      unsigned* err) {
+  grid_wait();
   extern __shared__ __align__(128) unsigned char fit_tc_raw[];
   __shared__ double red[2 * FT_EW];
   __shared__ FitTcShared sh;
@@ -86,6 +89,8 @@ void fit_f64(const FitArgs& a, const FitSplit& f, const void* X, char* wt, doubl
              int blocks, cudaStream_t st) {
   const unsigned rb = static_cast<unsigned>((f.cols + FNT / 32 - 1) / (FNT / 32));
   T* WT = reinterpret_cast<T*>(wt);
+  // (not as a chain: CTAs placed while the right factors' are still there are spread unevenly, 33 x 37 x
+  // 41, rank 9: 87 us a call, 129 so)
   k_fit_right<T><<<rb, FNT, 0, st>>>(a, f, WT);
   k_fit<T><<<blocks, FNT, fit_smem_bytes(f.K), st>>>(a, f, static_cast<const T*>(X), WT, partial,
                                                      blocks);
@@ -150,15 +155,16 @@ cudaError_t launch_fit(const FitArgs& a, const void* X, bool x_f64, FitRoom room
     if (tables) {
       const int64_t n = ((f.s > 1 ? a.dims[f.s - 1] : 0) + (f.s < a.N - 1 ? a.dims[a.N - 1] : 0) + 7) / 8;
       const int64_t tb = n < 8 * sm_count() ? n : 8 * sm_count();
-      k_fit_tables<<<static_cast<unsigned>(tb), 256, 0, st>>>(a, f, tables);
+      launch_pdl(k_fit_tables, static_cast<unsigned>(tb), 256, 0, st, a, f, tables);
     }
     const int jobs = fit_right_jobs(pl.tiles, pl.ks, FT_RW);
     if (f.s < a.N - 1 && a.dims[a.N - 1] < 8 && jobs <= 2 * sm_count())
-      k_fit_right_tc<FT_RW><<<jobs, 32 * FT_RW, 0, st>>>(a, f, tables, WS);
+      launch_pdl(k_fit_right_tc<FT_RW>, jobs, 32 * FT_RW, 0, st, a, f, tables, WS);
     else
-      k_fit_right_tc<FT_RWS><<<fit_right_jobs(pl.tiles, pl.ks, FT_RWS), 32 * FT_RWS, 0, st>>>(a, f, tables, WS);
-    k_fit_tc<<<blocks, FT_NT, kFitTcSmem, st>>>(a, f, pl, static_cast<const float*>(X), WS, tables,
-                                                partial, blocks, err);
+      launch_pdl(k_fit_right_tc<FT_RWS>, fit_right_jobs(pl.tiles, pl.ks, FT_RWS), 32 * FT_RWS, 0, st, a, f, tables,
+                 WS);
+    launch_pdl(k_fit_tc, blocks, FT_NT, kFitTcSmem, st, a, f, pl, static_cast<const float*>(X), WS, tables,
+               partial, blocks, err);
   }
   return cudaGetLastError();
 }

@@ -212,11 +212,10 @@ __device__ __forceinline__ void tile8(Panels& sm, int i0, int j0, int kb, int ke
   __syncthreads();
   const int warp = t >> 5, lane = t & 31, r = lane >> 2, c = 2 * (lane & 3);
   double x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
-  const int k1 = (warp + 1) * (kp / 2);
-  for (int kr = warp * (kp / 2); kr < k1; kr += kRun) {
-    double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+  const int k0 = warp * (kp / 2), k1 = (warp + 1) * (kp / 2);
+  auto terms = [&](int ka, int ke2, double& p0, double& p1, double& q0, double& q1) {
 #pragma unroll 4
-    for (int k = kr; k < min(kr + kRun, k1); k += 2) {
+    for (int k = ka; k < ke2; k += 2) {
       const double2 u = *reinterpret_cast<const double2*>(&sm.a[r][k]);
       const double2 v = *reinterpret_cast<const double2*>(&sm.b[c][k]);
       const double2 w = *reinterpret_cast<const double2*>(&sm.b[c + 1][k]);
@@ -225,10 +224,18 @@ __device__ __forceinline__ void tile8(Panels& sm, int i0, int j0, int kb, int ke
       p1 += u.y * v.y;
       q1 += u.y * w.y;
     }
-    x0 += p0;
-    y0 += q0;
-    x1 += p1;
-    y1 += q1;
+  };
+  if constexpr (kRun >= DLD) {
+    terms(k0, k1, x0, x1, y0, y1);
+  } else {
+    for (int kr = k0; kr < k1; kr += kRun) {
+      double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+      terms(kr, min(kr + kRun, k1), p0, p1, q0, q1);
+      x0 += p0;
+      y0 += q0;
+      x1 += p1;
+      y1 += q1;
+    }
   }
   x0 += x1;
   y0 += y1;

@@ -119,8 +119,7 @@ cudaError_t launch_ff_image(const double* Lrow, const double* Lcol, int n, const
   const int64_t count = static_cast<int64_t>(n) * (n + 1);
   const unsigned blocks = static_cast<unsigned>((count + 255) / 256 < sm_count() ? (count + 255) / 256 : sm_count());
   launch_pdl(k_ff_image, blocks, 256, 0, st, reinterpret_cast<const float*>(Lrow),
-                                     reinterpret_cast<const float*>(Lcol), count, info, img64,
-                                     run_if);
+             reinterpret_cast<const float*>(Lcol), count, info, img64, run_if);
   return cudaGetLastError();
 }
 
@@ -133,9 +132,8 @@ cudaError_t launch_cholesky_lev_mixed(const double* G, int n, double tol64, doub
   const size_t ff = static_cast<size_t>(panel_floats<FFOps>(n)) * 4;
   const size_t want = nn * 8 > ff ? nn * 8 : ff;
   const size_t dyn = want <= kCholDyn ? want : (nn * 8 <= kCholDyn ? nn * 8 : 0);
-  launch_pdl(k_cholesky_lev_mixed, 1, CNT, dyn, st, G, n, tol64, tolff, Lrow, Lcol, invdiag, keep, info,
-                                            err, static_cast<int>(dyn), img64, pre_hi, pre_lo,
-                                            run_if);
+  launch_pdl(k_cholesky_lev_mixed, 1, CNT, dyn, st, G, n, tol64, tolff, Lrow, Lcol, invdiag, keep,
+             info, err, static_cast<int>(dyn), img64, pre_hi, pre_lo, run_if);
   return cudaGetLastError();
 }
 
@@ -148,7 +146,7 @@ cudaError_t launch_cholesky_mixed(const double* G, int n, int mode, double tol64
   const bool tiles = wimg && fast && pre && n >= 4 && n <= kCiMaxN;
   if (tiles) {
     launch_pdl(k_chol_inv_solve, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(tol32), pre,
-                                                        (n + 3) & ~3, wimg, keep, info, err, fast);
+               (n + 3) & ~3, wimg, keep, info, err, fast);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -161,10 +159,9 @@ cudaError_t launch_cholesky_mixed(const double* G, int n, int mode, double tol64
     if (e != cudaSuccess) return e;
   }
   // (beyond kPanelCholMax the one-CTA factorisation reads G, and its work arrays may be pre's)
-  launch_pdl(k_cholesky_mixed<float>, 1, CNT, dyn, st, G, n, mode, tol64, tol32, Lrow, Lcol, invdiag, keep,
-                                               info, err, static_cast<int>(dyn), img32, gimg32,
-                                               n <= kPanelCholMax ? pre : nullptr,
-                                               tiles ? fast : nullptr, big ? fast + 1 : nullptr);
+  launch_pdl(k_cholesky_mixed<float>, 1, CNT, dyn, st, G, n, mode, tol64, tol32, Lrow, Lcol,
+             invdiag, keep, info, err, static_cast<int>(dyn), img32, gimg32,
+             n <= kPanelCholMax ? pre : nullptr, tiles ? fast : nullptr, big ? fast + 1 : nullptr);
   return cudaGetLastError();
 }
 
@@ -175,8 +172,8 @@ cudaError_t launch_cholesky(const double* G, int n, int mode, double tol_scale, 
   const size_t bytes = static_cast<size_t>(n) * n * sizeof(double);
   const int use_smem = bytes <= kCholDyn ? 1 : 0;
   const size_t dyn = use_smem ? bytes : 0;
-  launch_pdl(k_cholesky, 1, CNT, dyn, st, G, n, mode, tol_scale, Lrow, Lcol, invdiag, keep, info, err,
-                                  use_smem, img64, img32, gimg32, run_if);
+  launch_pdl(k_cholesky, 1, CNT, dyn, st, G, n, mode, tol_scale, Lrow, Lcol, invdiag, keep, info,
+             err, use_smem, img64, img32, gimg32, run_if);
   return cudaGetLastError();
 }
 

@@ -335,6 +335,7 @@ struct Lev64 {
 bool solve_f64_fits(int64_t I, int n, int splits);
 cudaError_t launch_solve_f64(const Lev64& w, int n, const double* rhs, int64_t ld, int64_t I, int Rl,
                              int Rr, double* core_out, cudaStream_t st);
+bool leverage_f64_fits(int64_t I, int n, int splits);
 cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,
                                 int64_t lda, double* ell, const CdfEpilogue& ep, cudaStream_t st);
 // The FP64 LS step through an FP32 inverse (lev64.cu) on a solve's workspace; the flags are in
@@ -355,10 +356,6 @@ Lev64 solve_f64_plan(const Plan& s, int L) {
   w.info = s.info;
   return w;
 }
-
-bool leverage_f64_fits(int64_t I, int n, int splits);
-cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64_t I, int n,
-                                int64_t lda, double* ell, const CdfEpilogue& ep, cudaStream_t st);
 
 // dst[e] = hi[e] + lo[e] in FP64 (lev_precond.cu).
 cudaError_t launch_planes_sum(const float* hi, const float* lo, int64_t count, double* dst,

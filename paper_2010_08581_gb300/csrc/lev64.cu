@@ -12,8 +12,9 @@
 // Why: one SM multiplies two FP64 pairs per clock, so the one-CTA FP64 factorisation of a 256 x
 // 256 matrix is 0.7 ms of arithmetic (1.85 ms measured), and one chain of 256 columns per
 // substitution follows. Here the only serial chains are the FP32 one-CTA passes of chol_inv.cuh;
-// the rest are matrix products in small tiles over all SMs, eight short launches bound by one
-// tile's FP64 arithmetic and a trip to L2 each (n = 256: 271 us, then 81 for 300 rows).
+// the rest are matrix products in small tiles over all SMs: with the factor's, eight short launches
+// up to 128 columns and 13 beyond, bound by one tile's FP64 arithmetic and a trip to L2 each, then
+// two for the rows (n = 256: 271 us, then 81 for 300 rows).
 //
 // Every kernel does nothing when the flag in its arguments says that the FP32 factorisation
 // failed (a pivot <= n * eps32 * max diag) or that ||E||_F is too large for the series; the
@@ -547,9 +548,10 @@ __global__ void __launch_bounds__(kCiMaxThreads) k_small_factor(int n, float tol
   if (threadIdx.x == 0) { bad[0] = ok ? 0 : 1; bad[1] = ok ? 0 : 1; }
 }
 
-// From about here on the products beat the one-CTA FP64 factorisation and the FP64 substitutions
-// (I = 300, with the gated launches: n = 64: 108 -> 122 us, n = 100: 193 -> 163, n = 128: 287 -> 180,
-// n = 256: 2205 -> 363).
+// From about here on the products beat the one-CTA FP64 factorisation and the FP64 substitutions. Whole
+// calls, 300 rows: n = 88: 191 -> 151 us, 100: 224 -> 160, 144: 402 -> 230, 256: 2285 -> 402. Where the
+// products are refused the call pays for both forms: a few us when a pivot is too small, the
+// FP32 inverse, U and E when ||E|| is too large (cond(K) of 1e5 and more): 240, 277, 507 and 1995 us.
 constexpr int kLev64MinN = 88;
 
 constexpr int64_t kMaxRows = 1 << 18;      // rows per launch: tiles in a grid's second dimension
@@ -680,8 +682,8 @@ cudaError_t launch_leverage_f64(int part, const Lev64& w, const double* A, int64
                                         w.bad, nullptr, nullptr, nullptr, st);
     if (e != cudaSuccess) return e;
   } else {
-    launch_pdl(k_small_factor, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(tol), w.K32, w.ldk,
-                                                      w.Ximg, w.bad);
+    launch_pdl(k_small_factor, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(tol), w.K32,
+               w.ldk, w.Ximg, w.bad);
   }
   launch_pdl(k_l64_u, dim3(nt, nt), DNT, 0, st, g);
   launch_pdl(k_l64_e, up, DNT, 0, st, g);

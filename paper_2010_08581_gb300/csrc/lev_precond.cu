@@ -550,8 +550,8 @@ cudaError_t launch_gram_dd(const float* Ah, const float* Al, int64_t I, int n, i
   int64_t chunk;
   const int splits = gram_dd_splits(I, &chunk);
   const int nt = (n + GD - 1) / GD;
-  launch_pdl(k_gram_dd, dim3(nt * (nt + 1) / 2, splits), GDNT, 0, st, Ah, Al, I, n, lda_a, chunk, splits,
-                                                              ph, pl, cnt, kh, kl, lda, k64);
+  launch_pdl(k_gram_dd, dim3(nt * (nt + 1) / 2, splits), GDNT, 0, st, Ah, Al, I, n, lda_a, chunk,
+             splits, ph, pl, cnt, kh, kl, lda, k64);
   return cudaGetLastError();
 }
 
@@ -571,23 +571,22 @@ cudaError_t launch_lev_precond(int stage, const LevPrecond& lp, int n, int64_t I
   switch (stage) {
     case 0: {
       const double eps32 = 1.1920928955078125e-07;
-      launch_pdl(k_chol_inv, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(n * eps32), lp.K_hi,
-                                                    lp.lda_k, lp.Ximg, lp.state);
+      launch_pdl(k_chol_inv, 1, chol_inv_threads(n), 0, st, n, static_cast<float>(n * eps32),
+                 lp.K_hi, lp.lda_k, lp.Ximg, lp.state);
       return cudaGetLastError();
     }
     case 1:
       launch_pdl(k_lev_u, dim3(nt, nt), dim3(LT, LT), 0, st, n, lp.K_hi, lp.K_lo, lp.lda_k, lp.Ximg,
-                                                     lp.state, lp.Uh, lp.Ul, ld);
+                 lp.state, lp.Uh, lp.Ul, ld);
       return cudaGetLastError();
     case 2:
       launch_pdl(k_lev_e, lev_precond_ctas(n), dim3(LT, LT), 0, st, n, lp.Uh, lp.Ul, ld, lp.Ximg,
-                                                           lp.state, lp.E, ld, lp.esq);
+                 lp.state, lp.E, ld, lp.esq);
       return cudaGetLastError();
     case 3: {
       const unsigned rb = static_cast<unsigned>((I + LR_ROWS - 1) / LR_ROWS);
       launch_pdl(k_lev_rows, rb, LR_NT, lev_rows_smem(n), st, n, I, Ah, Al, lda, lp.Ximg, lp.E, ld,
-                                                        lp.esq, lev_precond_ctas(n), lp.state,
-                                                        ell, ep, lp.tau);
+                 lp.esq, lev_precond_ctas(n), lp.state, ell, ep, lp.tau);
       return cudaGetLastError();
     }
     default:

@@ -186,9 +186,7 @@ void run_sample_chain(unsigned blocks, size_t dyn, cudaStream_t st, const Sample
                       uint32_t u1, int32_t* idx, double* w, void* A, int staged,
                       const GatherArgs& ga, const void* X, void* Y) {
   launch_pdl((k_sample_chain<T, TX>), blocks, FW * 32, dyn, st, sa, ca, J, k0, k1, u0, u1, idx, w,
-                                                      static_cast<T*>(A), staged, ga,
-                                                      static_cast<const TX*>(X),
-                                                      static_cast<T*>(Y));
+             static_cast<T*>(A), staged, ga, static_cast<const TX*>(X), static_cast<T*>(Y));
 }
 
 }  // namespace

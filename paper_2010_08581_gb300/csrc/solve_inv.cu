@@ -203,8 +203,8 @@ cudaError_t launch_solve_inv(int n, const float* Limg, const float* Mimg,
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned sb = static_cast<unsigned>((nvec + SNR - 1) / SNR);
-  launch_pdl(k_solve_inv, sb, SNT, solve_smem_bytes(n), st, n, Wimg, Mimg, info, nvec, rhs, ld, Rl, Rr,
-                                                     core_out);
+  launch_pdl(k_solve_inv, sb, SNT, solve_smem_bytes(n), st, n, Wimg, Mimg, info, nvec, rhs, ld, Rl,
+             Rr, core_out);
   return cudaGetLastError();
 }
 

@@ -336,7 +336,7 @@ cudaError_t launch_normal_eq_tc(const float* A, const float* Y, int64_t J, int L
   // is the shorter one and its CTAs are launched last: where only they are left over for one more
   // round, that round is as short. 800 sizes (L = 9 to 256, I = 3 to 4000, J = 300 to 40000): on average
   // 0.3 % slower than the fastest tile of each, 7 % without the 128-column tile (whose CTA, alone on
-  // its SM, counts 250). J = 4000, L = 100, I = 500: 125 CTAs of 128 columns, 250 of 64: 19 us and 20.6; J = 250,000:
+  // its SM, counts 250). J = 4000, L = 100, I = 500: 125 CTAs of 128 columns, 250 of 64: 15.6 us and 20.6; J = 250,000:
   // 310 CTAs of 64 or 248 of 80, three or two on an SM; J = 4000, L = 121, I = 300: 22.4 us with 128 columns,
   // 31.2 with 64.
   const int64_t mt = (L + TM - 1) / TM, sms = sm_count();

@@ -56,7 +56,8 @@ typedef enum tr_dtype { TR_F32 = 0, TR_F64 = 1 } tr_dtype;
  *                Cholesky factor, and one step of refinement, every product in FP64: z = V b,
  *                z += V (b - M z), whose residual is no larger than that of a factorisation
  *                (||b - M z|| <= 1.5 * 2^-53 ||M|| ||z|| in the tests); the FP64 factorisation
- *                when X is too poor for it.
+ *                when X is too poor for it or the right-hand sides are many (I > 6 L, 12 L beyond
+ *                L = 160).
  * TR_PREC_MIXED: design rows and fibres in FP32, contractions with FP32 accumulation.
  *                The normal matrix is factored in FP32 when every pivot exceeds
  *                L*eps32*max diag, else in FP64 (same singular rule as TR_PREC_FP64);
@@ -69,7 +70,9 @@ typedef enum tr_dtype { TR_F32 = 0, TR_F64 = 1 } tr_dtype;
  *                Gram and a double-float series, or, when that preconditioner is poor, the
  *                Gram factored in double-float (pairs of FP32, about 46 significant bits)
  *                when every pivot exceeds max(I,L)*2^-40*max diag, else in FP64 with column
- *                dropping. All other leverage arithmetic, and tr_leverage, is FP64.
+ *                dropping; the Gram's factor alone for the initial distributions, those of
+ *                TR_LS_RANK_DROP and 128 < L <= 160. All other leverage arithmetic, and
+ *                tr_leverage, is FP64.
  *                The drivers (both precisions) read the fibres of a strided mode from a
  *                copy of X with that mode last, made at the start of each call, when the
  *                scattered reads would move more bytes than the copy and memory allows;
@@ -115,8 +118,9 @@ tr_status tr_status_sync(tr_ctx* ctx, tr_stream stream);
  * above max(I,L)*eps*sigma_max (the rule of a singular value decomposition); otherwise from
  * a Cholesky-based thin QR of G_(2) (or of G_(2)^T when I < L), with dependent columns
  * dropped at pivot <= max(I,L)*eps*max diag, which resolves singular values down to about
- * sqrt(max(I,L)*eps)*sigma_max (I >= L >= 88 with every FP32 pivot above L*eps32*max diag: by FP64
- * products with X' of TR_PREC_FP64 above, which resolves as much). The drivers form every distribution the same way.
+ * sqrt(max(I,L)*eps)*sigma_max (L >= 88, L <= I <= 32 L, or 64 L beyond L = 160, with every FP32
+ * pivot above L*eps32*max diag: by FP64 products with X' of TR_PREC_FP64 above, which resolves as
+ * much). The FP64 drivers form every distribution the same way, the mixed ones as TR_PREC_MIXED says.
  * A zero core records TR_ERR_SINGULAR and yields the uniform distribution. */
 tr_status tr_leverage(tr_ctx* ctx, const double* core, int64_t I, int Rl, int Rr,
                       double* p, double* cdf, tr_stream stream);
